@@ -37,8 +37,9 @@
  *   HQ_NO_GRAPH=1  hq_sweep_step issues its launches instead of replaying a CUDA graph
  *   HQ_NO_FORK=1   hq_sweep_step keeps the witness sums and beam deposits on the grid's
  *                  stream instead of beside the final pass on a second stream
- *   HQ_SEPARATE_SRC=1  FP32: the psi/Ez/Bz and B_perp sources are formed by kernels of
- *                  their own ahead of each solve instead of in the solve's first phase
+ *   HQ_SEPARATE_SRC=1  the psi/Ez/Bz and B_perp sources are formed by kernels of their own
+ *                  ahead of each solve instead of in the solve's first phase or pass (FP64:
+ *                  and the B_perp mixing in one of its own behind it)
  *   HQ_NO_F4CACHE=1  FP32: every predictor-corrector trial pass and the final pass gather all
  *                  six fields (by default the first trial pass of a slice keeps ExmBy, EypBx,
  *                  Ez, Bz per particle and the later passes of the slice gather Bx, By alone;

@@ -49,7 +49,6 @@ cudaError_t dalloc(P** p, size_t bytes) {
 }
 
 int64_t round_up(int64_t v, int64_t m) { return (v + m - 1) / m * m; }
-bool is_pow2(int n) { return n > 0 && (n & (n - 1)) == 0; }
 
 void adj_free(hq_grid_s* g);
 
@@ -106,10 +105,12 @@ void free_all(hq_grid_s* g) {
 std::vector<double> scale_table(const hq_grid_s* g, int rows, int cols, double shift = 0.0) {
   std::vector<double> t((size_t)rows * cols, 0.0);
   const double pi = M_PI;
+  std::vector<double> sxs(g->nx, 0.0);
+  for (int k = 1; k < g->nx; ++k) sxs[k] = std::sin(pi * k / (2.0 * g->nx));
   for (int l = 1; l < g->ny; ++l) {
     const double sy = std::sin(pi * l / (2.0 * g->ny));
     for (int k = 1; k < g->nx; ++k) {
-      const double sx = std::sin(pi * k / (2.0 * g->nx));
+      const double sx = sxs[k];
       const double lam = -(4.0 / (g->geom.dx * g->geom.dx)) * sx * sx - (4.0 / (g->geom.dy * g->geom.dy)) * sy * sy;
       t[(size_t)l * cols + k] = (4.0 / ((double)g->nx * g->ny)) / (lam - shift);
     }
@@ -264,7 +265,7 @@ struct Prof {
 };
 
 void dst_solve(hq_grid_s* g, int nrhs) {
-  Prof p(g, HQ_K_DST, g->fp64 ? 4 : 1);   // FP64: four FFT passes; FP32: one fused cooperative launch
+  Prof p(g, HQ_K_DST, g->fp64 ? dst_f64_launches(g) : 1);   // FP32: one fused cooperative launch
   if (g->fp64) dst_solve_f64(g, nrhs, g->stream);
   else dst_solve_tc(g, nrhs, g->stream);
 }
@@ -280,6 +281,9 @@ hq_status solve_fields_impl(hq_grid_s* g, int slice) {
   if (fused_src) {
     Prof p(g, HQ_K_DST, 1);
     dst_solve_tc_main(g, cur, s);
+  } else if (g->fp64 && !g->sep_src && dst_f64_fused(g, 3)) {
+    Prof p(g, HQ_K_DST, dst_f64_launches(g));
+    dst_f64_main(g, cur, s);
   } else {
     { Prof p(g, HQ_K_FIELD, 1); launch_src_main<T>(g, cur, s); }
     dst_solve(g, 3);
@@ -297,7 +301,7 @@ hq_status solve_fields_impl(hq_grid_s* g, int slice) {
     { Prof p(g, HQ_K_FIELD, 1); launch_pcg_init<T>(g, slice, cur, chi_cur, prev, chi_prev, s); }
     for (int k = 0; k < npc; ++k) {
       {
-        Prof p(g, HQ_K_DST, g->fp64 ? 4 : 1);
+        Prof p(g, HQ_K_DST, g->fp64 ? dst_f64_launches(g) : 1);
         if (g->fp64) dst_solve_f64(g, 2, s, reinterpret_cast<const double*>(g->scale_h));
         else dst_solve_tc_shifted(g, 2, s);
       }
@@ -318,6 +322,11 @@ hq_status solve_fields_impl(hq_grid_s* g, int slice) {
     if (fused_src) {
       Prof p(g, HQ_K_DST, 1);   // sources, solve and the mixing in one launch
       dst_solve_tc_bmix_src(g, cur, prev, chi_prev, last, s);
+      continue;
+    }
+    if (g->fp64 && !g->sep_src && dst_f64_fused(g, 2)) {
+      Prof p(g, HQ_K_DST, dst_f64_launches(g));   // sources in the first pass, mixing in the last
+      dst_f64_bmix(g, cur, prev, chi_prev, last, s);
       continue;
     }
     { Prof p(g, HQ_K_FIELD, 1); launch_src_bperp<T>(g, cur, prev, chi_prev, last, s); }
@@ -1103,21 +1112,30 @@ hq_status hq_grid_create(const hq_grid_desc* desc, void* cuda_stream, hq_grid_t*
   cudaMemset(g->d_status, 0, sizeof(int));
   cudaMemset(g->d_removed, 0, sizeof(unsigned long long));
 
+  const char* ss = std::getenv("HQ_SEPARATE_SRC");
+  g->sep_src = (ss && ss[0] == '1') ? 1 : 0;
   // DST tables
   if (g->fp64) {
     HQ_ALLOC(g->f64_a, 8 * kMaxRhs * nn);
     HQ_ALLOC(g->f64_b, 8 * kMaxRhs * nn);
     cudaMemset(g->f64_a, 0, 8 * kMaxRhs * nn);
-    std::vector<double> sc = scale_table(g, g->ny, g->nx);
+    // [nx][ny]: the y passes read a row of one kx along ky
+    auto upload_scale = [&](double* d, double shift) {
+      const std::vector<double> sc = scale_table(g, g->ny, g->nx, shift);
+      const double norm = dst_f64_norm(g->nx, g->ny);
+      std::vector<double> tr(nn);
+      for (int y = 0; y < g->ny; ++y)
+        for (int x = 0; x < g->nx; ++x) tr[(size_t)x * g->ny + y] = norm * sc[(size_t)y * g->nx + x];
+      cudaMemcpy(d, tr.data(), 8 * nn, cudaMemcpyHostToDevice);
+    };
     HQ_ALLOC(g->f64_scale, 8 * nn);
-    cudaMemcpy(g->f64_scale, sc.data(), 8 * nn, cudaMemcpyHostToDevice);
+    upload_scale(g->f64_scale, 0.0);
     if (g->explicit_b) {
-      std::vector<double> sh = scale_table(g, g->ny, g->nx, g->xshift);
       HQ_ALLOC(g->scale_h, 8 * nn);
-      cudaMemcpy(g->scale_h, sh.data(), 8 * nn, cudaMemcpyHostToDevice);
+      upload_scale(reinterpret_cast<double*>(g->scale_h), g->xshift);
     }
     auto tables = [&](int n, double** tw, double** sn) -> hq_status {
-      if (is_pow2(n)) {
+      if (dst_f64_twiddles(n)) {
         std::vector<double> t(2 * (size_t)n);
         for (int k = 0; k < n; ++k) {
           t[2 * k] = std::cos(M_PI * k / n);
@@ -1126,9 +1144,7 @@ hq_status hq_grid_create(const hq_grid_desc* desc, void* cuda_stream, hq_grid_t*
         if (dalloc(tw, 8 * t.size()) != cudaSuccess) return HQ_ERR_OOM;
         cudaMemcpy(*tw, t.data(), 8 * t.size(), cudaMemcpyHostToDevice);
       } else {
-        std::vector<double> t((size_t)n * n);
-        for (int j = 0; j < n; ++j)
-          for (int k = 0; k < n; ++k) t[(size_t)j * n + k] = sin_jk(j, k, n);
+        const std::vector<double> t = dst_f64_table(n, sin_jk);
         if (dalloc(sn, 8 * t.size()) != cudaSuccess) return HQ_ERR_OOM;
         cudaMemcpy(*sn, t.data(), 8 * t.size(), cudaMemcpyHostToDevice);
       }
@@ -1148,8 +1164,6 @@ hq_status hq_grid_create(const hq_grid_desc* desc, void* cuda_stream, hq_grid_t*
     g->no_srccache = nsc && nsc[0] == '1';
     const char* nf4 = std::getenv("HQ_NO_F4CACHE");
     g->no_f4 = nf4 && nf4[0] == '1';
-    const char* ss = std::getenv("HQ_SEPARATE_SRC");
-    g->sep_src = (ss && ss[0] == '1') ? 1 : 0;
     const char* fb = std::getenv("HQ_FAULT_BARRIER");
     g->fault_barrier = (fb && fb[0] == '1') ? 1 : 0;
     HQ_ALLOC(g->d_gbar, sizeof(unsigned long long));
@@ -1557,10 +1571,14 @@ hq_status hq_poisson_solve(hq_grid_t g, const void* src, void* dst, int32_t nrhs
   if (!g) return fail(nullptr, HQ_ERR_ARG, "grid is NULL");
   if (!src || !dst || nrhs < 1 || nrhs > kMaxRhs) return fail(g, HQ_ERR_ARG, "src/dst NULL or nrhs not in 1..5");
   cudaStream_t s = g->stream;
+  if (g->fp64) {
+    Prof p(g, HQ_K_DST, dst_f64_launches(g));
+    dst_solve_f64(g, nrhs, s, nullptr, static_cast<const double*>(src), static_cast<double*>(dst));
+    return check_launch(g);
+  }
   {
     Prof p(g, HQ_K_FIELD, 1);
-    if (g->fp64) launch_src_copy<double>(g, src, nrhs, s);
-    else launch_src_copy<float>(g, src, nrhs, s);
+    launch_src_copy<float>(g, src, nrhs, s);
   }
   dst_solve(g, nrhs);
   HQ_CUDA(g, cudaMemcpyAsync(dst, g->solved, (size_t)nrhs * g->nnode * g->tsize, cudaMemcpyDeviceToDevice, s));

@@ -225,7 +225,8 @@ struct hq_grid_s {
                        // (B_perp of slice i-1 is gf[3..4] until then)
   void* solved;        // kMaxRhs x nnode: DST results
 
-  // DST, FP64: [kMaxRhs][nnode] ping-pong buffers, per-mode scale, twiddles, sine tables
+  // DST, FP64: [kMaxRhs][nnode] ping-pong buffers, per-mode scale [nx][ny], twiddles or folded sine
+  // tables by extent (dst_f64_twiddles)
   double *f64_a, *f64_b, *f64_scale, *tw_x, *tw_y, *sin_x, *sin_y;
   // DST, FP32/bf16x3: padded operand buffers and sine matrices
   int nxp, nyp;
@@ -318,8 +319,19 @@ template <typename T> void launch_finish_bperp(const hq_grid_s* g, const void* r
 template <typename T> void launch_store(const hq_grid_s* g, const hq_field_out* out, int64_t slot, const void* dep, const void* chi, cudaStream_t s);
 template <typename T> void launch_zero(void* p, int64_t n, cudaStream_t s);
 // DST backends: transform the nrhs sources prepared by the src kernels into g->solved
-// scale: the spectral factors (null: the Poisson table f64_scale; scale_h: the shifted one)
-void dst_solve_f64(hq_grid_s* g, int nrhs, cudaStream_t s, const double* scale = nullptr);
+// scale: the spectral factors (null: the Poisson table f64_scale; scale_h: the shifted one);
+// src null: the sources in f64_a; dst null: into g->solved
+void dst_solve_f64(hq_grid_s* g, int nrhs, cudaStream_t s, const double* scale = nullptr, const double* src = nullptr,
+                   double* dst = nullptr);
+// FP64 solves with the source assembly (and the B_perp mixing) in their first (last) pass;
+// available for nr right-hand sides when dst_f64_fused(g, nr)
+bool dst_f64_fused(const hq_grid_s* g, int nr);
+void dst_f64_main(hq_grid_s* g, const void* dep, cudaStream_t s);
+void dst_f64_bmix(hq_grid_s* g, const void* cur, void* prev, void* chi_prev, int last, cudaStream_t s);
+std::vector<double> dst_f64_table(int n, double (*sin_jk)(int64_t, int64_t, int));
+bool dst_f64_twiddles(int n);          // rows of n points use the twiddle table (else the sine table)
+double dst_f64_norm(int nx, int ny);   // factor of the FP64 scale table (see k_dst_f64.cu)
+int dst_f64_launches(const hq_grid_s* g);   // kernel launches of one FP64 solve
 void dst_solve_tc(hq_grid_s* g, int nrhs, cudaStream_t s);
 void dst_solve_tc_shifted(hq_grid_s* g, int nrhs, cudaStream_t s);   // (L - c)^{-1}: g->scale_h
 void dst_solve_tc_bmix(hq_grid_s* g, int last, cudaStream_t s);   // B_perp solve + fused mixing (FP32)
