@@ -40,10 +40,10 @@
  *   HQ_SEPARATE_SRC=1  the psi/Ez/Bz and B_perp sources are formed by kernels of their own
  *                  ahead of each solve instead of in the solve's first phase or pass (FP64:
  *                  and the B_perp mixing in one of its own behind it)
- *   HQ_NO_F4CACHE=1  FP32: every predictor-corrector trial pass and the final pass gather all
- *                  six fields (by default the first trial pass of a slice keeps ExmBy, EypBx,
- *                  Ez, Bz per particle and the later passes of the slice gather Bx, By alone;
- *                  the gathered values are bit for bit the same)
+ *   HQ_NO_F4CACHE=1  every predictor-corrector trial pass and the final pass evaluate everything
+ *                  (by default the first trial pass of a slice keeps per particle what does
+ *                  not depend on B_perp, and the later passes of the slice gather Bx, By alone:
+ *                  the same values up to rounding)
  *   HQ_NO_SRCCACHE=1  FP32: every B_perp source phase of the predictor-corrector forms all its
  *                  terms from the records (by default the first iteration of a slice keeps
  *                  the part that does not depend on the trial J_perp, and the others add the

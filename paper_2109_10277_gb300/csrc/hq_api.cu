@@ -54,14 +54,19 @@ void adj_free(hq_grid_s* g);
 
 void free_all(hq_grid_s* g) {
   auto F = [](void* p) { if (p) cudaFree(p); };
+  auto free_tc = [&](auto& t) {
+    F(t.idx); F(t.e); F(t.te); F(t.a); F(t.qt); F(t.f4); F(t.rate); F(t.tg); F(t.tx); F(t.ty); F(t.tpsi);
+  };
   for (hq::Plasma<double>* p : {&g->p64}) {
     F(p->x); F(p->y); F(p->psi); F(p->ux); F(p->uy); F(p->w); F(p->alive); F(p->hist);
+    free_tc(p->tc);
   }
   {
     hq::Plasma<float>& p = g->p32;
     if (!g->fp64) {
       // x, y, psi, alive are shared with p64 storage (freed above); free the typed arrays
-      F(p.ux); F(p.uy); F(p.w); F(p.hist); F(p.cell); F(p.fx); F(p.fy); F(p.opp); F(p.hsum); F(p.f4);
+      F(p.ux); F(p.uy); F(p.w); F(p.hist); F(p.cell); F(p.fx); F(p.fy); F(p.opp); F(p.hsum);
+      free_tc(p.tc);
     }
   }
   if (g->det_arena) {
@@ -317,7 +322,7 @@ hq_status solve_fields_impl(hq_grid_s* g, int slice) {
     tape_b_iterate(g, m);
     g->pc_iter = m;   // the B_perp sources of iteration 0 keep their invariant part for the others
     { Prof p(g, HQ_K_TRIAL, 1); launch_trial_pass<T>(g, slice, m, s); }
-    if (m == 0) g->f4_slice = (g->fp64 || g->no_f4) ? -1 : slice;   // the final pass may reuse it
+    if (m == 0) g->f4_slice = g->no_f4 ? -1 : slice;   // the final pass may reuse it
     if (g->det) launch_fx_decode(g, g->tj, 2 * g->nnode, nullptr, s);
     if (fused_src) {
       Prof p(g, HQ_K_DST, 1);   // sources, solve and the mixing in one launch
@@ -1001,7 +1006,23 @@ hq_status hq_grid_create(const hq_grid_desc* desc, void* cuda_stream, hq_grid_t*
     HQ_ALLOC(g->p32.hist, 4 * np * kRing * 5);
     HQ_ALLOC(g->p32.cell, 4 * np); HQ_ALLOC(g->p32.fx, 4 * np); HQ_ALLOC(g->p32.fy, 4 * np); HQ_ALLOC(g->p32.opp, 4 * np);
     HQ_ALLOC(g->p32.hsum, 4 * np * 5);
-    HQ_ALLOC(g->p32.f4, 16 * np);
+  }
+  const char* nf4 = std::getenv("HQ_NO_F4CACHE");
+  g->no_f4 = nf4 && nf4[0] == '1';
+  if (!g->explicit_b && !g->no_f4 && d.n_pc_iter > 0) {
+    auto alloc_tc = [&](auto& t, size_t z) -> hq_status {
+      HQ_ALLOC(t.idx, 8 * np); HQ_ALLOC(t.e, 2 * z * np); HQ_ALLOC(t.te, 2 * z * np); HQ_ALLOC(t.a, 2 * z * np);
+      HQ_ALLOC(t.qt, z * np);
+      if (z == 4) {
+        HQ_ALLOC(t.f4, 16 * np);
+      } else {
+        HQ_ALLOC(t.rate, 32 * np);
+        HQ_ALLOC(t.tg, z * np); HQ_ALLOC(t.tx, 8 * np); HQ_ALLOC(t.ty, 8 * np); HQ_ALLOC(t.tpsi, 8 * np);
+      }
+      return HQ_OK;
+    };
+    const hq_status st = g->fp64 ? alloc_tc(g->p64.tc, 8) : alloc_tc(g->p32.tc, 4);
+    if (st != HQ_OK) return st;   // (everything is freed)
   }
   if (d.resort_every > 0) {
     HQ_ALLOC(g->porigin, 4 * np);
@@ -1162,8 +1183,6 @@ hq_status hq_grid_create(const hq_grid_desc* desc, void* cuda_stream, hq_grid_t*
     g->fold = (g->nx % 128 == 0 && g->ny % 128 == 0 && !(nf && nf[0] == '1')) ? 1 : 0;
     const char* nsc = std::getenv("HQ_NO_SRCCACHE");
     g->no_srccache = nsc && nsc[0] == '1';
-    const char* nf4 = std::getenv("HQ_NO_F4CACHE");
-    g->no_f4 = nf4 && nf4[0] == '1';
     const char* fb = std::getenv("HQ_FAULT_BARRIER");
     g->fault_barrier = (fb && fb[0] == '1') ? 1 : 0;
     HQ_ALLOC(g->d_gbar, sizeof(unsigned long long));

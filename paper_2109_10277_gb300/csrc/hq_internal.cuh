@@ -62,6 +62,28 @@ template <typename T> struct V2 { T a, b; };          // packed jx, jy or bx, by
 // (V2 per node, hq_grid_s::bm), which the mixing updates in place.
 constexpr int kGF = 4;
 
+// What the predictor-corrector's iterations of one slice share, per particle.  Of a trial step
+// only u_perp depends on B_perp, linearly: f_ux = A + m By, f_uy = C - m Bx (m = -q/M), so the
+// trial position, its deposit stencil and 1 / (1 + Psi) are the same in every iteration and the
+// deposited J_perp is (a.x - k By, a.y + k Bx) with k = qt m dzeta beta_0.  The slice's first
+// trial pass writes these, the later ones read them and gather B_perp alone.
+template <typename T> struct TrialCache {
+  int2* idx;      // first stencil node (iy << 16 | ix & 0xffff) at the particle (x), at the trial position (y;
+                  // kNoTrial: the particle or its trial state is out)
+  V2<T>* e;       // stencil offsets at the particle (shape_offset)
+  V2<T>* te;      // and at the trial position
+  V2<T>* a;       // (q w / A) / (1 + Psi_trial) times u_perp of the trial step without B_perp
+  T* qt;          // (q w / A) / (1 + Psi_trial)
+  // for the final pass.  FP32: the gathered ExmBy, EypBx, Ez, Bz
+  float4* f4;
+  // FP64: A, C, f_Psi and 1 / (1 + Psi); 1 / (1 + Psi_trial) and the trial state's x, y, Psi (the
+  // final step moves them as the trial step does)
+  V4<T>* rate;
+  T* tg;
+  double *tx, *ty, *tpsi;
+};
+constexpr int kNoTrial = (int)0x80000000;
+
 // Plasma slice, structure of arrays.  x, y, psi are FP64 accumulators in both
 // modes; the rest is of the field type T.
 template <typename T> struct Plasma {
@@ -80,9 +102,7 @@ template <typename T> struct Plasma {
   // f_{i-k}, [5][n]: the same for all predictor-corrector trial passes of the slice, so they
   // read 5 values instead of the 20 of the ring (written by the final pass).
   float* hsum;
-  // FP32 mode: ExmBy, EypBx, Ez, Bz gathered at the slice's first predictor-corrector iteration,
-  // read by the later ones of the same slice (only Bx, By change between them)
-  float4* f4;
+  TrialCache<T> tc;
   // With the re-sort (resort_every > 0): each particle's index in the initial placement (its
   // ion's position is recomputed from it); null otherwise (the array index is that index).
   int32_t* origin;
@@ -240,7 +260,7 @@ struct hq_grid_s {
   unsigned long long* d_gbar;                // grid-barrier counter of the fused solve kernel (zero between launches)
   int fault_barrier;                         // HQ_FAULT_BARRIER=1: the solve's first grid barrier never fills
   int no_f4;                                 // HQ_NO_F4CACHE=1: every trial pass gathers all six fields
-  int f4_slice;                              // slice whose first trial pass filled p32.f4 (-1: none)
+  int f4_slice;                              // slice whose first trial pass filled the trial cache (-1: none)
   int sep_src;                               // HQ_SEPARATE_SRC=1: source kernels ahead of the solve launches
 
   // beams
@@ -426,6 +446,29 @@ __device__ __forceinline__ int shape_weights(int jf, T d, T* w) {
     w[2] = (T(1) + T(3) * d + T(3) * d2 - T(3) * d3) * T(1.0 / 6.0);
     w[3] = d3 * T(1.0 / 6.0);
     return jf - 1;
+  }
+}
+
+// The same weights in two steps: the first node and the offset the weights are formed from, which
+// can be kept per particle, then the weights.
+template <int P, typename T> __device__ __forceinline__ int shape_offset(int jf, T d, T& e) {
+  e = d;
+  if constexpr (P == 0) return jf + (d >= T(0.5) ? 1 : 0);
+  if constexpr (P == 2) {
+    const bool up = d >= T(0.5);
+    e = up ? d - T(1) : d;
+    return jf + (up ? 1 : 0) - 1;
+  }
+  return P == 3 ? jf - 1 : jf;
+}
+template <int P, typename T> __device__ __forceinline__ void shape_from_offset(T e, T* w) {
+  if constexpr (P == 2) {
+    const T a = T(0.5) - e, b = T(0.5) + e;
+    w[0] = T(0.5) * a * a;
+    w[1] = T(0.75) - e * e;
+    w[2] = T(0.5) * b * b;
+  } else {
+    shape_weights<P, T>(0, e, w);
   }
 }
 

@@ -81,12 +81,40 @@ __device__ __forceinline__ F6<T> gather6(const T* __restrict__ gf, const T* __re
   return F;
 }
 
-// Bx, By alone at the same stencil, accumulated node by node exactly as gather6 does (the same
-// products and sums in the same order, so the result is bit for bit gather6's v[3], v[4]).
-template <int P>
-__device__ __forceinline__ float2 gather_bperp(const float* __restrict__ bm, int nx, int ny, int ix0, int iy0,
-                                               const float* wx, const float* wy) {
-  float bx = 0.0f, by = 0.0f;
+__device__ __forceinline__ V2<float> load_b(const float* b) {
+  const float2 c = __ldg(reinterpret_cast<const float2*>(b));
+  return V2<float>{c.x, c.y};
+}
+__device__ __forceinline__ V2<double> load_b(const double* b) {
+  const double2 c = __ldg(reinterpret_cast<const double2*>(b));
+  return V2<double>{c.x, c.y};
+}
+
+// Bx, By alone at the same stencil, accumulated node by node as gather6 does.  BATCH: a stencil
+// inside the array (wall nodes hold zeros) is read without per-node checks, all loads first; not
+// in the FP32 final pass, whose 48 registers it would spill (33 us with the checks, 41 without,
+// at 262144 particles, quadratic shape).
+template <int P, typename T, bool BATCH = true>
+__device__ __forceinline__ V2<T> gather_bperp(const T* __restrict__ bm, int nx, int ny, int ix0, int iy0, const T* wx,
+                                              const T* wy) {
+  T bx = T(0), by = T(0);
+  if (BATCH && ix0 >= 0 && iy0 >= 0 && ix0 + P < nx && iy0 + P < ny) {
+    const T* r = bm + ((int64_t)iy0 * nx + ix0) * 2;
+    V2<T> c[P + 1][P + 1];
+#pragma unroll
+    for (int b = 0; b <= P; ++b)
+#pragma unroll
+      for (int a = 0; a <= P; ++a) c[b][a] = load_b(r + ((int64_t)b * nx + a) * 2);
+#pragma unroll
+    for (int b = 0; b <= P; ++b)
+#pragma unroll
+      for (int a = 0; a <= P; ++a) {
+        const T wgt = wx[a] * wy[b];
+        bx += wgt * c[b][a].a;
+        by += wgt * c[b][a].b;
+      }
+    return V2<T>{bx, by};
+  }
 #pragma unroll
   for (int b = 0; b <= P; ++b) {
     const int iy = iy0 + b;
@@ -95,13 +123,13 @@ __device__ __forceinline__ float2 gather_bperp(const float* __restrict__ bm, int
     for (int a = 0; a <= P; ++a) {
       const int ix = ix0 + a;
       if (!in_interior(ix, nx)) continue;
-      const float2 c = __ldg(reinterpret_cast<const float2*>(bm + ((int64_t)iy * nx + ix) * 2));
-      const float wgt = wx[a] * wy[b];
-      bx += wgt * c.x;
-      by += wgt * c.y;
+      const V2<T> c = load_b(bm + ((int64_t)iy * nx + ix) * 2);
+      const T wgt = wx[a] * wy[b];
+      bx += wgt * c.a;
+      by += wgt * c.b;
     }
   }
-  return make_float2(bx, by);
+  return V2<T>{bx, by};
 }
 
 // zeta-derivatives of a plasma particle, Sec. 3.2; opp = 1 + Psi.  Written for an electron
@@ -122,6 +150,25 @@ __device__ __forceinline__ void derivs(T ux, T uy, T opp, const F6<T>& F, T* f, 
     f[4] = mqm * f[4];
   }
 }
+
+// The rates that do not depend on B_perp (TrialCache::rate): f_ux = A + m By, f_uy = C - m Bx.
+template <typename T, bool MS>
+__device__ __forceinline__ V4<T> rates_without_b(T ux, T uy, T opp, const F6<T>& F, T mqm) {
+  const T g = T(1) / opp;
+  const T gam = (T(1) + ux * ux + uy * uy + opp * opp) * T(0.5) * g;
+  V4<T> r{gam * g * F.v[0] + F.v[5] * g * uy, gam * g * F.v[1] - F.v[5] * g * ux,
+          g * (ux * F.v[0] + uy * F.v[1]) - F.v[2], g};
+  if constexpr (MS) {
+    r.a *= mqm;
+    r.b *= mqm;
+    r.c *= mqm;
+  }
+  return r;
+}
+
+__device__ __forceinline__ int pack_node(int iy, int ix) { return (iy << 16) | (ix & 0xffff); }
+__device__ __forceinline__ int node_x(int i) { return (int)(short)(i & 0xffff); }
+__device__ __forceinline__ int node_y(int i) { return i >> 16; }
 
 // A particle's species constants on a multi-species grid (MS), else the electron's: -q/M,
 // q/M (the chi factor q^2/M over q) and q, in the kernel's type.
@@ -185,6 +232,17 @@ template <int P, typename T>
 __device__ __forceinline__ void deposit_perp(V2<T>* tj, const Geom& gm, int ix0, int iy0,
                                              const T* wx, const T* wy, T jx, T jy) {
   const int nx = gm.nx, ny = gm.ny;
+  if (ix0 >= 1 && iy0 >= 1 && ix0 + P < nx && iy0 + P < ny) {   // no wall node in the stencil
+    V2<T>* r = tj + (int64_t)iy0 * nx + ix0;
+#pragma unroll
+    for (int b = 0; b <= P; ++b)
+#pragma unroll
+      for (int a = 0; a <= P; ++a) {
+        const T wgt = wx[a] * wy[b];
+        atomic_add2(r + (int64_t)b * nx + a, wgt * jx, wgt * jy, gm);
+      }
+    return;
+  }
 #pragma unroll
   for (int b = 0; b <= P; ++b) {
     const int iy = iy0 + b;
@@ -353,20 +411,24 @@ __global__ void k_species_c0(Plasma<float> pl, Geom gm, double* out, SpeciesTab 
 
 // ---------------------------------------------------------------- trial pass (predictor-corrector)
 // Gather with B^(m-1), AB5 trial step to slice i+1, deposit J_perp of the trial
-// particles into tj (Sec. 3.2, predictor-corrector field solver).  Within a slice only Bx, By
-// change between the iterations: the FP32 path gathers the other four fields (ExmBy, EypBx,
-// Ez, Bz) in the first iteration and keeps them per particle in pl.f4 (fmode 1), and the later
-// iterations read them back and gather Bx, By alone (FM 2); FM 0 gathers all six.
+// particles into tj (Sec. 3.2, predictor-corrector field solver).  A slice's first iteration
+// (FM 1) also writes the trial cache that its later iterations (k_trial_lin) and the final pass
+// read; FM 0 (HQ_NO_F4CACHE=1) evaluates everything in every iteration.
 template <int P, typename T, bool CACHE, bool MS, int FM>
 __global__ void __launch_bounds__(kThreads) k_trial_pass(Plasma<T> pl, Geom gm, const T* __restrict__ gf, const T* __restrict__ bm,
                                                          V2<T>* tj, int slice, double guard, SpeciesTab tab) {
   pdl_trigger();
   pdl_wait();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= pl.n || !pl.alive[p]) return;
+  if (p >= pl.n) return;
+  if (!pl.alive[p]) {
+    if constexpr (FM == 1) pl.tc.idx[p] = make_int2(0, kNoTrial);
+    return;
+  }
   const SpC<T> sc = spc_of<T, MS>(tab, MS ? species_of(tab, p) : 0);
   const int64_t n = pl.n;
   T wx[P + 1], wy[P + 1];
+  T ex, ey;
   int ix0, iy0;
   T opp;
   int jx = 0, jy = 0;
@@ -377,25 +439,23 @@ __global__ void __launch_bounds__(kThreads) k_trial_pass(Plasma<T> pl, Geom gm, 
     jy = cell >> 16;
     fxr = T(pl.fx[p]);
     fyr = T(pl.fy[p]);
-    ix0 = shape_weights<P, T>(jx, fxr, wx);
-    iy0 = shape_weights<P, T>(jy, fyr, wy);
     opp = T(pl.opp[p]);
   } else {
-    stencil_f64<P, T>(gm, pl.x[p], pl.y[p], ix0, iy0, wx, wy);
+    double dx, dy;
+    split_coord(pl.x[p], gm.xmin, gm.dx, jx, dx);
+    split_coord(pl.y[p], gm.ymin, gm.dy, jy, dy);
+    fxr = T(dx);
+    fyr = T(dy);
     opp = T(1.0 + pl.psi[p]);
   }
+  ix0 = shape_offset<P, T>(jx, fxr, ex);
+  iy0 = shape_offset<P, T>(jy, fyr, ey);
+  shape_from_offset<P, T>(ex, wx);
+  shape_from_offset<P, T>(ey, wy);
   const T ux = pl.ux[p], uy = pl.uy[p];
-  F6<T> F;
-  if constexpr (CACHE && FM == 2) {
-    const float4 c = pl.f4[p];
-    const float2 b = gather_bperp<P>(bm, gm.nx, gm.ny, ix0, iy0, wx, wy);
-    F.v[0] = c.x; F.v[1] = c.y; F.v[2] = c.z; F.v[3] = b.x; F.v[4] = b.y; F.v[5] = c.w;
-  } else {
-    F = gather6<P, T>(gf, bm, gm.nx, gm.ny, ix0, iy0, wx, wy);
-    if constexpr (CACHE && FM == 1) pl.f4[p] = make_float4(F.v[0], F.v[1], F.v[2], F.v[5]);
-  }
-  T f[5];
-  derivs<T, MS>(ux, uy, opp, F, f, sc.mqm);
+  const F6<T> F = gather6<P, T>(gf, bm, gm.nx, gm.ny, ix0, iy0, wx, wy);
+  const V4<T> r = rates_without_b<T, MS>(ux, uy, opp, F, sc.mqm);
+  const T f[5] = {-ux * r.d, -uy * r.d, r.a, r.b, r.c};   // f[2], f[3] without B_perp
   const T dz = CACHE ? T(gm.f_dz) : T(gm.dzeta);
   // AB5 combination beta_0 f_i + sum_{k>=1} beta_k f_{i-k}; FP32 reads the precomputed history part
   auto comb = [&](int c) -> T {
@@ -404,12 +464,14 @@ __global__ void __launch_bounds__(kThreads) k_trial_pass(Plasma<T> pl, Geom gm, 
   };
   const T cx = comb(0);
   const T cy = comb(1);
-  const T tux = ux - dz * comb(2);
-  const T tuy = uy - dz * comb(3);
+  const T ax0 = ux - dz * comb(2);   // trial u_perp without B_perp
+  const T ay0 = uy - dz * comb(3);
   const T cpsi = comb(4);
-  T twx[P + 1], twy[P + 1];
+  T tex, tey;
   int tix0, tiy0;
   T topp;
+  bool ok;
+  double tx = 0.0, ty = 0.0, tpsi = 0.0;
   if constexpr (CACHE) {
     // trial step in cell-relative coordinates (FP32 only)
     T ux_ = fxr - T(gm.f_dz_inv_dx) * cx;
@@ -420,22 +482,84 @@ __global__ void __launch_bounds__(kThreads) k_trial_pass(Plasma<T> pl, Geom gm, 
     uy_ -= fly;
     topp = opp - dz * cpsi;
     const T ax = T(tjx) + ux_, ay = T(tjy) + uy_;
-    const bool ok = isfinite(ax) && isfinite(ay) && isfinite(topp) && ax > T(0) && ax < T(gm.nx) &&
-                    ay > T(0) && ay < T(gm.ny) && topp >= T(gm.f_guard);
-    if (!ok) return;
-    tix0 = shape_weights<P, T>(tjx, ux_, twx);
-    tiy0 = shape_weights<P, T>(tjy, uy_, twy);
+    ok = isfinite(ax) && isfinite(ay) && isfinite(topp) && ax > T(0) && ax < T(gm.nx) && ay > T(0) && ay < T(gm.ny) &&
+         topp >= T(gm.f_guard);
+    tix0 = shape_offset<P, T>(tjx, ux_, tex);
+    tiy0 = shape_offset<P, T>(tjy, uy_, tey);
   } else {
-    const double tx = pl.x[p] - (double)dz * (double)cx;
-    const double ty = pl.y[p] - (double)dz * (double)cy;
-    const double tpsi = pl.psi[p] - (double)dz * (double)cpsi;
-    if (!state_ok(gm, tx, ty, 1.0 + tpsi, guard)) return;
+    tx = pl.x[p] - (double)dz * (double)cx;
+    ty = pl.y[p] - (double)dz * (double)cy;
+    tpsi = pl.psi[p] - (double)dz * (double)cpsi;
     topp = T(1.0 + tpsi);
-    stencil_f64<P, T>(gm, tx, ty, tix0, tiy0, twx, twy);
+    ok = state_ok(gm, tx, ty, 1.0 + tpsi, guard);
+    int tjx, tjy;
+    double dx, dy;
+    split_coord(tx, gm.xmin, gm.dx, tjx, dx);
+    split_coord(ty, gm.ymin, gm.dy, tjy, dy);
+    tix0 = shape_offset<P, T>(tjx, T(dx), tex);
+    tiy0 = shape_offset<P, T>(tjy, T(dy), tey);
   }
-  const T qw = charge_density<T>(pl.w[p], gm, sc.q);
   const T tg = T(1) / topp;
-  deposit_perp<P, T>(tj, gm, tix0, tiy0, twx, twy, qw * tux * tg, qw * tuy * tg);
+  const T qt = charge_density<T>(pl.w[p], gm, sc.q) * tg;
+  const T k = qt * (sc.mqm * dz * T(ab5(0)));
+  if constexpr (FM == 1) {
+    const TrialCache<T>& tc = pl.tc;
+    tc.idx[p] = make_int2(pack_node(iy0, ix0), ok ? pack_node(tiy0, tix0) : kNoTrial);
+    tc.e[p] = V2<T>{ex, ey};
+    tc.te[p] = V2<T>{tex, tey};
+    tc.a[p] = V2<T>{qt * ax0, qt * ay0};
+    tc.qt[p] = qt;
+    if constexpr (sizeof(T) == 4) {
+      tc.f4[p] = make_float4(F.v[0], F.v[1], F.v[2], F.v[5]);
+    } else {
+      tc.rate[p] = r;
+      tc.tg[p] = tg;
+      tc.tx[p] = tx;
+      tc.ty[p] = ty;
+      tc.tpsi[p] = tpsi;
+    }
+  }
+  if (!ok) return;
+  T twx[P + 1], twy[P + 1];
+  shape_from_offset<P, T>(tex, twx);
+  shape_from_offset<P, T>(tey, twy);
+  deposit_perp<P, T>(tj, gm, tix0, tiy0, twx, twy, qt * ax0 - k * F.v[4], qt * ay0 + k * F.v[3]);
+}
+
+// The later iterations of a slice: what they share is in the trial cache, so an iteration reads
+// 36 B per particle (FP32) instead of 65 B, gathers B_perp and deposits.  FP32 is bound by memory
+// latency and the atomics (262144 particles, quadratic: 12.4 -> 9.3 us; 4.2e6, cubic: 161 -> 134 us),
+// FP64 by its pipe (100 instead of 300 FP64 instructions: 133 -> 52 us).
+template <int P, typename T, bool MS>
+__global__ void __launch_bounds__(kThreads) k_trial_lin(TrialCache<T> tc, int64_t n, Geom gm, const T* __restrict__ bm, V2<T>* tj, SpeciesTab tab) {
+  pdl_trigger();
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  // FP32: the launch before is the cooperative solve, which started after the trial pass that
+  // filled the cache had ended: the cache is read while that solve drains.  (The FP64 solve's
+  // launches overlap their predecessors: wait first.)
+  if constexpr (sizeof(T) == 8) pdl_wait();
+  const bool in = p < n;
+  const int2 idx = in ? tc.idx[p] : make_int2(0, kNoTrial);
+  const bool ok = idx.y != kNoTrial;
+  V2<T> e{}, te{}, a{};
+  T k = T(0);
+  if (ok) {
+    e = tc.e[p];
+    te = tc.te[p];
+    a = tc.a[p];
+    const SpC<T> sc = spc_of<T, MS>(tab, MS ? species_of(tab, p) : 0);
+    k = tc.qt[p] * (sc.mqm * (sizeof(T) == 8 ? T(gm.dzeta) : T(gm.f_dz)) * T(ab5(0)));
+  }
+  T wx[P + 1], wy[P + 1];
+  shape_from_offset<P, T>(e.a, wx);
+  shape_from_offset<P, T>(e.b, wy);
+  if constexpr (sizeof(T) == 4) pdl_wait();
+  if (!ok) return;
+  const V2<T> b = gather_bperp<P, T>(bm, gm.nx, gm.ny, node_x(idx.x), node_y(idx.x), wx, wy);
+  T twx[P + 1], twy[P + 1];
+  shape_from_offset<P, T>(te.a, twx);
+  shape_from_offset<P, T>(te.b, twy);
+  deposit_perp<P, T>(tj, gm, node_x(idx.y), node_y(idx.y), twx, twy, a.a - k * b.b, a.b + k * b.a);
 }
 
 // ---------------------------------------------------------------- FP32 psi source
@@ -648,7 +772,7 @@ template <int P, typename T> constexpr int final_min_blocks() {
 }
 
 // FM 2 (FP32, after a predictor-corrector whose first iteration kept the slice's ExmBy, EypBx,
-// Ez, Bz per particle in pl.f4): read those back and gather the converged Bx, By alone.
+// Ez, Bz per particle in the trial cache): read those back and gather the converged Bx, By alone.
 template <int P, typename T, bool CACHE, bool MS, int FM>
 __global__ void __launch_bounds__(kThreads, final_min_blocks<P, T>()) k_final_pass(Plasma<T> pl, Geom gm, const T* __restrict__ gf, const T* __restrict__ bm,
                                                          V4<T>* dep, T* chi, float* ps, PpcInfo pc, int slice,
@@ -694,9 +818,9 @@ __global__ void __launch_bounds__(kThreads, final_min_blocks<P, T>()) k_final_pa
   const T ux = pl.ux[p], uy = pl.uy[p];
   F6<T> F;
   if constexpr (CACHE && FM == 2) {
-    const float4 c = pl.f4[p];
-    const float2 b = gather_bperp<P>(bm, gm.nx, gm.ny, ix0, iy0, wx, wy);
-    F.v[0] = c.x; F.v[1] = c.y; F.v[2] = c.z; F.v[3] = b.x; F.v[4] = b.y; F.v[5] = c.w;
+    const float4 c = pl.tc.f4[p];
+    const V2<T> b = gather_bperp<P, T, false>(bm, gm.nx, gm.ny, ix0, iy0, wx, wy);
+    F.v[0] = c.x; F.v[1] = c.y; F.v[2] = c.z; F.v[3] = b.a; F.v[4] = b.b; F.v[5] = c.w;
   } else {
     F = gather6<P, T>(gf, bm, gm.nx, gm.ny, ix0, iy0, wx, wy);
   }
@@ -776,6 +900,54 @@ __global__ void __launch_bounds__(kThreads, final_min_blocks<P, T>()) k_final_pa
     if (ps) deposit_psi_src<P>(ps, gm, jx, frx, dfx, jy, fry, dfy, s0, qw);
 }
 
+// FP64 after a predictor-corrector: the final step moves x, y and Psi exactly as the trial step
+// does (only u_perp sees B_perp), so the new position, its stencil, 1 / (1 + Psi), the removal test
+// and the rates without B_perp come from the trial cache; left are the gather of the converged
+// B_perp, u_perp, the history and the deposit.  The pass is bound by the FP64 pipe: 145 instead of
+// 350 FP64 instructions per particle (155 us -> 85 us at 262144 particles, quadratic shape).
+template <int P, bool MS>
+__global__ void __launch_bounds__(kThreads) k_final_cached(Plasma<double> pl, Geom gm, const double* __restrict__ bm,
+                                                           V4<double>* dep, double* chi, int slice,
+                                                           unsigned long long* removed, SpeciesTab tab) {
+  pdl_trigger();
+  pdl_wait();
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, n = pl.n;
+  if (p >= n || !pl.alive[p]) return;
+  const TrialCache<double>& tc = pl.tc;
+  const SpC<double> sc = spc_of<double, MS>(tab, MS ? species_of(tab, p) : 0);
+  double wx[P + 1], wy[P + 1];
+  const int2 idx = tc.idx[p];
+  const V2<double> e = tc.e[p];
+  shape_from_offset<P, double>(e.a, wx);
+  shape_from_offset<P, double>(e.b, wy);
+  const V2<double> b = gather_bperp<P, double>(bm, gm.nx, gm.ny, node_x(idx.x), node_y(idx.x), wx, wy);
+  const V4<double> r = tc.rate[p];
+  const double ux = pl.ux[p], uy = pl.uy[p];
+  const double f[5] = {-ux * r.d, -uy * r.d, r.a + sc.mqm * b.b, r.b - sc.mqm * b.a, r.c};
+  const double nux = ux - gm.dzeta * ab5_comb<double>(pl.hist, n, p, slice, 2, f[2]);
+  const double nuy = uy - gm.dzeta * ab5_comb<double>(pl.hist, n, p, slice, 3, f[3]);
+#pragma unroll
+  for (int c = 0; c < 5; ++c) pl.hist[((int64_t)(slice % kRing) * 5 + c) * n + p] = f[c];
+  if (idx.y == kNoTrial) {
+    pl.alive[p] = 0;
+    atomicAdd(removed, 1ull);
+    return;
+  }
+  const double psi = tc.tpsi[p], opp = 1.0 + psi, g = tc.tg[p], qg = tc.qt[p];
+  pl.x[p] = tc.tx[p];
+  pl.y[p] = tc.ty[p];
+  pl.psi[p] = psi;
+  pl.ux[p] = nux;
+  pl.uy[p] = nuy;
+  const V2<double> te = tc.te[p];
+  shape_from_offset<P, double>(te.a, wx);
+  shape_from_offset<P, double>(te.b, wy);
+  const double gam = (1.0 + nux * nux + nuy * nuy + opp * opp) * 0.5 * g;
+  const double uz = uz_of<double>(nux, nuy, opp, psi, g);
+  deposit_full<P, double>(dep, chi, gm, node_x(idx.y), node_y(idx.y), wx, wy, qg * gam, qg * nux, qg * nuy, qg * uz,
+                          qg * sc.qm);
+}
+
 template <typename T> Plasma<T> plasma_of(const hq_grid_s* g);
 template <> Plasma<double> plasma_of<double>(const hq_grid_s* g) { return g->p64; }
 template <> Plasma<float> plasma_of<float>(const hq_grid_s* g) { return g->p32; }
@@ -833,21 +1005,22 @@ void launch_species_c0(const hq_grid_s* g, double* out, cudaStream_t s) {
 template <typename T>
 void launch_trial_pass(const hq_grid_s* g, int slice, int iter, cudaStream_t s) {
   const unsigned nb = blocks_for(g->np);
-  // FP32: the first predictor-corrector iteration of a slice keeps the four static gathered
-  // fields per particle, the others read them (HQ_NO_F4CACHE=1: every pass gathers all six)
-  const int fmode = (sizeof(T) == 8 || g->no_f4) ? 0 : (iter == 0 ? 1 : 2);
   const T* gf = reinterpret_cast<const T*>(g->gf);
   const T* bm = reinterpret_cast<const T*>(g->bm);
   V2<T>* tj = reinterpret_cast<V2<T>*>(g->tj);
   constexpr bool C = sizeof(T) == 4;
   const double gd = g->d.psi_guard;
+  const Plasma<T> pl = plasma_of<T>(g);
+  if (!g->no_f4 && iter > 0) {
+    HQ_PDISPATCH(g->d.shape_order, g->multi,
+                 (launch_pdl(k_trial_lin<P, T, M>, nb, kThreads, 0, s, pl.tc, g->np, g->geom, bm, tj, g->sp)));
+    return;
+  }
   HQ_PDISPATCH(g->d.shape_order, g->multi,
-               (fmode == 2 ? launch_pdl(k_trial_pass<P, T, C, M, C ? 2 : 0>, nb, kThreads, 0, s, plasma_of<T>(g), g->geom,
-                                        gf, bm, tj, slice, gd, g->sp)
-                : fmode == 1 ? launch_pdl(k_trial_pass<P, T, C, M, C ? 1 : 0>, nb, kThreads, 0, s, plasma_of<T>(g),
-                                          g->geom, gf, bm, tj, slice, gd, g->sp)
-                             : launch_pdl(k_trial_pass<P, T, C, M, 0>, nb, kThreads, 0, s, plasma_of<T>(g), g->geom, gf,
-                                          bm, tj, slice, gd, g->sp)));
+               (g->no_f4 ? launch_pdl(k_trial_pass<P, T, C, M, 0>, nb, kThreads, 0, s, pl, g->geom, gf, bm, tj, slice,
+                                      gd, g->sp)
+                         : launch_pdl(k_trial_pass<P, T, C, M, 1>, nb, kThreads, 0, s, pl, g->geom, gf, bm, tj, slice,
+                                      gd, g->sp)));
 }
 
 template <typename T>
@@ -860,6 +1033,12 @@ void launch_final_pass(const hq_grid_s* g, int slice, void* dep, void* chi, bool
   constexpr bool C = sizeof(T) == 4;
   const double gd = g->d.psi_guard;
   unsigned long long* rm = g->d_removed;
+  if constexpr (!C)
+    if (f4) {
+      HQ_PDISPATCH(g->d.shape_order, g->multi,
+                   (launch_pdl(k_final_cached<P, M>, nb, kThreads, 0, s, g->p64, g->geom, bm, d, c, slice, rm, g->sp)));
+      return;
+    }
   float* ps = psrc_of(g, dep);
   PpcInfo pc;
   pc.px = g->d.ppc_x;
