@@ -80,13 +80,14 @@ void free_all(hq_grid_s* g) {
   F(g->c0);
   F(g->porigin); F(g->sort_key); F(g->sort_perm); F(g->sort_count); F(g->sort_offset); F(g->sort_tsum);
   F(g->sort_scratch);
-  for (int i = 0; i < 2; ++i) { F(g->dep[i]); F(g->chi[i]); F(g->op_hi[i]); F(g->op_lo[i]); F(g->psrc[i]); }
+  for (int i = 0; i < 2; ++i) { F(g->dep[i]); F(g->chi[i]); F(g->psrc[i]); }
+  for (int i = 0; i < 3; ++i) { F(g->op_hi[i]); F(g->op_lo[i]); }
   F(g->rho_ion); F(g->tj); F(g->bsrc0); F(g->bjn); F(g->bjp); F(g->xs4); F(g->xs1); F(g->pcg_r); F(g->pcg_p); F(g->pcg_s);
   F(g->pcg_part);
   F(g->d_pcres);
   F(g->scale_h); F(g->gf); F(g->bm); F(g->psi); F(g->bprev1); F(g->solved);
   F(g->f64_a); F(g->f64_b); F(g->f64_scale); F(g->tw_x); F(g->tw_y); F(g->sin_x); F(g->sin_y);
-  F(g->sx_hi); F(g->sx_lo); F(g->sy_hi); F(g->sy_lo); F(g->f32_scale);
+  F(g->sx_hi); F(g->sx_lo); F(g->sy_hi); F(g->sy_lo); F(g->fxt); F(g->fyt); F(g->f32_scale);
   for (int b = 0; b < kMaxBeams; ++b) {
     F(g->bins[b].bin); F(g->bins[b].count); F(g->bins[b].offset); F(g->bins[b].cursor); F(g->bins[b].perm);
   }
@@ -1181,15 +1182,16 @@ hq_status hq_grid_create(const hq_grid_desc* desc, void* cuda_stream, hq_grid_t*
     // folded DST-I (half the contraction) when both extents are multiples of 128
     const char* nf = std::getenv("HQ_NO_FOLD");
     g->fold = (g->nx % 128 == 0 && g->ny % 128 == 0 && !(nf && nf[0] == '1')) ? 1 : 0;
-    const char* nsc = std::getenv("HQ_NO_SRCCACHE");
-    g->no_srccache = nsc && nsc[0] == '1';
     const char* fb = std::getenv("HQ_FAULT_BARRIER");
     g->fault_barrier = (fb && fb[0] == '1') ? 1 : 0;
-    HQ_ALLOC(g->d_gbar, sizeof(unsigned long long));
-    cudaMemset(g->d_gbar, 0, sizeof(unsigned long long));
+    const int cl = dst_tc_cluster_mode(g);
+    const char* nsc = std::getenv("HQ_NO_SRCCACHE");
+    g->no_srccache = nsc && nsc[0] == '1';
+    HQ_ALLOC(g->d_gbar, kGbarBytes);
+    cudaMemset(g->d_gbar, 0, kGbarBytes);
     const size_t opn = (size_t)kMaxRhs * g->nxp * g->nyp;
     const size_t esz = g->tf32 ? 4 : 2;   // bytes per split operand element
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < (dst_tc_resident(g) ? 3 : 2); ++i) {
       HQ_ALLOC(g->op_hi[i], esz * opn);
       HQ_ALLOC(g->op_lo[i], esz * opn);
       cudaMemset(g->op_hi[i], 0, esz * opn);
@@ -1197,7 +1199,7 @@ hq_status hq_grid_create(const hq_grid_desc* desc, void* cuda_stream, hq_grid_t*
     }
     // S (zero-padded [np][np]) or, folded, the fold matrix [n][n/2]; split into hi + lo (bf16,
     // or TF32 in FP32 words)
-    auto smat = [&](int n, int np_, void** hi, void** lo) -> hq_status {
+    auto smat = [&](int n, int np_, void** hi, void** lo, void** tm) -> hq_status {
       const int cols = g->fold ? n / 2 : np_;
       const std::vector<double> fm = g->fold ? fold_matrix(n) : std::vector<double>();
       const size_t cnt = (size_t)np_ * cols;
@@ -1217,12 +1219,29 @@ hq_status hq_grid_create(const hq_grid_desc* desc, void* cuda_stream, hq_grid_t*
             l[o] = __float2bfloat16_rn(v - __bfloat162float(vh));
           }
         }
+      if (cl >= 0 || dst_tc_resident(g)) {
+        // [block of 128 rows][hi, lo][8-column group][row][8 bf16]: what a lane stores as 4 columns
+        // (128 x 128 folded: 128 columns, zeros where the slot's half is the other one)
+        const bool both = cl == 2;
+        const int tc = both ? np_ : cols, groups = tc / 8;
+        std::vector<__nv_bfloat16> tv(2 * (size_t)np_ * tc, __float2bfloat16_rn(0.0f));
+        for (int k = 0; k < np_; ++k)
+          for (int j = 0; j < cols; ++j)
+            for (int z = 0; z < 2; ++z) {
+              const int c = j + (both && k >= n / 2 ? cols : 0);
+              tv[((((size_t)(k / 128) * 2 + z) * groups + c / 8) * 128 + k % 128) * 8 + c % 8] =
+                  (z ? l : h)[(size_t)k * cols + j];
+            }
+        if (dalloc(tm, 2 * tv.size()) != cudaSuccess) return HQ_ERR_OOM;
+        cudaMemcpy(*tm, tv.data(), 2 * tv.size(), cudaMemcpyHostToDevice);
+      }
       if (dalloc(hi, esz * cnt) != cudaSuccess || dalloc(lo, esz * cnt) != cudaSuccess) return HQ_ERR_OOM;
       cudaMemcpy(*hi, g->tf32 ? (const void*)hf.data() : (const void*)h.data(), esz * cnt, cudaMemcpyHostToDevice);
       cudaMemcpy(*lo, g->tf32 ? (const void*)lf.data() : (const void*)l.data(), esz * cnt, cudaMemcpyHostToDevice);
       return HQ_OK;
     };
-    if (smat(g->nx, g->nxp, &g->sx_hi, &g->sx_lo) != HQ_OK || smat(g->ny, g->nyp, &g->sy_hi, &g->sy_lo) != HQ_OK) {
+    if (smat(g->nx, g->nxp, &g->sx_hi, &g->sx_lo, &g->fxt) != HQ_OK ||
+        smat(g->ny, g->nyp, &g->sy_hi, &g->sy_lo, &g->fyt) != HQ_OK) {
       g->err = "DST matrix allocation failed";
       return bail(HQ_ERR_OOM);
     }
@@ -1595,6 +1614,12 @@ hq_status hq_poisson_solve(hq_grid_t g, const void* src, void* dst, int32_t nrhs
     dst_solve_f64(g, nrhs, s, nullptr, static_cast<const double*>(src), static_cast<double*>(dst));
     return check_launch(g);
   }
+  if (!g->sep_src && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
+    // one launch from the caller's sources to the caller's array
+    Prof p(g, HQ_K_DST, 1);
+    dst_solve_tc_given(g, nrhs, static_cast<const float*>(src), static_cast<float*>(dst), s);
+    return check_launch(g);
+  }
   {
     Prof p(g, HQ_K_FIELD, 1);
     launch_src_copy<float>(g, src, nrhs, s);
@@ -1632,7 +1657,7 @@ hq_status hq_sync(hq_grid_t g, int64_t* removed) {
   if (status) {
     HQ_CUDA(g, cudaMemset(g->d_status, 0, sizeof(int)));
     if (status & DEV_TIMEOUT) {
-      if (g->d_gbar) HQ_CUDA(g, cudaMemset(g->d_gbar, 0, sizeof(unsigned long long)));  // an aborted solve left it
+      if (g->d_gbar) HQ_CUDA(g, cudaMemset(g->d_gbar, 0, kGbarBytes));  // as an aborted solve left them
       return fail(g, HQ_ERR_TIMEOUT, "a bounded device wait ran out (tensor-core DST)");
     }
     if (status & DEV_NONFINITE)

@@ -251,13 +251,14 @@ struct hq_grid_s {
   // DST, FP32/bf16x3: padded operand buffers and sine matrices
   int nxp, nyp;
   // elements: bf16, or (tf32) FP32 words holding TF32 values
-  void *op_hi[2], *op_lo[2];                // ping-pong [kMaxRhs * max(nxp,nyp)^2]
+  void *op_hi[3], *op_lo[3];                // [kMaxRhs * max(nxp,nyp)^2] ([2]: resident fold-matrix solve only)
   void *sx_hi, *sx_lo, *sy_hi, *sy_lo;
+  void *fxt, *fyt;     // resident and cluster solves: the same matrices as tensor-memory columns (else null)
   float* f32_scale;                          // [nyp][nxp] (1/lambda)(4/(nx ny)), slot order if folded
   hq::TensorMaps* tmaps;
   int fold;                                  // folded DST-I (nx, ny multiples of 128; FP32 mode)
   float* psrc[2];                            // FP32 mode: psi source rho - J_z of dep[0], dep[1]
-  unsigned long long* d_gbar;                // grid-barrier counter of the fused solve kernel (zero between launches)
+  unsigned long long* d_gbar;                // barrier and dependency counters of the fused solves (zero between launches)
   int fault_barrier;                         // HQ_FAULT_BARRIER=1: the solve's first grid barrier never fills
   int no_f4;                                 // HQ_NO_F4CACHE=1: every trial pass gathers all six fields
   int f4_slice;                              // slice whose first trial pass filled the trial cache (-1: none)
@@ -354,6 +355,10 @@ double dst_f64_norm(int nx, int ny);   // factor of the FP64 scale table (see k_
 int dst_f64_launches(const hq_grid_s* g);   // kernel launches of one FP64 solve
 void dst_solve_tc(hq_grid_s* g, int nrhs, cudaStream_t s);
 void dst_solve_tc_shifted(hq_grid_s* g, int nrhs, cudaStream_t s);   // (L - c)^{-1}: g->scale_h
+void dst_solve_tc_given(hq_grid_s* g, int nrhs, const float* src, float* dst, cudaStream_t s);
+int dst_tc_cluster_mode(const hq_grid_s* g);             // 0, 1, 2: the cluster solve's mode; -1: not used
+bool dst_tc_resident(const hq_grid_s* g);                // the resident fold-matrix solve serves this grid
+constexpr size_t kGbarBytes = 128 * (1 + 16 + 3 * kMaxRhs * 4);   // exit counter, source and product counters
 void dst_solve_tc_bmix(hq_grid_s* g, int last, cudaStream_t s);   // B_perp solve + fused mixing (FP32)
 // FP32 solves with the source assembly as their first phase (no separate source kernel)
 void dst_solve_tc_main(hq_grid_s* g, const void* dep, cudaStream_t s);
@@ -860,12 +865,13 @@ template <typename T> struct SrcBperp {
   __device__ void effects(int iy, int ix) const {
     const int64_t o = (int64_t)iy * gm.nx + ix;
     tj[o] = V2<T>{T(0), T(0)};
-    if (reset_prev) {
-      prev[o] = V4<T>{rho_ion[o], T(0), T(0), T(0)};
-      chi_prev[o] = T(0);
-      if (ps_prev) ps_prev[o] = 0.0f;
-      bjn[o] = V2<T>{T(0), T(0)};
-    }
+    if (reset_prev) reset(o);
+  }
+  __device__ void reset(int64_t o) const {
+    prev[o] = V4<T>{rho_ion[o], T(0), T(0), T(0)};
+    chi_prev[o] = T(0);
+    if (ps_prev) ps_prev[o] = 0.0f;
+    bjn[o] = V2<T>{T(0), T(0)};
   }
   __device__ void operator()(int iy, int ix, T* v) const {
     eval(iy, ix, load(iy, ix), v);

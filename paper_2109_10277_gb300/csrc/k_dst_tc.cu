@@ -49,12 +49,16 @@ struct TensorMaps {
   CUtensorMap scale_h[2];     // the shifted (Helmholtz) spectral factors, same boxes (explicit solver)
   int ctas[2];                // co-resident CTAs of each width
   bool wide_only;             // HQ_SOLVE_BN=64: never use the 32-wide tiles
-  // resident fold-matrix solve (square folded grids, n = 256 or 512): the fold matrix in
-  // 128-row boxes, op[0] and op[1] in BN-row boxes ([0]: 64, [1]: 32)
+  // resident fold-matrix solve (square folded grids, n = 256 or 512) and cluster solve:
+  // op[0] .. op[2] in BN-row boxes ([0]: 64, [1]: 32)
   bool rs;
-  CUtensorMap rf_hi, rf_lo;
-  CUtensorMap rx_hi[2][2], rx_lo[2][2];   // [operand][width]
+  CUtensorMap rx_hi[3][2], rx_lo[3][2];   // [operand][width]
   int rs_ctas[2];
+  // cluster solve: its mode (0, 1, 2; -1: not used for this grid), and for 32 and 64 data rows per CTA the
+  // largest number of right-hand sides whose clusters are all resident at once
+  int cl_mode;
+  int cl_rhs[2];
+  int cl_max;   // resident clusters of mode 1
 };
 
 namespace {
@@ -359,11 +363,35 @@ __global__ void __launch_bounds__(128, 1)
 // 128-byte K block per stage, 4-stage ring), warp 1 lane 0 the MMAs (two per K step:
 // A_hi x [B_hi; B_lo] with N = 2 BN, A_lo x B_hi with N = BN, into a 2 BN-column TMEM
 // accumulator), and all 8 warps the epilogue, each warpgroup half of the columns.
+// The caller's sources [nr][ny][nx] (hq_poisson_solve); row and column 0 read zero.
+struct SrcGiven {
+  static constexpr int NR = kMaxRhs;
+  static constexpr bool kEffects = false;
+  const float* src;
+  Geom gm;
+  int nr;
+  struct In {
+    float v[kMaxRhs];
+  };
+  __device__ In load(int iy, int ix) const {
+    In q;
+    const int64_t nn = (int64_t)gm.nx * gm.ny, o = (int64_t)iy * gm.nx + ix;
+#pragma unroll
+    for (int r = 0; r < kMaxRhs; ++r) q.v[r] = (r < nr && ix > 0 && iy > 0) ? src[r * nn + o] : 0.0f;
+    return q;
+  }
+  __device__ void eval(int, int, const In& q, float* v) const {
+#pragma unroll
+    for (int r = 0; r < kMaxRhs; ++r) v[r] = q.v[r];
+  }
+  __device__ void effects(int, int) const {}
+};
+
 struct SolveArgs {
   int R;                               // right-hand sides
   int nxp, nyp;                        // operand extents (= nx, ny when folded)
   int fold;
-  void *op_hi[2], *op_lo[2];           // op[0]: [R][nyp][nxp], op[1]: [R][nxp][nyp] (bf16 or TF32 words)
+  void *op_hi[3], *op_lo[3];           // op[0]: [R][nyp][nxp], op[1]: [R][nxp][nyp] (bf16 or TF32 words)
   const float* scale;                  // [nyp][nxp]: (4/(nx ny)) / lambda, slot order when folded
   int final_mode;                      // 2: FP32 store into out [R][ny][nx]; 3: predictor-corrector mixing
   float* out;
@@ -371,22 +399,33 @@ struct SolveArgs {
   float* bm;                           // mode 3: B <- w B_solved + (1 - w) B in bm[node * 2 + r]
   float w;
   double* rsum;                        // mode 3: sum (B_new - B_old)^2, sum B_new^2 added here (or null)
-  unsigned long long* gbar;            // grid-barrier counter (zero at launch, reset by the last CTA)
+  unsigned long long* gbar;            // grid-barrier counter (zero at launch, reset by the last CTA);
+                                       // resident solve: exit counter, then the dependency counters
   int* status;
   int barrier_skew;                    // added to the first barrier's target (fault injection; 0)
   // source phase ahead of the four products: 0 none (sources already in op[0]); 1 the psi,
-  // Ez, Bz sources of a deposit record (sm); 2 the B_perp sources of the predictor-corrector (sb)
+  // Ez, Bz sources of a deposit record (sm); 2 the B_perp sources of the predictor-corrector (sb);
+  // 3 R given fields (sc)
   int pre;
   SrcMain<float> sm;
   SrcBperp<float> sb;
+  SrcGiven sc;
+  // the reset of the slice i-1 record (SrcBperp::reset) by the warps that filled tensor memory, off
+  // the source phase: the later iterations' sources (mode 2) do not read what it writes
+  int reset_late;
 };
+// Nodes of the reset, by `count` threads, this one `me`.
+__device__ __forceinline__ void reset_nodes(const SolveArgs& a, int me, int count) {
+  const int nn = a.nx * a.ny;
+  for (int o = me; o < nn; o += count) a.sb.reset(o);
+}
 
 // Source phase: every thread of the launch takes (row, column) items of the operand writer
 // in turn (consecutive threads along a row), KB items at a time: all their reads are issued
 // before any write, then the sources are evaluated, split into op[0] and the functor's own
 // writes (clearing the trial J_perp) follow.
 template <typename Sink, typename F, int NR>
-__device__ __forceinline__ void solve_sources(const Geom& gm, const Sink& sink, const F& f) {
+__device__ __forceinline__ void solve_sources(const Geom& gm, const Sink& sink, const F& f, int nr = NR) {
   constexpr int KB = 4;
   constexpr int NN = Sink::kFold ? 2 : 1;   // nodes per item
   const int w = visit_width<Sink>(gm);
@@ -418,6 +457,7 @@ __device__ __forceinline__ void solve_sources(const Geom& gm, const Sink& sink, 
       for (int j = 0; j < NN; ++j) f.eval(iy[k][j], ix[k][j], in[k][j], v[j]);
 #pragma unroll
       for (int r = 0; r < NR; ++r) {
+        if (r >= nr) break;
         if constexpr (Sink::kFold) sink.put_pair(r, t / w, t % w, v[0][r], v[NN - 1][r]);
         else sink.put(r, t / w, t % w, v[0][r]);
       }
@@ -474,6 +514,39 @@ __device__ __forceinline__ bool grid_barrier(unsigned long long* ctr, unsigned l
   }
   __syncthreads();
   return !*abort_f;
+}
+
+// Dependency counters of the resident solve, one per 128-byte line, zero at launch and reset by
+// the last CTA to leave.  A producer's arrival follows its stores, a proxy fence and a CTA barrier;
+// the consumer's TMA-issuing thread waits.
+__device__ __forceinline__ void dep_arrive(unsigned long long* c) {
+  asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(c) : "memory");
+}
+__device__ __forceinline__ bool dep_wait(const unsigned long long* c, unsigned long long target, int* status,
+                                         volatile int* abort_f) {
+  const long long t0 = clock64();
+  uint32_t it = 0;
+  while (true) {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(c) : "memory");
+    if (v >= target) break;
+    if ((++it & 15u) == 0 &&
+        ((*reinterpret_cast<volatile int*>(status) & DEV_TIMEOUT) || clock64() - t0 > (4ll << 30))) {
+      atomicOr(status, DEV_TIMEOUT);
+      *abort_f = 1;
+      return false;
+    }
+  }
+  asm volatile("fence.proxy.async;" ::: "memory");
+  return true;
+}
+
+// One lane of a converged warp, chosen without divergence the compiler cannot see through (its
+// tensor-core instructions then take their descriptors from uniform registers).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred P1;\n\telect.sync _|P1, 0xffffffff;\n\tselp.b32 %0, 1, 0, P1;\n\t}\n" : "=r"(p));
+  return p != 0;
 }
 
 // The fused solve runs 256 threads per CTA (warps 0, 1: TMA producer, MMA issuer; all 8
@@ -561,17 +634,19 @@ __global__ void __launch_bounds__(kSolveThreads, 1)
   const unsigned nb0 = a.pre ? 1u : 0u;   // barriers before phase 0
   bool go = true;
   if (a.pre) {
-    const Geom& gm = a.pre == 1 ? a.sm.gm : a.sb.gm;
+    const Geom& gm = a.pre == 1 ? a.sm.gm : (a.pre == 2 ? a.sb.gm : a.sc.gm);
     E* hi0 = reinterpret_cast<E*>(a.op_hi[0]);
     E* lo0 = reinterpret_cast<E*>(a.op_lo[0]);
     if (a.fold) {
       const SinkFold<E> sink{hi0, lo0, a.nx, a.ny};
       if (a.pre == 1) solve_sources<SinkFold<E>, SrcMain<float>, 3>(gm, sink, a.sm);
-      else solve_sources<SinkFold<E>, SrcBperp<float>, 2>(gm, sink, a.sb);
+      else if (a.pre == 2) solve_sources<SinkFold<E>, SrcBperp<float>, 2>(gm, sink, a.sb);
+      else solve_sources<SinkFold<E>, SrcGiven, kMaxRhs>(gm, sink, a.sc, a.R);
     } else {
       const SinkSplit<E> sink{hi0, lo0, a.nxp, a.nyp};
       if (a.pre == 1) solve_sources<SinkSplit<E>, SrcMain<float>, 3>(gm, sink, a.sm);
-      else solve_sources<SinkSplit<E>, SrcBperp<float>, 2>(gm, sink, a.sb);
+      else if (a.pre == 2) solve_sources<SinkSplit<E>, SrcBperp<float>, 2>(gm, sink, a.sb);
+      else solve_sources<SinkSplit<E>, SrcGiven, kMaxRhs>(gm, sink, a.sc, a.R);
     }
     go = grid_barrier(a.gbar, (unsigned long long)gridDim.x + (unsigned)a.barrier_skew, a.status, abort_f);
   }
@@ -744,25 +819,90 @@ __global__ void __launch_bounds__(kSolveThreads, 1)
   }
 }
 
+// Threads of the resident and cluster solves: warps 0-7 as in the streamed solve, 8-11 fill tensor
+// memory while the others form the sources.
+constexpr int kClThreads = 384;
+__device__ __forceinline__ void main_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }   // warps 0-7
+__device__ __forceinline__ void mma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t b, uint32_t idesc, uint32_t accum) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(tmem_d),
+      "r"(tmem_a), "l"(b), "r"(idesc), "r"(accum));
+}
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint4* v) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
+      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
+      "r"(v[0].x), "r"(v[0].y), "r"(v[0].z), "r"(v[0].w), "r"(v[1].x), "r"(v[1].y), "r"(v[1].z), "r"(v[1].w), "r"(v[2].x),
+      "r"(v[2].y), "r"(v[2].z), "r"(v[2].w), "r"(v[3].x), "r"(v[3].y), "r"(v[3].z), "r"(v[3].w), "r"(v[4].x), "r"(v[4].y),
+      "r"(v[4].z), "r"(v[4].w), "r"(v[5].x), "r"(v[5].y), "r"(v[5].z), "r"(v[5].w), "r"(v[6].x), "r"(v[6].y), "r"(v[6].z),
+      "r"(v[6].w), "r"(v[7].x), "r"(v[7].y), "r"(v[7].z), "r"(v[7].w)
+      : "memory");
+}
+
+// pc_residual_add for the first 256 threads of a block.
+__device__ __forceinline__ void residual_add_main(double* rs, double d2, double b2) {
+  __shared__ double part[2][kSolveThreads / 32];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    d2 += __shfl_down_sync(0xffffffffu, d2, o);
+    b2 += __shfl_down_sync(0xffffffffu, b2, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    part[0][threadIdx.x >> 5] = d2;
+    part[1][threadIdx.x >> 5] = b2;
+  }
+  main_sync();
+  if (threadIdx.x < 2) {
+    double s = 0.0;
+    for (int k = 0; k < kSolveThreads / 32; ++k) s += part[threadIdx.x][k];
+    if (s != 0.0) atomicAdd(rs + 2 * (int)(blockIdx.x % kResLanes) + threadIdx.x, s);
+  }
+  main_sync();
+}
+
+// A slice of the fold (or sine) matrix, 128 slots x K, into tensor memory as a tcgen05.mma A operand:
+// lane = slot, a 32-bit column = two consecutive K elements, K / 2 hi columns then K / 2 lo columns.
+// By one warp per quarter of the lanes (quarter = warp mod 4); f: hq_grid_s::fxt.
+template <int K>
+__device__ __forceinline__ void fill_tmem(const uint4* __restrict__ f, int block, uint32_t taddr, int quarter, int lane) {
+  const uint4* p = f + (int64_t)block * (K / 4) * BM + quarter * 32 + lane;
+  const uint32_t t = taddr + ((uint32_t)(quarter * 32) << 16);
+#pragma unroll 2
+  for (int g = 0; g < K / 32; ++g) {
+    uint4 v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = __ldg(p + (g * 8 + k) * BM);
+    tmem_st32(t + 32u * g, v);
+  }
+}
+
 // ---------------------------------------------------------------- resident fold-matrix solve
 // The same four products for a square folded grid (nx = ny = n, n = 256 or 512) with the
 // operand roles swapped: each CTA owns one block of 128 output slots for the whole launch,
-// so its 128 x n/2 slice of the fold matrix (bf16 hi + lo, 64 or 128 KB) is loaded into
-// shared memory once, while the source phase runs, and only the data operand (BN rows of
+// so its 128 x n/2 slice of the fold matrix (bf16 hi + lo, 64 or 128 KB) is put into tensor
+// memory once, while the source phase runs, and only the data operand (BN rows of
 // the previous phase's output) is streamed per tile:
-//   D[s][c] = sum_u F[s][u] X[c][koff + u]   (A = F in shared memory, B = X streamed),
+//   D[s][c] = sum_u F[s][u] X[c][koff + u]   (A = F in tensor memory, B = X streamed),
 // with koff = 0 for the odd-index slots (pair sums) and n/2 for the even ones (differences).
+// A from tensor memory: with A in shared memory a tcgen05.mma costs ~90 clocks here whatever its
+// N (4 KB of A at 64 B per clock; 1.4 us per product at n = 512), with A in tensor memory ~50.
 // TMEM lane = output slot s, column = data row c.  The fold of the next operand pairs
 // adjacent columns of one thread (no shuffle), and each thread stores its row of the next
 // operand as contiguous 16-byte runs.  The third product writes its rows in node order, so
 // the last one's output columns are consecutive x nodes.
+// Between the products a tile waits for its own producers only (dependency counters: the 16 tiles
+// that wrote its rows at n = 512) instead of a barrier of the whole grid.
 template <int BN> struct RsSmem {
   static constexpr int KB_MAX = 4;                          // folded K = n/2 <= 256
-  static constexpr int F = 0;                               // F_hi blocks 0..3, F_lo blocks 4..7
   static constexpr int STAGE = 2 * BN * BK * 2;             // X_hi + X_lo rows of one K block
-  static constexpr int RING = 2 * KB_MAX * A_BYTES;
-  static constexpr int BARS = RING + KB_MAX * STAGE;
+  static constexpr int RING = 0;
+  static constexpr int TILE = BM * (BN + 1) * 4;            // the mixing's staged tile
+  static constexpr int BARS = KB_MAX * STAGE > TILE ? KB_MAX * STAGE : TILE;
   static constexpr int BYTES = BARS + 256 + 1024 /*alignment*/;
+  static constexpr uint32_t TX = 128;                       // tensor-memory columns: accumulator (2 BN), F slice
 };
 
 // bf16 hi/lo split of 8 values packed for two 16-byte stores.
@@ -821,33 +961,32 @@ __device__ __forceinline__ void rs_epilogue(const SolveArgs& a, int mode, int s,
   }
 }
 
-// Source phase of the resident fold-matrix solve (square folded grid, n <= 512): a CTA takes
-// whole rows (RPP per pass, all their reads issued first), its threads read and evaluate the
-// sources at consecutive nodes of a row (coalesced), stage them in shared memory S
-// ([RPP rows][NR][n] floats), and then write the folded pairs (x_a + x_b, x_a - x_b) of
-// consecutive folded columns.
-template <typename F, int NR>
-__device__ __forceinline__ void solve_sources_rows(const Geom& gm, const F& f, const SinkFold<__nv_bfloat16>& sink,
-                                                   float* S) {
+// Source phase of the resident and cluster solves (square folded grid, n <= 512): a CTA takes
+// kSrcRows consecutive slot rows at a time (all their reads issued first), its threads read and
+// evaluate the sources at consecutive nodes of a row (coalesced), stage them in shared memory S
+// ([rows][nr][n] floats), write the folded pairs (x_a + x_b, x_a - x_b) of eight consecutive folded
+// columns each (16-byte stores), and the CTA reports the rows to the counter of their data tile.
+constexpr int kSrcRows = 4;
+template <int BN, typename F, int NR>
+__device__ __forceinline__ void solve_sources_rows(const Geom& gm, const F& f, __nv_bfloat16* hi, __nv_bfloat16* lo,
+                                                   float* S, int nr, unsigned long long* ctr) {
   constexpr int NPT = 2;   // nodes per thread per row (n <= 2 x 256)
-  constexpr int RPP = 4;   // rows per pass
-  const int n = gm.nx, w = n / 2;
-  for (int sy0 = blockIdx.x; sy0 < gm.ny; sy0 += RPP * gridDim.x) {
+  constexpr int RPP = kSrcRows;
+  const int n = gm.nx, H = n / 2;
+  for (int sy0 = RPP * blockIdx.x; sy0 < gm.ny; sy0 += RPP * gridDim.x) {
     typename F::In in[RPP][NPT];
     int iy[RPP];
 #pragma unroll
     for (int q = 0; q < RPP; ++q) {
-      const int sy = sy0 + q * gridDim.x;
-      iy[q] = sy < gm.ny ? fold_node(sy, gm.ny) : -1;
+      iy[q] = fold_node(sy0 + q, gm.ny);
 #pragma unroll
       for (int k = 0; k < NPT; ++k) {
         const int x = threadIdx.x + k * kSolveThreads;
-        in[q][k] = (iy[q] >= 0 && x < n) ? f.load(iy[q], x) : typename F::In{};
+        in[q][k] = x < n ? f.load(iy[q], x) : typename F::In{};
       }
     }
 #pragma unroll
     for (int q = 0; q < RPP; ++q) {
-      if (iy[q] < 0) continue;
 #pragma unroll
       for (int k = 0; k < NPT; ++k) {
         const int x = threadIdx.x + k * kSolveThreads;
@@ -855,24 +994,48 @@ __device__ __forceinline__ void solve_sources_rows(const Geom& gm, const F& f, c
         float v[NR];
         f.eval(iy[q], x, in[q][k], v);
 #pragma unroll
-        for (int r = 0; r < NR; ++r) S[(q * NR + r) * n + x] = v[r];
+        for (int r = 0; r < NR; ++r)
+          if (r < nr) S[(q * nr + r) * n + x] = v[r];
         if constexpr (F::kEffects) f.effects(iy[q], x);
       }
     }
-    __syncthreads();
+    main_sync();
+    const int groups = H / 8;   // of eight folded columns
+    for (int t = threadIdx.x; t < RPP * nr * groups; t += kSolveThreads) {
+      const int qr = t / groups, u0 = (t - qr * groups) * 8, q = qr / nr, r = qr - q * nr;
+      const float* row = S + qr * n;
+      float sum[8], dif[8];
 #pragma unroll
-    for (int q = 0; q < RPP; ++q) {
-      if (iy[q] < 0) continue;
-      const int sy = sy0 + q * gridDim.x;
-      for (int u = threadIdx.x; u < w; u += kSolveThreads) {
+      for (int k = 0; k < 8; ++k) {
         int xa, xb;
-        fold_pair(u, n, xa, xb);
-#pragma unroll
-        for (int r = 0; r < NR; ++r) sink.put_pair(r, sy, u, S[(q * NR + r) * n + xa], S[(q * NR + r) * n + xb]);
+        fold_pair(u0 + k, n, xa, xb);
+        const float va = row[xa], vb = row[xb];
+        const bool wall = u0 + k == n / 4;
+        sum[k] = wall ? vb : va + vb;
+        dif[k] = wall ? 0.0f : va - vb;
       }
+      const int64_t o = ((int64_t)r * gm.ny + sy0 + q) * n + u0;
+      uint4 h, l;
+      split8(sum, h, l);
+      *reinterpret_cast<uint4*>(hi + o) = h;
+      *reinterpret_cast<uint4*>(lo + o) = l;
+      split8(dif, h, l);
+      *reinterpret_cast<uint4*>(hi + o + H) = h;
+      *reinterpret_cast<uint4*>(lo + o + H) = l;
     }
-    __syncthreads();
+    asm volatile("fence.proxy.async;" ::: "memory");
+    main_sync();
+    if (threadIdx.x == 0) dep_arrive(ctr + 16 * (sy0 / BN));
   }
+}
+// The sources a launch asks for.  S: kSrcRows x R x n floats.
+template <int BN>
+__device__ __forceinline__ void solve_sources_any(const SolveArgs& a, float* S, unsigned long long* ctr) {
+  __nv_bfloat16* hi = reinterpret_cast<__nv_bfloat16*>(a.op_hi[0]);
+  __nv_bfloat16* lo = reinterpret_cast<__nv_bfloat16*>(a.op_lo[0]);
+  if (a.pre == 1) solve_sources_rows<BN, SrcMain<float>, 3>(a.sm.gm, a.sm, hi, lo, S, 3, ctr);
+  else if (a.pre == 2) solve_sources_rows<BN, SrcBperp<float>, 2>(a.sb.gm, a.sb, hi, lo, S, 2, ctr);
+  else solve_sources_rows<BN, SrcGiven, kMaxRhs>(a.sc.gm, a.sc, hi, lo, S, a.R, ctr);
 }
 
 // Predictor-corrector mixing B <- w B_solved + (1 - w) B of one tile (128 slots of y x BN
@@ -910,14 +1073,14 @@ __device__ __forceinline__ void rs_mix(const SolveArgs& a, const float* tile, in
     }
   }
   if (bad) atomicOr(a.status, DEV_NONFINITE);
-  if constexpr (RES) pc_residual_add(a.rsum, (double)d2, (double)b2);
+  if constexpr (RES) residual_add_main(a.rsum, (double)d2, (double)b2);
 }
 
-template <int BN, bool RES>
-__global__ void __launch_bounds__(kSolveThreads, 1)
-    k_dst_solve_rs(const __grid_constant__ CUtensorMap fh, const __grid_constant__ CUtensorMap fl,
-                   const __grid_constant__ CUtensorMap x0h, const __grid_constant__ CUtensorMap x0l,
-                   const __grid_constant__ CUtensorMap x1h, const __grid_constant__ CUtensorMap x1l, const SolveArgs a) {
+template <int BN, int N, bool RES>
+__global__ void __launch_bounds__(kClThreads, 1)
+    k_dst_solve_rs(const uint4* __restrict__ fxt, const __grid_constant__ CUtensorMap x0h, const __grid_constant__ CUtensorMap x0l,
+                   const __grid_constant__ CUtensorMap x1h, const __grid_constant__ CUtensorMap x1l,
+                   const __grid_constant__ CUtensorMap x2h, const __grid_constant__ CUtensorMap x2l, const SolveArgs a) {
   using L = RsSmem<BN>;
   constexpr int STAGES = L::KB_MAX;
   constexpr int CH = BN / 2;
@@ -929,29 +1092,33 @@ __global__ void __launch_bounds__(kSolveThreads, 1)
   uint64_t* bars = reinterpret_cast<uint64_t*>(basep + L::BARS);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 2);
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES), done = smem_u32(bars + 2 * STAGES);
-  const uint32_t fbar = smem_u32(bars + 2 * STAGES + 1);
+  const uint32_t tbar = smem_u32(bars + 2 * STAGES + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort_f = &s_abort;
-  const int n = a.nx, H = n / 2, nk = H / BK, MB = n / BM;
+  constexpr int n = N, H = n / 2, nk = H / BK, MB = n / BM, K = H;
   const int mb = (int)blockIdx.x % MB, s0 = mb * BM;
   const int koff = s0 < H ? 0 : H;          // odd slots (first half) contract over the pair sums
   const int NT = a.R * n / BN;               // data-row tiles per product
   const int nt0 = (int)blockIdx.x / MB, ntstep = (int)gridDim.x / MB;
+  const bool tiles = nt0 < NT;               // a CTA beyond the tiles only forms sources
+  const int NTR = n / BN;                    // data-row tiles per right-hand side
+  unsigned long long* ctr_src = a.gbar + 16; // [NTR]: source rows of a data tile formed
+  unsigned long long* ctr_p = ctr_src + 16 * NTR;   // [3][R][MB]: product p's rows of a slot block written
 
   if (threadIdx.x == 0) {
-    for (const CUtensorMap* m : {&fh, &fl, &x0h, &x0l, &x1h, &x1l}) prefetch_map(m);
+    for (const CUtensorMap* m : {&x0h, &x0l, &x1h, &x1l, &x2h, &x2l}) prefetch_map(m);
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(full0 + 8 * s, 1);
       mbar_init(empty0 + 8 * s, 1);
     }
     mbar_init(done, 1);
-    mbar_init(fbar, 1);
+    mbar_init(tbar, 128);
     s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"((uint32_t)(2 * BN))
+                 "r"(512u)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -959,37 +1126,45 @@ __global__ void __launch_bounds__(kSolveThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  // this CTA's fold-matrix slice (rows s0 .. s0 + 127, all n/2 columns), resident for the launch
-  if (threadIdx.x == 0) {
-    mbar_expect_tx(fbar, (uint32_t)(2 * nk * A_BYTES));
-    for (int kb = 0; kb < nk; ++kb) {
-      tma_load_2d(base + L::F + kb * A_BYTES, &fh, kb * BK, s0, fbar);
-      tma_load_2d(base + L::F + (STAGES + kb) * A_BYTES, &fl, kb * BK, s0, fbar);
+  if (warp >= 8) {
+    // this CTA's fold-matrix slice (slots s0 .. s0 + 127), resident for the launch
+    if (tiles) {
+      fill_tmem<K>(fxt, mb, tmem + L::TX, warp & 3, lane);
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      tc_fence_before();
+      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tbar) : "memory");
     }
+    if (a.reset_late) reset_nodes(a, (int)blockIdx.x * 128 + (int)threadIdx.x - 256, (int)gridDim.x * 128);
+    return;
   }
-  const unsigned nb0 = a.pre ? 1u : 0u;
-  bool go = true;
-  if (a.pre) {
-    // (the stage ring is idle until the first product: it holds the staged sources)
-    const SinkFold<__nv_bfloat16> sink{reinterpret_cast<__nv_bfloat16*>(a.op_hi[0]),
-                                       reinterpret_cast<__nv_bfloat16*>(a.op_lo[0]), a.nx, a.ny};
-    float* S = reinterpret_cast<float*>(basep + L::RING);   // 4 rows x 3 x 512 floats = 24 KB
-    if (a.pre == 1) solve_sources_rows<SrcMain<float>, 3>(a.sm.gm, a.sm, sink, S);
-    else solve_sources_rows<SrcBperp<float>, 2>(a.sb.gm, a.sb, sink, S);
-    go = grid_barrier(a.gbar, (unsigned long long)gridDim.x + (unsigned)a.barrier_skew, a.status, abort_f);
-  }
+  // (the stage ring is idle until the first product: it holds the staged sources)
+  if (a.pre) solve_sources_any<BN>(a, reinterpret_cast<float*>(basep + L::RING), ctr_src);
   uint32_t kb_run = 0, tiles_run = 0;
   bool f_ready = false;
-  for (int p = 0; p < 4 && go; ++p) {
-    const CUtensorMap* xh = (p & 1) ? &x1h : &x0h;
-    const CUtensorMap* xl = (p & 1) ? &x1l : &x0l;
+  for (int p = 0; p < 4; ++p) {
+    // Operands 0 -> 1 -> 2 -> 0: product 2 may overwrite operand 0, because its wait (every data
+    // tile of the right-hand side through product 1, each of which waited for a slot block of
+    // product 0) implies that all of product 0's tiles, operand 0's readers, are done; the same
+    // does not hold for operand 1 in products 1 and 2, hence the third buffer.
+    const CUtensorMap* xh = p == 1 ? &x1h : (p == 2 ? &x2h : &x0h);
+    const CUtensorMap* xl = p == 1 ? &x1l : (p == 2 ? &x2l : &x0l);
     const int mode = p == 3 ? a.final_mode : (p == 1 ? 1 : 0);
     if (p == 3) pdl_trigger();   // the next kernel may be scheduled (it waits for this grid's end)
     for (int nt = nt0; nt < NT; nt += ntstep) {
       const int c0 = nt * BN;
       if (warp == 0 && lane == 0) {
-        // data-tile producer: the whole folded K of BN rows, one stage per 64-wide K block
-        for (int kb = 0; kb < nk; ++kb) {
+        // data-tile producer: the whole folded K of BN rows, one stage per 64-wide K block, once
+        // the rows' producers have reported (the source rows of the tile, or every data tile's
+        // product with the slot block that holds these rows)
+        bool ok = true;
+        const int r_ = c0 / n, row0 = c0 - r_ * n;
+        if (p > 0)
+          ok = dep_wait(ctr_p + 16 * (((p - 1) * a.R + r_) * MB + row0 / BM),
+                        (unsigned long long)NTR + (p == 1 && !a.pre ? (unsigned)a.barrier_skew : 0u), a.status, abort_f);
+        else if (a.pre)
+          ok = dep_wait(ctr_src + 16 * (row0 / BN), (unsigned long long)(BN / kSrcRows) + (unsigned)a.barrier_skew, a.status,
+                        abort_f);
+        for (int kb = 0; ok && kb < nk; ++kb) {
           const uint32_t g = kb_run + kb;
           const int s = g % STAGES;
           const uint32_t st = base + L::RING + s * L::STAGE;
@@ -999,28 +1174,31 @@ __global__ void __launch_bounds__(kSolveThreads, 1)
           tma_load_2d(st, xh, koff + kb * BK, c0, fb);
           tma_load_2d(st + BN * BK * 2, xl, koff + kb * BK, c0, fb);
         }
-      } else if (warp == 1 && lane == 0) {
+      } else if (warp == 1) {
         // MMA issuer: A = fold-matrix slice (resident), B = [X_hi; X_lo] (N = 2 BN) and X_hi
-        bool ok = f_ready || mbar_wait_a(fbar, 0, a.status, abort_f);
+        bool ok = __all_sync(0xffffffffu, f_ready || mbar_wait_a(tbar, 0, a.status, abort_f));
         f_ready = ok;
         for (int kb = 0; ok && kb < nk; ++kb) {
           const uint32_t g = kb_run + kb;
           const int s = g % STAGES;
-          if (!mbar_wait_a(full0 + 8 * s, (g / STAGES) & 1, a.status, abort_f)) break;
+          ok = mbar_wait_a(full0 + 8 * s, (g / STAGES) & 1, a.status, abort_f);
+          if (!__all_sync(0xffffffffu, ok)) break;
           tc_fence_after();
           const uint32_t st = base + L::RING + s * L::STAGE;
-          const uint64_t ah = desc_k_sw128(base + L::F + kb * A_BYTES);
-          const uint64_t al = desc_k_sw128(base + L::F + (STAGES + kb) * A_BYTES);
+          const uint32_t ta = tmem + L::TX + (uint32_t)(kb * 32);
           const uint64_t bh = desc_k_sw128(st);
+          if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            const uint64_t off = (uint64_t)((k * 32) >> 4);
-            mma_bf16(tmem, ah + off, bh + off, Cfg<BN>::IDESC2, (kb | k) != 0 ? 1u : 0u);
-            mma_bf16(tmem, al + off, bh + off, Cfg<BN>::IDESC, 1u);
+            for (int k = 0; k < BK / 16; ++k) {
+              const uint64_t off = (uint64_t)((k * 32) >> 4);
+              mma_bf16_ta(tmem, ta + 8u * k, bh + off, Cfg<BN>::IDESC2, (kb | k) != 0 ? 1u : 0u);
+              mma_bf16_ta(tmem, ta + (uint32_t)(K / 2) + 8u * k, bh + off, Cfg<BN>::IDESC, 1u);
+            }
+            mma_commit(empty0 + 8 * s);
           }
-          mma_commit(empty0 + 8 * s);
+          __syncwarp();
         }
-        mma_commit(done);
+        if (elect_one()) mma_commit(done);
       }
       __syncwarp();
       // epilogue: TMEM lane = slot s0 + row, the two warpgroups take one half of the columns each
@@ -1054,40 +1232,462 @@ __global__ void __launch_bounds__(kSolveThreads, 1)
           float* tile = reinterpret_cast<float*>(basep + L::RING);
 #pragma unroll
           for (int j = 0; j < CH; ++j) tile[row * LD + half * CH + j] = x[j];
-          __syncthreads();
+          main_sync();
           if (!*abort_f) rs_mix<BN, RES>(a, tile, s0, r, c0 - r * n);
         } else if (!*abort_f) {
-          rs_epilogue<CH>(a, mode, s, orow, r, i0, x, sc, reinterpret_cast<__nv_bfloat16*>(a.op_hi[(p + 1) & 1]),
-                          reinterpret_cast<__nv_bfloat16*>(a.op_lo[(p + 1) & 1]));
+          const int o = p == 2 ? 0 : p + 1;
+          rs_epilogue<CH>(a, mode, s, orow, r, i0, x, sc, p < 3 ? reinterpret_cast<__nv_bfloat16*>(a.op_hi[o]) : nullptr,
+                          p < 3 ? reinterpret_cast<__nv_bfloat16*>(a.op_lo[o]) : nullptr);
         }
       }
       kb_run += nk;
       ++tiles_run;
+      if (p < 3) asm volatile("fence.proxy.async;" ::: "memory");
       tc_fence_before();
-      __syncthreads();
+      main_sync();
       tc_fence_after();
       if (*abort_f) break;
+      if (p < 3 && threadIdx.x == 0) dep_arrive(ctr_p + 16 * ((p * a.R + r) * MB + mb));
     }
     if (*abort_f) break;
-    if (p < 3 && !grid_barrier(a.gbar,
-                               (unsigned long long)(nb0 + p + 1) * gridDim.x +
-                                   (nb0 == 0 && p == 0 ? (unsigned)a.barrier_skew : 0u),
-                               a.status, abort_f))
-      break;
   }
-  // the fold-matrix load must have landed before the CTA leaves (a CTA without tiles, or one
-  // that gave up, may not have waited for it): a bounded wait that ignores the abort flag
-  if (threadIdx.x == 0) mbar_wait(fbar, 0, a.status);
-  // exit arrival: the last CTA through resets the counter for the next launch
+  // the slice's stores must have ended before the tensor memory is given back (a CTA that gave up
+  // may not have waited for them): a bounded wait that ignores the abort flag
+  if (warp == 0 && tiles) mbar_wait(tbar, 0, a.status);
+  // exit arrival: the last CTA through resets the counters for the next launch
   if (threadIdx.x == 0 && !*abort_f) {
     const unsigned long long seen = atomicAdd(a.gbar, 1ull);
-    if (seen == (nb0 + 4ull) * gridDim.x - 1ull) atomicExch(a.gbar, 0ull);
+    if (seen == gridDim.x - 1ull) {
+      for (int i = 0; i < NTR + 3 * a.R * MB; ++i) ctr_src[16 * i] = 0ull;
+      atomicExch(a.gbar, 0ull);
+    }
+  }
+  tc_fence_before();
+  main_sync();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+}
+
+// ---------------------------------------------------------------- cluster solve
+// The same four products with the operand exchanged inside thread-block clusters where the
+// dependencies allow it.  A phase of the resident solve above spends 1.0 us until its stores are
+// visible, 1.4 us on the dependency counter and 0.6 us on the TMA load of the next operand, against
+// 0.7 us of MMAs and 0.7 us of epilogue.  Here the CTAs that hold one block of 128 kx slots of one
+// right-hand side for every y (product 0: 8 CTAs of 32 data rows at n = 256) form a cluster: product
+// 1 (along y) contracts exactly what the cluster holds, so product 0's epilogue writes the next
+// operand, folded, split and swizzled, straight into the peers' shared memory, and a hardware
+// cluster barrier replaces store, counter and load.  Product 1 -> 2 exchanges between clusters
+// through global memory and the counters; product 2 -> 3 is again within the cluster.
+//
+// A CTA's output slots change between the x products (the cluster's block b) and the y products
+// (block j = rank / TPB), so it needs two slices of the fold matrix.  The x slice lives in tensor
+// memory (filled by four extra warps while the others form the sources): a tcgen05.mma whose A comes
+// from shared memory costs ~90 clocks here whatever its N (4 KB of A at 64 B per clock), one
+// whose A comes from tensor memory ~half.  n = 256 keeps both slices there.
+//
+// MODE 0 (nx, ny <= 128, sine matrices padded to 128, not folded) and MODE 2 (128 x 128, folded): one
+// cluster holds all right-hand sides, sources included, and nothing but the results touches global
+// memory.
+// MODE 1: square folded grids of 256.  (512: eight clusters of 16 CTAs do not fit the GPU at once, and
+// with 8 CTAs of 64 rows the exchange, 64 KB per CTA, takes 4 us: slower than through L2.)
+// BN = 32 data rows per CTA and two data buffers, or (LOCAL, five right-hand sides) 64 and one.
+template <int BN, int MODE> struct Cl {
+  static constexpr bool LOCAL = MODE != 1, FOLD = MODE != 0;
+  // MODE 2's one slot block has odd and even slots: its data rows keep sums and differences side by
+  // side (K = 128) against a fold matrix with zeros in the other half
+  static constexpr int N = LOCAL ? 128 : 256, K = 128, NK = K / BK, MB = N / BM;
+  static constexpr int TPB = BM / BN, CPR = N / BN;        // tiles per slot block, CTAs per right-hand side (and block)
+  static constexpr bool DB = BN == 32;                      // two data buffers
+  static constexpr int STAGE = 2 * BN * 128;                // hi and lo rows of one K block
+  static constexpr int BUF = NK * STAGE;
+  static constexpr int TILE = BM * (BN + 1) * 4;            // staged output tile
+  static constexpr int DATA = 0;
+  static constexpr int DATA_BYTES = (DB ? 2 : 1) * BUF > TILE ? (DB ? 2 : 1) * BUF : (TILE + 127) / 128 * 128;
+  // LOCAL: staged sources, BN rows (shared by R CTAs, rounded up) of R x 128 floats over R CTAs
+  static constexpr int SRC = DATA + DATA_BYTES, SRC_BYTES = LOCAL ? (BN + kMaxRhs - 1) * 512 : 0;
+  static constexpr int BARS = SRC + SRC_BYTES;
+  static constexpr int BYTES = BARS + 128 + 1024;
+  static constexpr uint32_t TX = 128, TY = TX + K;          // tensor-memory columns: accumulator, x slice, y slice
+  // cluster barriers of a launch (each thread arrives at and waits for every one): the start, the
+  // end of each exchange, and where a peer's buffer has to be drained first
+  static constexpr int barriers(int pre) { return 1 + (LOCAL ? (pre ? 1 : 0) + 3 + (DB ? 0 : 3) : 2 + (DB ? 1 : 2)); }
+};
+
+__device__ __forceinline__ void cl_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cl_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_cluster(uint32_t addr, const uint4& v) {
+  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+               : "memory");
+}
+// 8 consecutive columns (col a multiple of 8) of operand row `row` into the data buffer at `buf` of
+// CTA `rank`: 128B-swizzled K blocks, hi rows then lo rows.
+template <int BN> __device__ __forceinline__ void put_operand8(uint32_t buf, uint32_t rank, int row, int col, const float* v) {
+  uint4 h, l;
+  split8(v, h, l);
+  const uint32_t o = (uint32_t)((col >> 6) * (2 * BN * 128) + row * 128 + ((((col & 63) >> 3) ^ (row & 7)) << 4));
+  const uint32_t d = mapa(buf + o, rank);
+  st_cluster(d, h);
+  st_cluster(d + BN * 128, l);
+}
+// LOCAL source phase: the R CTAs of data tile q share its rows (row i of the tile by the CTA of
+// right-hand side i mod R): threads read and evaluate consecutive nodes (all of a batch's reads first),
+// stage them in shared memory S ([rows][R][128] floats) and store eight operand columns at a time into the
+// CTA that multiplies them.
+template <int BN, bool FOLD, typename F, int NR>
+__device__ __forceinline__ void cl_sources(const Geom& gm, const F& f, float* S, int R, int r, int q, uint32_t buf) {
+  constexpr int CPR = 128 / BN, KB = 8;
+  const int rows = (BN - r + R - 1) / R, W = gm.nx, total = rows * W;
+  for (int e0 = threadIdx.x; e0 < total; e0 += KB * kSolveThreads) {
+    typename F::In in[KB];
+    int iy[KB], at[KB];   // node row (-1: none), place in S
+#pragma unroll
+    for (int k = 0; k < KB; ++k) {
+      const int e = e0 + k * kSolveThreads, i = e / W, x = e - i * W, y = q * BN + r + i * R;
+      at[k] = i * R * 128 + x;
+      iy[k] = e < total ? (FOLD ? fold_node(y, 128) : y) : -2;
+      if (iy[k] >= gm.ny) iy[k] = -1;
+      in[k] = iy[k] >= 0 ? f.load(iy[k], x) : typename F::In{};
+    }
+#pragma unroll
+    for (int k = 0; k < KB; ++k) {
+      if (iy[k] == -2) break;
+      const int x = at[k] & 127;
+      float v[NR];
+#pragma unroll
+      for (int i = 0; i < NR; ++i) v[i] = 0.0f;
+      if (iy[k] >= 0) {
+        f.eval(iy[k], x, in[k], v);
+        if constexpr (F::kEffects) f.effects(iy[k], x);
+      }
+#pragma unroll
+      for (int i = 0; i < NR; ++i)
+        if (i < R) S[at[k] + i * 128] = v[i];
+    }
+  }
+  main_sync();
+  constexpr int G = FOLD ? 8 : 16;   // groups of eight folded columns or nodes
+  for (int t = threadIdx.x; t < rows * R * G; t += kSolveThreads) {
+    const int qr = t / G, c = (t - qr * G) * 8, i = qr / R, k = qr - i * R;
+    const float* row = S + qr * 128;
+    const uint32_t rank = (uint32_t)(k * CPR + q);
+    if constexpr (FOLD) {
+      float sum[8], dif[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        int xa, xb;
+        fold_pair(c + u, 128, xa, xb);
+        const float va = row[xa], vb = row[xb];
+        const bool wall = c + u == 32;
+        sum[u] = wall ? vb : va + vb;
+        dif[u] = wall ? 0.0f : va - vb;
+      }
+      put_operand8<BN>(buf, rank, r + i * R, c, sum);
+      put_operand8<BN>(buf, rank, r + i * R, 64 + c, dif);
+    } else {
+      float v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = c + u < W ? row[c + u] : 0.0f;
+      put_operand8<BN>(buf, rank, r + i * R, c, v);
+    }
+  }
+}
+
+// Node of column c (0 .. 127) of slot block b in the last product: the block's first nodes of the
+// pairs in order, then their partners in reverse, so that a tile's columns are (almost) ascending
+// nodes; and its inverse, the column of slot s of the block.
+__device__ __forceinline__ int cl_node(int b, int c, int n) { return fold_node(b * BM + (c < 64 ? 2 * c : 2 * (127 - c) + 1), n); }
+__device__ __forceinline__ int cl_col(int s) { return (s & 1) ? 127 - (s >> 1) : (s >> 1); }
+
+// The solve's result: the tile [128 y slots][BN x columns] staged in shared memory is stored (final
+// mode 2) or mixed into bm (mode 3); consecutive threads take consecutive columns of a row.
+template <int BN, int MODE, bool RES>
+__device__ __forceinline__ void cl_out(const SolveArgs& a, const float* tile, int j, int b, int t, int r) {
+  using C = Cl<BN, MODE>;
+  constexpr int LD = BN + 1, NE = BM * BN, UN = 16;
+  bool bad = false;
+  float d2 = 0.0f, b2 = 0.0f;
+  for (int e0 = threadIdx.x; e0 < NE; e0 += UN * kSolveThreads) {
+    float v[UN], old[UN];
+    int64_t at[UN];
+#pragma unroll
+    for (int k = 0; k < UN; ++k) {
+      const int e = e0 + k * kSolveThreads, row = e / BN, c = e - row * BN;
+      const int y = C::FOLD ? fold_node(j * BM + row, C::N) : row;
+      const int x = C::FOLD ? cl_node(b, t * BN + c, C::N) : t * BN + c;
+      v[k] = tile[row * LD + c];
+      at[k] = (C::FOLD || (y < a.ny && x < a.nx)) ? (int64_t)y * a.nx + x : -1;
+      if (a.final_mode == 3) old[k] = at[k] >= 0 ? a.bm[at[k] * 2 + r] : 0.0f;
+    }
+#pragma unroll
+    for (int k = 0; k < UN; ++k) {
+      if (at[k] < 0) continue;
+      if (a.final_mode == 2) {
+        a.out[(int64_t)r * a.ny * a.nx + at[k]] = v[k];
+        continue;
+      }
+      bad |= !isfinite(v[k]);
+      const float nb = a.w * v[k] + (1.0f - a.w) * old[k];
+      a.bm[at[k] * 2 + r] = nb;
+      if constexpr (RES) {
+        const float d = nb - old[k];
+        d2 += d * d;
+        b2 += nb * nb;
+      }
+    }
+  }
+  if (bad) atomicOr(a.status, DEV_NONFINITE);
+  if constexpr (RES) residual_add_main(a.rsum, (double)d2, (double)b2);
+}
+
+template <int BN, int MODE, bool RES>
+__global__ void __launch_bounds__(kClThreads, 1)
+    k_dst_solve_cl(const __grid_constant__ CUtensorMap x0h, const __grid_constant__ CUtensorMap x0l,
+                   const __grid_constant__ CUtensorMap x1h, const __grid_constant__ CUtensorMap x1l,
+                   const uint4* __restrict__ fxt, const uint4* __restrict__ fyt, const SolveArgs a) {
+  using C = Cl<BN, MODE>;
+  constexpr int N = C::N, K = C::K, NK = C::NK, MB = C::MB, TPB = C::TPB, CPR = C::CPR;
+  constexpr int CH = BN / 2, H = N / 2;
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ int s_abort;
+  const uint32_t raw = smem_u32(smem_raw);
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  uint8_t* basep = smem_raw + (base - raw);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(basep + C::BARS);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + NK + 2);
+  const uint32_t full0 = smem_u32(bars), done = smem_u32(bars + NK), tbar = smem_u32(bars + NK + 1);
+  const uint32_t buf0 = base + C::DATA, buf1 = C::DB ? buf0 + C::BUF : buf0;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  volatile int* abort_f = &s_abort;
+  uint32_t rank;
+  asm("mov.u32 %0, %cluster_ctarank;" : "=r"(rank));
+  // right-hand side r, x slot block b, position q among the CTAs of (r, b), y slot block j, tile t
+  const int q = (int)rank % CPR, j = q / TPB, t = q - j * TPB;
+  const int cl = (int)blockIdx.x / CPR;   // MODE > 0: cluster index (clusters of CPR CTAs)
+  const int r = C::LOCAL ? (int)rank / CPR : cl / MB, b = C::LOCAL ? 0 : cl % MB;
+  const int koffb = !C::LOCAL && b >= MB / 2 ? H : 0;
+  unsigned long long* ctr_src = a.gbar + 16;          // [CPR]
+  unsigned long long* ctr_p = ctr_src + 16 * CPR;     // [R][MB]
+
+  if (threadIdx.x == 0) {
+    for (const CUtensorMap* m : {&x0h, &x0l, &x1h, &x1l}) prefetch_map(m);
+    for (int k = 0; k < NK; ++k) mbar_init(full0 + 8 * k, 1);
+    mbar_init(done, 1);
+    mbar_init(tbar, 128);
+    s_abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)(2 * BN)) : "memory");
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  if (!C::LOCAL && cl >= a.R * MB) {
+    // clusters beyond the products' only form sources (256^2, two right-hand sides: 32 CTAs multiply)
+    if (warp < 8) {
+      solve_sources_any<BN>(a, reinterpret_cast<float*>(basep + C::DATA), ctr_src);
+      if (threadIdx.x == 0) {
+        const unsigned long long seen = atomicAdd(a.gbar, 1ull);
+        if (seen == gridDim.x - 1ull) {
+          for (int i = 0; i < CPR + a.R * MB; ++i) ctr_src[16 * i] = 0ull;
+          atomicExch(a.gbar, 0ull);
+        }
+      }
+      main_sync();
+      if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+    } else if (a.reset_late) {
+      const int first = a.R * MB * CPR;
+      reset_nodes(a, ((int)blockIdx.x - first) * 128 + (int)threadIdx.x - 256, ((int)gridDim.x - first) * 128);
+    }
+    return;
   }
+  cl_arrive();   // barrier 0: every CTA of the cluster runs
+
+  if (warp >= 8) {
+    // the x slice (block b) and the y slice (block j)
+    fill_tmem<K>(fxt, b, tmem + C::TX, warp & 3, lane);
+    fill_tmem<K>(fyt, j, tmem + C::TY, warp & 3, lane);
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    tc_fence_before();
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tbar) : "memory");
+    cl_wait();
+    for (int k = 1; k < C::barriers(a.pre); ++k) {
+      cl_arrive();
+      cl_wait();
+    }
+    return;
+  }
+
+  bool started = false;   // barrier 0 waited for
+  if (a.pre) {
+    if constexpr (C::LOCAL) {
+      cl_wait();
+      started = true;
+      float* S = reinterpret_cast<float*>(basep + C::SRC);
+      if (a.pre == 1) cl_sources<BN, C::FOLD, SrcMain<float>, 3>(a.sm.gm, a.sm, S, a.R, r, q, buf0);
+      else if (a.pre == 2) cl_sources<BN, C::FOLD, SrcBperp<float>, 2>(a.sb.gm, a.sb, S, a.R, r, q, buf0);
+      else cl_sources<BN, C::FOLD, SrcGiven, kMaxRhs>(a.sc.gm, a.sc, S, a.R, r, q, buf0);
+      asm volatile("fence.proxy.async;" ::: "memory");
+      cl_arrive();
+      cl_wait();
+      asm volatile("fence.proxy.async;" ::: "memory");
+    } else {
+      solve_sources_any<BN>(a, reinterpret_cast<float*>(basep + C::DATA), ctr_src);   // staged in the data buffers
+    }
+  }
+  const int row = (warp & 3) * 32 + lane, half = warp >> 2;
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    const bool along_x = (p & 1) == 0;
+    const bool exchange = p < 3 && (C::LOCAL || p != 1);   // the next operand goes to the cluster's peers
+    const uint32_t buf = along_x ? buf0 : buf1;
+    const bool load = p == 0 ? (!C::LOCAL || !a.pre) : (p == 2 && !C::LOCAL);   // the operand comes by TMA
+    if (p == 3) pdl_trigger();
+    if (warp == 0 && lane == 0 && load) {
+      bool ok = true;
+      if (p == 0 && a.pre && !C::LOCAL)
+        ok = dep_wait(ctr_src + 16 * q, (unsigned long long)(BN / kSrcRows) + (unsigned)a.barrier_skew, a.status, abort_f);
+      if (p == 2)
+        ok = dep_wait(ctr_p + 16 * (r * MB + j), (unsigned long long)CPR + (a.pre ? 0u : (unsigned)a.barrier_skew), a.status,
+                      abort_f);
+      const CUtensorMap* mh = p == 0 ? &x0h : &x1h;
+      const CUtensorMap* ml = p == 0 ? &x0l : &x1l;
+      for (int kb = 0; ok && kb < NK; ++kb) {
+        const uint32_t fb = full0 + 8 * kb;
+        mbar_expect_tx(fb, C::STAGE);
+        tma_load_2d(buf + kb * C::STAGE, mh, koffb + kb * BK, r * N + q * BN, fb);
+        tma_load_2d(buf + kb * C::STAGE + BN * 128, ml, koffb + kb * BK, r * N + q * BN, fb);
+      }
+    } else if (warp == 1) {
+      bool ok = true;
+      if (p == 0) ok = mbar_wait_a(tbar, 0, a.status, abort_f);
+      ok = __all_sync(0xffffffffu, ok);
+      for (int kb = 0; ok && kb < NK; ++kb) {
+        if (load) ok = __all_sync(0xffffffffu, mbar_wait_a(full0 + 8 * kb, (uint32_t)(p >> 1), a.status, abort_f));
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t bh = desc_k_sw128(buf + kb * C::STAGE);
+        const uint32_t ta = tmem + (along_x ? C::TX : C::TY) + (uint32_t)(kb * 32);
+        if (elect_one()) {
+#pragma unroll
+          for (int k = 0; k < BK / 16; ++k) {
+            const uint64_t off = (uint64_t)((k * 32) >> 4);
+            mma_bf16_ta(tmem, ta + 8u * k, bh + off, Cfg<BN>::IDESC2, (kb | k) != 0 ? 1u : 0u);
+            mma_bf16_ta(tmem, ta + (uint32_t)(K / 2) + 8u * k, bh + off, Cfg<BN>::IDESC, 1u);
+          }
+        }
+        __syncwarp();
+      }
+      if (elect_one()) mma_commit(done);
+    }
+    __syncwarp();
+    // output slot of this thread's lane and its first data row
+    const int s = (along_x ? b : j) * BM + row;
+    const int i0 = (along_x ? q * BN : b * BM + t * BN) + half * CH;
+    float sc[CH];
+    if (p == 1) {
+      const float4* f4 = reinterpret_cast<const float4*>(a.scale + (int64_t)s * N + i0);
+#pragma unroll
+      for (int k = 0; k < CH / 4; ++k) {
+        const float4 f = __ldg(f4 + k);
+        sc[4 * k] = f.x;
+        sc[4 * k + 1] = f.y;
+        sc[4 * k + 2] = f.z;
+        sc[4 * k + 3] = f.w;
+      }
+    }
+    mbar_wait_a(done, (uint32_t)(p & 1), a.status, abort_f);
+    tc_fence_after();
+    float x[CH];
+    tmem_ld_pair<BN, CH>(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(half * CH), x);
+    tc_fence_before();
+    if (p == 3) {
+      float* tile = reinterpret_cast<float*>(basep + C::DATA);
+      constexpr int LD = BN + 1;
+#pragma unroll
+      for (int k = 0; k < CH; ++k) tile[row * LD + half * CH + k] = x[k];
+      main_sync();
+      if (!*abort_f) cl_out<BN, MODE, RES>(a, tile, j, b, t, r);
+      break;
+    }
+    if (p == 1) {
+#pragma unroll
+      for (int k = 0; k < CH; ++k) x[k] *= sc[k];
+    }
+    if (exchange) {
+      if (!started) {
+        cl_wait();
+        started = true;
+      }
+      // the peers' buffer must be drained of their MMAs: with one buffer those of this product, with
+      // two those of product 1 (whose end this CTA announced below)
+      if (!C::DB) {
+        cl_arrive();
+        cl_wait();
+      } else if (!C::LOCAL && p == 2) {
+        cl_wait();
+      }
+      const uint32_t dst = along_x ? buf1 : buf0;
+      if constexpr (C::FOLD) {
+        const int v0 = i0 >> 1, cs = row;
+        const int col = p == 2 ? cl_col(cs) : cs, tt = col / BN, orow = col - tt * BN;
+        float sum[CH / 2], dif[CH / 2];
+#pragma unroll
+        for (int k = 0; k < CH / 2; ++k) {
+          const bool wall = v0 + k == N / 4;
+          sum[k] = wall ? x[2 * k + 1] : x[2 * k] + x[2 * k + 1];
+          dif[k] = wall ? 0.0f : x[2 * k] - x[2 * k + 1];
+        }
+#pragma unroll
+        for (int c = 0; c < CH / 2; c += 8) {
+          if constexpr (C::LOCAL) {
+            put_operand8<BN>(dst, (uint32_t)(r * CPR + tt), orow, v0 + c, sum + c);
+            put_operand8<BN>(dst, (uint32_t)(r * CPR + tt), orow, H + v0 + c, dif + c);
+          } else {
+            put_operand8<BN>(dst, (uint32_t)tt, orow, v0 + c, sum + c);
+            put_operand8<BN>(dst, (uint32_t)(TPB + tt), orow, v0 + c, dif + c);
+          }
+        }
+      } else {
+        const int tt = row / BN;
+#pragma unroll
+        for (int c = 0; c < CH; c += 8) put_operand8<BN>(dst, (uint32_t)(r * CPR + tt), row - tt * BN, i0 + c, x + c);
+      }
+      asm volatile("fence.proxy.async;" ::: "memory");
+      cl_arrive();
+      cl_wait();
+      asm volatile("fence.proxy.async;" ::: "memory");
+      tc_fence_after();
+    } else {
+      // product 1 of several clusters: through global memory, counted per slot block of y
+      if (C::DB) cl_arrive();   // this CTA's product 1 has read its buffer
+      if (!*abort_f)
+        rs_epilogue<CH>(a, 0, s, s, r, i0, x, sc, reinterpret_cast<__nv_bfloat16*>(a.op_hi[1]),
+                        reinterpret_cast<__nv_bfloat16*>(a.op_lo[1]));
+      asm volatile("fence.proxy.async;" ::: "memory");
+      main_sync();
+      tc_fence_after();
+      if (threadIdx.x == 0 && !*abort_f) dep_arrive(ctr_p + 16 * (r * MB + j));
+    }
+  }
+  if (!C::LOCAL && threadIdx.x == 0 && !*abort_f) {
+    // the last CTA through resets the counters for the next launch
+    const unsigned long long seen = atomicAdd(a.gbar, 1ull);
+    if (seen == gridDim.x - 1ull) {
+      for (int i = 0; i < CPR + a.R * MB; ++i) ctr_src[16 * i] = 0ull;
+      atomicExch(a.gbar, 0ull);
+    }
+  }
+  tc_fence_before();
+  main_sync();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
 }
 
 using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -1145,6 +1745,67 @@ void gemm(const CUtensorMap& ah, const CUtensorMap& al, const CUtensorMap* bh, c
 
 }  // namespace
 
+bool dst_tc_resident(const hq_grid_s* g) {
+  const char* nors = std::getenv("HQ_NO_RS");
+  return !g->fp64 && !g->tf32 && g->fold && g->nx == g->ny && (g->nx == 256 || g->nx == 512) && !(nors && nors[0] == '1');
+}
+
+int dst_tc_cluster_mode(const hq_grid_s* g) {
+  const char* nc = std::getenv("HQ_NO_CLUSTER");
+  const char* nors = std::getenv("HQ_NO_RS");
+  const char* bn = std::getenv("HQ_SOLVE_BN");
+  if (g->fp64 || g->tf32 || (nc && nc[0] == '1') || (nors && nors[0] == '1') || (bn && std::atoi(bn) == 64)) return -1;
+  if (g->nx <= 128 && g->ny <= 128) return g->fault_barrier ? -1 : (g->fold ? 2 : 0);   // (one cluster: no counter to fail)
+  if (!g->fold || g->nx != g->ny) return -1;
+  return g->nx == 256 ? 1 : -1;
+}
+
+namespace {
+template <int BN, int N, bool RES> auto* rs_kernel() { return &k_dst_solve_rs<BN, N, RES>; }
+template <typename K> struct Sized {   // a kernel, its shared memory and where its co-resident CTA count goes
+  K k;
+  int smem;
+  int* ctas;
+};
+template <typename K> Sized(K, int, int*) -> Sized<K>;
+template <int BN, int MODE, bool RES> auto* cl_kernel() { return &k_dst_solve_cl<BN, MODE, RES>; }
+
+// Right-hand sides whose clusters fit the GPU at once (0: none).
+template <int BN, int MODE, bool RES> int cl_capacity(int* most = nullptr) {
+  using C = Cl<BN, MODE>;
+  auto kern = cl_kernel<BN, MODE, RES>();
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::BYTES) != cudaSuccess ||
+      cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  int best = 0;
+  for (int R = 1; R <= kMaxRhs; ++R) {
+    const int cs = C::LOCAL ? R * C::CPR : C::CPR, need = C::LOCAL ? 1 : R * C::MB;
+    if (cs > 16) break;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(cs * need));
+    cfg.blockDim = dim3(kClThreads);
+    cfg.dynamicSmemBytes = C::BYTES;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cs;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      break;
+    }
+    if (most) *most = n;
+    if (n < need) break;
+    best = R;
+  }
+  return best;
+}
+}  // namespace
+
 int dst_tc_init(hq_grid_s* g, std::string& err) {
   void* fn = nullptr;
   cudaDriverEntryPointQueryResult q;
@@ -1159,10 +1820,10 @@ int dst_tc_init(hq_grid_s* g, std::string& err) {
     err = "cannot read the SM count";
     return 1;
   }
-  auto size_solve = [&](auto kern, int smem, int& ctas) {
+  auto size_solve = [&](auto kern, int smem, int& ctas, int threads = kSolveThreads) {
     int per_sm = 0;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSolveThreads, smem) != cudaSuccess || per_sm < 1) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess || per_sm < 1) {
       err = "cannot size the cooperative DST solve";
       return false;
     }
@@ -1184,14 +1845,29 @@ int dst_tc_init(hq_grid_s* g, std::string& err) {
     return 1;
   const char* bn = std::getenv("HQ_SOLVE_BN");
   t.wide_only = bn != nullptr && std::atoi(bn) == 64;
-  const char* nors = std::getenv("HQ_NO_RS");
   // (the resident fold matrix is bf16: as TF32 words it would need 256 KB of shared memory at 512^2)
-  t.rs = !tf && g->fold && g->nx == g->ny && (g->nx == 256 || g->nx == 512) && !(nors && nors[0] == '1');
-  if (t.rs && (!size_solve(k_dst_solve_rs<64, false>, RsSmem<64>::BYTES, t.rs_ctas[0]) ||
-               !size_solve(k_dst_solve_rs<32, false>, RsSmem<32>::BYTES, t.rs_ctas[1]) ||
-               !size_solve(k_dst_solve_rs<64, true>, RsSmem<64>::BYTES, spare) ||
-               !size_solve(k_dst_solve_rs<32, true>, RsSmem<32>::BYTES, spare)))
+  t.rs = dst_tc_resident(g);
+  auto size_rs = [&](auto... kern) { return (size_solve(kern.k, kern.smem, *kern.ctas, kClThreads) && ...); };
+  if (t.rs && !(g->nx == 512 ? size_rs(Sized{rs_kernel<64, 512, false>(), RsSmem<64>::BYTES, &t.rs_ctas[0]},
+                                       Sized{rs_kernel<32, 512, false>(), RsSmem<32>::BYTES, &t.rs_ctas[1]},
+                                       Sized{rs_kernel<64, 512, true>(), RsSmem<64>::BYTES, &spare},
+                                       Sized{rs_kernel<32, 512, true>(), RsSmem<32>::BYTES, &spare})
+                             : size_rs(Sized{rs_kernel<64, 256, false>(), RsSmem<64>::BYTES, &t.rs_ctas[0]},
+                                       Sized{rs_kernel<32, 256, false>(), RsSmem<32>::BYTES, &t.rs_ctas[1]},
+                                       Sized{rs_kernel<64, 256, true>(), RsSmem<64>::BYTES, &spare},
+                                       Sized{rs_kernel<32, 256, true>(), RsSmem<32>::BYTES, &spare})))
     return 1;
+  t.cl_mode = dst_tc_cluster_mode(g);
+  t.cl_rhs[0] = t.cl_rhs[1] = t.cl_max = 0;
+  if (t.cl_mode == 0) {
+    t.cl_rhs[0] = std::min(cl_capacity<32, 0, false>(), cl_capacity<32, 0, true>());
+    t.cl_rhs[1] = cl_capacity<64, 0, false>();
+  } else if (t.cl_mode == 2) {
+    t.cl_rhs[0] = std::min(cl_capacity<32, 2, false>(), cl_capacity<32, 2, true>());
+    t.cl_rhs[1] = cl_capacity<64, 2, false>();
+  } else if (t.cl_mode == 1) {
+    t.cl_rhs[0] = std::min(cl_capacity<32, 1, false>(&t.cl_max), cl_capacity<32, 1, true>());
+  }
   const uint64_t nxp = g->nxp, nyp = g->nyp;
   int bad = 0;
   bad |= make_map(enc, &t.a0_hi, g->op_hi[0], kMaxRhs * nyp, nxp, err, 128, tf);
@@ -1210,10 +1886,8 @@ int dst_tc_init(hq_grid_s* g, std::string& err) {
     if (g->scale_h)
       bad |= make_map_plain(enc, &t.scale_h[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g->scale_h, nyp, nxp, BM, bn, err);
   }
-  if (t.rs) {
-    bad |= make_map(enc, &t.rf_hi, g->sx_hi, nxp, kx, err, 128);
-    bad |= make_map(enc, &t.rf_lo, g->sx_lo, nxp, kx, err, 128);
-    for (int o = 0; o < 2; ++o)
+  if (t.rs || t.cl_mode >= 0) {
+    for (int o = 0; o < (t.rs ? 3 : 2); ++o)
       for (int i = 0; i < 2; ++i) {
         const uint32_t bn = i == 0 ? 64 : 32;
         bad |= make_map(enc, &t.rx_hi[o][i], g->op_hi[o], kMaxRhs * nyp, nxp, err, bn);
@@ -1234,7 +1908,7 @@ namespace {
 // first from the deposit records (pre = 1: psi, Ez, Bz of dep_cur; pre = 2: B_perp).
 void solve_fused(hq_grid_s* g, int R, int final_mode, int last, cudaStream_t s, int pre = 0,
                  const void* dep_cur = nullptr, void* dep_prev = nullptr, void* chi_prev = nullptr,
-                 bool shifted = false) {
+                 bool shifted = false, const float* src = nullptr, float* dst = nullptr) {
   const TensorMaps& t = *g->tmaps;
   SolveArgs a{};
   a.R = R;
@@ -1245,9 +1919,11 @@ void solve_fused(hq_grid_s* g, int R, int final_mode, int last, cudaStream_t s, 
   a.op_lo[0] = g->op_lo[0];
   a.op_hi[1] = g->op_hi[1];
   a.op_lo[1] = g->op_lo[1];
+  a.op_hi[2] = g->op_hi[2];
+  a.op_lo[2] = g->op_lo[2];
   a.scale = reinterpret_cast<const float*>(shifted ? g->scale_h : g->f32_scale);
   a.final_mode = final_mode;
-  a.out = reinterpret_cast<float*>(g->solved);
+  a.out = dst ? dst : reinterpret_cast<float*>(g->solved);
   a.nx = g->nx;
   a.ny = g->ny;
   a.bm = reinterpret_cast<float*>(g->bm);
@@ -1259,6 +1935,53 @@ void solve_fused(hq_grid_s* g, int R, int final_mode, int last, cudaStream_t s, 
   a.pre = pre;
   if (pre == 1) a.sm = src_main_of<float>(g, dep_cur);
   if (pre == 2) a.sb = src_bperp_of<float>(g, dep_cur, dep_prev, chi_prev, last);
+  if (pre == 3) a.sc = SrcGiven{src, g->geom, R};
+  auto late_reset = [&]() {
+    if (pre == 2 && a.sb.reset_prev && a.sb.mode == 2) {
+      a.sb.reset_prev = 0;
+      a.reset_late = 1;
+    }
+  };
+  if (t.cl_mode >= 0 && (R <= t.cl_rhs[0] || (R <= t.cl_rhs[1] && !a.rsum))) {
+    const bool local = t.cl_mode != 1;
+    const int v = R <= t.cl_rhs[0] ? 1 : 0, BNv = v ? 32 : 64, N = local ? 128 : 256;
+    const int cpr = N / BNv, cs = local ? R * cpr : cpr;
+    cudaLaunchConfig_t cfg = {};
+    // (mode 1 with sources: at least a CTA per kSrcRows source rows)
+    const int ctas = local ? cs : std::max(R * (N / BM) * cpr, pre ? std::min(N / kSrcRows, t.cl_max * cs) : 0);
+    cfg.gridDim = dim3((unsigned)ctas);
+    if (t.cl_mode == 1 && ctas > R * (N / BM) * cpr) late_reset();
+    cfg.blockDim = dim3(kClThreads);
+    cfg.stream = s;
+    // cooperative: clusters wait for each other (the single cluster of a local solve does not)
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cs;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeCooperative;
+    at[1].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = local ? 1 : 2;
+    auto go = [&](auto* kern, int smem) {
+      cfg.dynamicSmemBytes = (size_t)smem;
+      cudaLaunchKernelEx(&cfg, kern, t.rx_hi[0][v], t.rx_lo[0][v], t.rx_hi[1][v], t.rx_lo[1][v],
+                         static_cast<const uint4*>(g->fxt), static_cast<const uint4*>(g->fyt), a);
+    };
+    const bool res = a.rsum != nullptr;   // (the B_perp solves, two right-hand sides)
+    if (t.cl_mode == 0) {
+      if (!v) go(cl_kernel<64, 0, false>(), Cl<64, 0>::BYTES);
+      else if (res) go(cl_kernel<32, 0, true>(), Cl<32, 0>::BYTES);
+      else go(cl_kernel<32, 0, false>(), Cl<32, 0>::BYTES);
+    } else if (t.cl_mode == 2) {
+      if (!v) go(cl_kernel<64, 2, false>(), Cl<64, 2>::BYTES);
+      else if (res) go(cl_kernel<32, 2, true>(), Cl<32, 2>::BYTES);
+      else go(cl_kernel<32, 2, false>(), Cl<32, 2>::BYTES);
+    } else {
+      if (res) go(cl_kernel<32, 1, true>(), Cl<32, 1>::BYTES);
+      else go(cl_kernel<32, 1, false>(), Cl<32, 1>::BYTES);
+    }
+    return;
+  }
   if (t.rs) {
     // resident fold-matrix solve: MB slot blocks x (R n / BN) data-row tiles per product; the
     // grid is a multiple of MB (a CTA keeps its slot block)
@@ -1268,8 +1991,9 @@ void solve_fused(hq_grid_s* g, int R, int final_mode, int last, cudaStream_t s, 
     const int v = narrow ? 1 : 0;
     const int tiles_v = MB * (R * n / (narrow ? 32 : 64));
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)std::min(tiles_v, t.rs_ctas[v] / MB * MB));
-    cfg.blockDim = dim3(kSolveThreads);
+    // (at least a CTA per kSrcRows source rows: 256^2, two right-hand sides has 32 tiles)
+    cfg.gridDim = dim3((unsigned)std::min(std::max(tiles_v, pre ? n / kSrcRows : 0), t.rs_ctas[v] / MB * MB));
+    cfg.blockDim = dim3(kClThreads);
     cfg.dynamicSmemBytes = narrow ? RsSmem<32>::BYTES : RsSmem<64>::BYTES;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -1277,9 +2001,14 @@ void solve_fused(hq_grid_s* g, int R, int final_mode, int last, cudaStream_t s, 
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    auto kern = a.rsum ? (narrow ? k_dst_solve_rs<32, true> : k_dst_solve_rs<64, true>)
-                       : (narrow ? k_dst_solve_rs<32, false> : k_dst_solve_rs<64, false>);
-    cudaLaunchKernelEx(&cfg, kern, t.rf_hi, t.rf_lo, t.rx_hi[0][v], t.rx_lo[0][v], t.rx_hi[1][v], t.rx_lo[1][v], a);
+    late_reset();
+    auto pick = [&](auto* w0, auto* w1, auto* n0, auto* n1) { return a.rsum ? (narrow ? n1 : w1) : (narrow ? n0 : w0); };
+    auto* kern = n == 512 ? pick(rs_kernel<64, 512, false>(), rs_kernel<64, 512, true>(), rs_kernel<32, 512, false>(),
+                                 rs_kernel<32, 512, true>())
+                          : pick(rs_kernel<64, 256, false>(), rs_kernel<64, 256, true>(), rs_kernel<32, 256, false>(),
+                                 rs_kernel<32, 256, true>());
+    cudaLaunchKernelEx(&cfg, kern, static_cast<const uint4*>(g->fxt), t.rx_hi[0][v], t.rx_lo[0][v], t.rx_hi[1][v], t.rx_lo[1][v],
+                       t.rx_hi[2][v], t.rx_lo[2][v], a);
     return;
   }
   // tiles of one product (the larger of the x and y products) at N-tile width bn
@@ -1316,6 +2045,11 @@ void dst_solve_tc_bmix(hq_grid_s* g, int last, cudaStream_t s) { solve_fused(g, 
 
 // sources (split) in op[0] -> FP32 solution in g->solved [R][ny][nx]
 void dst_solve_tc(hq_grid_s* g, int R, cudaStream_t s) { solve_fused(g, R, 2, 0, s); }
+// src [R][ny][nx] -> dst (16-byte aligned), both the caller's: read by the source phase, written by
+// the last product
+void dst_solve_tc_given(hq_grid_s* g, int R, const float* src, float* dst, cudaStream_t s) {
+  solve_fused(g, R, 2, 0, s, 3, nullptr, nullptr, nullptr, false, src, dst);
+}
 void dst_solve_tc_shifted(hq_grid_s* g, int R, cudaStream_t s) {
   solve_fused(g, R, 2, 0, s, 0, nullptr, nullptr, nullptr, true);
 }

@@ -54,6 +54,18 @@ def test_poisson_fp64_sizes(hq, nx, ny, nrhs):
     assert err <= 1e-12 and same
 
 
+@pytest.mark.parametrize("precision,nx,ny,nrhs", [("fp32", 8, 8, 1), ("fp32", 96, 80, 5), ("fp32", 128, 128, 2),
+                                                    ("fp32", 256, 256, 1), ("fp32", 256, 256, 5), ("fp32", 256, 384, 2),
+                                                    ("fp32", 512, 512, 1), ("fp32", 512, 512, 4), ("fp32", 512, 512, 5),
+                                                    ("tf32x3", 200, 72, 4), ("tf32x3", 256, 256, 3)])
+def test_poisson_fp32_sizes(hq, precision, nx, ny, nrhs):
+    """FP32 from the caller's sources to the caller's array in one launch: 3e-5 (bf16x3) and 8e-6
+    (TF32x3), the bars of the parity tests of these operand splits."""
+    err, same = solve_case(hq, nx, ny, nrhs, precision)
+    print(f"{precision} {nx}x{ny} x {nrhs}: {err:.1e}")
+    assert err <= (3e-5 if precision == "fp32" else 8e-6) and same
+
+
 @pytest.mark.parametrize("nx,ny", [(48, 40), (128, 64), (64, 130)])
 def test_fp64_sources_in_the_first_pass(hq, monkeypatch, nx, ny):
     """FP64 sweeps with the sources formed by the solve's first pass and the mixing done by its
@@ -75,3 +87,51 @@ def test_fp64_sources_in_the_first_pass(hq, monkeypatch, nx, ny):
         assert float((a - b).abs().max()) <= 1e-9 * float(b.abs().max()), k
     for a, b in zip(outs[0][1], outs[1][1]):
         assert abs(a - b) <= 1e-6 * b + 1e-12
+
+
+@pytest.mark.parametrize("nx,ny", [(72, 48), (128, 128), (256, 256)])
+def test_cluster_solve_matches_without(hq, monkeypatch, nx, ny):
+    """FP32 sweeps whose solves exchange their operands inside thread-block clusters, against
+    HQ_NO_CLUSTER=1 (through global memory).  The operand splits differ where small grids are no
+    longer folded, by the bf16x3 error of a solve (3e-5 is its bar, here of each field's peak)."""
+    g = I.scaled_grid(I.grid_params("linear64"), nx, ny, 16, zeta_min=-1.0, zeta_max=1.0)
+    beam = I.random_beam(20_000, 0.4, 0.4, 0.4, 0.5)
+    outs = []
+    for mode in ("0", "1"):
+        monkeypatch.setenv("HQ_NO_CLUSTER", mode)
+        grid = hq.Grid(dict(g, pc_residuals=1), precision="fp32")
+        out = grid.alloc_out(("ez", "psi", "bx", "by", "bz"))
+        grid.sweep([hq.Beam(beam)], out=out)
+        assert grid.sync() == 0
+        outs.append((out, grid.pc_residuals()))
+        grid.close()
+    for k in outs[0][0]:
+        a, b = outs[0][0][k], outs[1][0][k]
+        dev = float(torch.linalg.norm((a - b).double()) / torch.linalg.norm(b.double()))
+        print(f"{nx}x{ny} {k}: {dev:.1e}")
+        if k != "bz":   # (a small residual of two large terms for a round driver)
+            assert dev <= 3e-5, k
+    for a, b in zip(outs[0][1], outs[1][1]):
+        assert abs(a - b) <= 1e-2 * b + 1e-9
+
+
+@pytest.mark.parametrize("n", [256, 512])
+def test_dependency_wait_times_out(hq, monkeypatch, n):
+    """A dependency counter that never reaches its target (HQ_FAULT_BARRIER=1): the bounded wait
+    runs out, every CTA leaves, hq_sync reports HQ_ERR_TIMEOUT, and another grid solves."""
+    g = dict(nx=n, ny=n, nzeta=2, xmin=-4.0, xmax=4.0, ymin=-4.0, ymax=4.0, zeta_min=0.0, zeta_max=1.0)
+    src = torch.randn(2, n, n, device="cuda", generator=torch.Generator(device="cuda").manual_seed(5))
+    monkeypatch.setenv("HQ_FAULT_BARRIER", "1")
+    bad = hq.Grid(g, precision="fp32")
+    monkeypatch.delenv("HQ_FAULT_BARRIER")
+    bad.poisson_solve(src)
+    with pytest.raises(hq.HQError) as e:
+        bad.sync()
+    assert e.value.status == 5
+    bad.close()
+    good = hq.Grid(g, precision="fp32")
+    got = good.poisson_solve(src)
+    good.sync()
+    for r in range(2):
+        assert rel(got[r], O.poisson_solve(O.GridSpec(**g), src[r].double().cpu())) <= 3e-5
+    good.close()
