@@ -38,8 +38,8 @@
  *                  through the shared memory of a thread-block cluster where they can)
  *   HQ_NO_PDL=1    no programmatic dependent launch between the per-slice kernels
  *   HQ_NO_GRAPH=1  hq_sweep_step issues its launches instead of replaying a CUDA graph
- *   HQ_NO_FORK=1   hq_sweep_step keeps the witness sums and beam deposits on the grid's
- *                  stream instead of beside the final pass on a second stream
+ *   HQ_NO_FORK=1   hq_sweep_step keeps the witness sums, beam pushes and beam deposits on the
+ *                  grid's stream instead of beside the final pass on a second stream
  *   HQ_SEPARATE_SRC=1  the psi/Ez/Bz and B_perp sources are formed by kernels of their own
  *                  ahead of each solve instead of in the solve's first phase or pass (FP64:
  *                  and the B_perp mixing in one of its own behind it)

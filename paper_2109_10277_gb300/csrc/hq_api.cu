@@ -745,12 +745,13 @@ bool aux_ready(hq_grid_t g) {
 hq_status sweep_body(hq_grid_t g, hq_beam_view* beams, int32_t nbeams, double dt, const hq_field_out* out,
                      int32_t witness_beam, double* witness_sums) {
   hq_status st;
-  // Without a beam push, the witness sum of slice i-1 and the beam deposit of slice i do not
-  // depend on slice i's final pass (disjoint buffers, or commutative atomics into the same
-  // records), so from slice 1 on they run on a second stream beside it, forked and joined with
-  // events (a graph capture records the fork as parallel branches).  Slice 0 stays in order
-  // (the beams are binned and the records reset there).
-  const bool fork = dt == 0.0 && !g->prof_on && !g->det && aux_ready(g);
+  // The witness sum and the beam push of slice i-1 and the beam deposit of slice i (whose
+  // particles, those of slices i and i+1, that push does not move) do not depend on slice i's
+  // final pass (disjoint buffers, or commutative atomics into the same records), so from slice 1
+  // on they run on a second stream beside it, forked and joined with events (a graph capture
+  // records the fork as parallel branches).  Slice 0 stays in order (the beams are binned and the
+  // records reset there).
+  const bool fork = !g->prof_on && !g->det && aux_ready(g);
   const bool wit = witness_beam >= 0;
   for (int i = 0; i < g->nz; ++i) {
     if (fork && i > 0) {
@@ -760,6 +761,7 @@ hq_status sweep_body(hq_grid_t g, hq_beam_view* beams, int32_t nbeams, double dt
       cudaStreamWaitEvent(g->aux_stream, g->ev_fork, 0);
       g->stream = g->aux_stream;
       st = wit ? hq_witness_accumulate(g, &beams[witness_beam], i - 1, witness_sums) : HQ_OK;
+      if (st == HQ_OK && dt != 0.0) st = hq_push_beams(g, beams, nbeams, i - 1, dt);
       if (st == HQ_OK) st = hq_beam_deposit(g, beams, nbeams, i);
       cudaEventRecord(g->ev_join, g->aux_stream);
       g->stream = s;
@@ -771,10 +773,9 @@ hq_status sweep_body(hq_grid_t g, hq_beam_view* beams, int32_t nbeams, double dt
     }
     if ((st = hq_solve_fields(g, i)) != HQ_OK) return st;
     if (out && (st = hq_store_fields(g, out, i)) != HQ_OK) return st;
-    // forked sweeps sum slice i's witness beside the next slice's final pass
-    if (wit && !(fork && i + 1 < g->nz) &&
-        (st = hq_witness_accumulate(g, &beams[witness_beam], i, witness_sums)) != HQ_OK)
-      return st;
+    // forked sweeps sum slice i's witness and push its beams beside the next slice's final pass
+    if (fork && i + 1 < g->nz) continue;
+    if (wit && (st = hq_witness_accumulate(g, &beams[witness_beam], i, witness_sums)) != HQ_OK) return st;
     if (dt != 0.0 && (st = hq_push_beams(g, beams, nbeams, i, dt)) != HQ_OK) return st;
   }
   // advance once past the tail so the plasma state matches a completed sweep

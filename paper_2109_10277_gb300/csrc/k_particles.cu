@@ -283,13 +283,22 @@ __device__ __forceinline__ bool state_ok(const Geom& gm, double x, double y, dou
          y < gm.ymax && opp >= guard;
 }
 
+// Plasma particles per cell per axis, with the FP32 and FP64 reciprocals.
+struct PpcInfo {
+  int px, py;
+  int pow2;   // both powers of two: the sub-cell offsets are exact in FP32
+  float finv_x, finv_y;
+  double inv_x, inv_y;
+  double cell_w;   // dx dy / particles per cell
+};
+
 // ---------------------------------------------------------------- init
 // Placement of plasma particle p (Sec. 2: unperturbed plasma ahead of the beams): cell-row-major,
 // ppc_x x ppc_y at sub-cell centres, at rest.  A multi-species grid (MS) places each species'
 // block [off[s], off[s + 1]) with that species' particles per cell, profile and density.
 template <typename T, bool MS>
 __global__ void k_plasma_init(Plasma<T> pl, Geom gm, int ppx, int ppy, const double* prof, int npf,
-                              double rmax, double n0s, SpeciesTab tab) {
+                              double rmax, double n0s, SpeciesTab tab, PpcInfo pc) {
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= pl.n) return;
   int64_t lp = p;
@@ -302,14 +311,21 @@ __global__ void k_plasma_init(Plasma<T> pl, Geom gm, int ppx, int ppy, const dou
     npf = tab.npf[s];
     rmax = tab.rmax[s];
     n0s = tab.n0[s];
+    pc.pow2 = tab.pow2[s];
+    pc.inv_x = tab.inv_px[s];
+    pc.inv_y = tab.inv_py[s];
+    pc.cell_w = gm.dx * gm.dy / (double)(ppx * ppy);
   }
-  const int ppc = ppx * ppy;
-  const int64_t c = lp / ppc;
-  const int sub = (int)(lp - c * ppc);
-  const int ix = (int)(c % gm.nx), iy = (int)(c / gm.nx);
+  const unsigned ppc = (unsigned)(ppx * ppy), l32 = (unsigned)lp;   // (fewer than 2^31 particles)
+  const unsigned c = l32 / ppc;
+  const int sub = (int)(l32 - c * ppc);
+  const int iy = (int)(c / (unsigned)gm.nx), ix = (int)(c - (unsigned)iy * (unsigned)gm.nx);
   const int sx = sub % ppx, sy = sub / ppx;
-  const double x = gm.xmin + ((double)ix + ((double)sx + 0.5) / ppx) * gm.dx;
-  const double y = gm.ymin + ((double)iy + ((double)sy + 0.5) / ppy) * gm.dy;
+  // (particle counts that are powers of two: the reciprocal is exact, and the FP64 pipe, which bounds
+  // this kernel, is spared two divisions of ~10 instructions each)
+  const double ox = (double)sx + 0.5, oy = (double)sy + 0.5;
+  const double x = gm.xmin + ((double)ix + (pc.pow2 ? ox * pc.inv_x : ox / ppx)) * gm.dx;
+  const double y = gm.ymin + ((double)iy + (pc.pow2 ? oy * pc.inv_y : oy / ppy)) * gm.dy;
   double dens = 1.0;
   if (prof) {
     const double r = sqrt(x * x + y * y);
@@ -325,22 +341,18 @@ __global__ void k_plasma_init(Plasma<T> pl, Geom gm, int ppx, int ppy, const dou
   pl.psi[p] = 0.0;
   pl.ux[p] = T(0);
   pl.uy[p] = T(0);
-  pl.w[p] = T(n0s * dens * (gm.dx * gm.dy / (double)ppc));
+  pl.w[p] = T(n0s * dens * pc.cell_w);
   pl.alive[p] = 1;
   if (pl.origin) pl.origin[p] = (int32_t)p;
   for (int k = 0; k < kRing * 5; ++k) pl.hist[(int64_t)k * pl.n + p] = T(0);
   if (pl.hsum)
     for (int c = 0; c < 5; ++c) pl.hsum[(int64_t)c * pl.n + p] = 0.0f;
   if (pl.cell) {
-    int jx, jy;
-    double fx, fy;
-    jx = (int)floor((x - gm.xmin) * gm.inv_dx);
-    jy = (int)floor((y - gm.ymin) * gm.inv_dy);
-    fx = (x - gm.xmin) * gm.inv_dx - jx;
-    fy = (y - gm.ymin) * gm.inv_dy - jy;
-    pl.cell[p] = (jy << 16) | jx;
-    pl.fx[p] = (float)fx;
-    pl.fy[p] = (float)fy;
+    const double ux = (x - gm.xmin) * gm.inv_dx, uy = (y - gm.ymin) * gm.inv_dy;
+    const double jx = floor(ux), jy = floor(uy);
+    pl.cell[p] = ((int)jy << 16) | (int)jx;
+    pl.fx[p] = (float)(ux - jx);
+    pl.fy[p] = (float)(uy - jy);
     pl.opp[p] = 1.0f;
   }
 }
@@ -360,7 +372,13 @@ __global__ void k_deposit_initial(Plasma<T> pl, Geom gm, V4<T>* dep, T* chi, T* 
   const SpC<T> sc = spc_of<T, MS>(tab, s);
   T wx[P + 1], wy[P + 1];
   int ix0, iy0;
-  stencil_f64<P, T>(gm, pl.x[p], pl.y[p], ix0, iy0, wx, wy);
+  if constexpr (sizeof(T) == 4) {   // FP32: the cached cell coordinates (no FP64 work)
+    const int cell = pl.cell[p];
+    ix0 = shape_weights<P, T>(cell & 0xFFFF, pl.fx[p], wx);
+    iy0 = shape_weights<P, T>(cell >> 16, pl.fy[p], wy);
+  } else {
+    stencil_f64<P, T>(gm, pl.x[p], pl.y[p], ix0, iy0, wx, wy);
+  }
   const T qw = charge_density<T>(pl.w[p], gm, sc.q);
   if (rho_ion) {
 #pragma unroll
@@ -571,14 +589,6 @@ __global__ void __launch_bounds__(kThreads) k_trial_lin(TrialCache<T> tc, int64_
 // exact polynomial differences carrying the factor (x - x0); otherwise the two stencils are
 // deposited with opposite signs.  Node coordinates u = (x - x_min) / dx enter split as cell +
 // fraction; only the move u - u0 is formed from the FP64 fractions.
-
-// Plasma particles per cell per axis, with the FP32 and FP64 reciprocals.
-struct PpcInfo {
-  int px, py;
-  int pow2;   // both powers of two: the sub-cell offsets are exact in FP32
-  float finv_x, finv_y;
-  double inv_x, inv_y;
-};
 
 // Start (ion) node coordinate of plasma particle p, split as cell + fraction: u0 = cx + fx,
 // v0 = cy + fy (the placement of k_plasma_init: 32-bit index arithmetic, the sub-cell offset
@@ -954,6 +964,19 @@ template <> Plasma<float> plasma_of<float>(const hq_grid_s* g) { return g->p32; 
 
 inline unsigned blocks_for(int64_t n) { return (unsigned)((n + kThreads - 1) / kThreads); }
 
+PpcInfo ppc_of(const hq_grid_s* g) {
+  PpcInfo pc;
+  pc.px = g->d.ppc_x;
+  pc.py = g->d.ppc_y;
+  pc.pow2 = (pc.px & (pc.px - 1)) == 0 && (pc.py & (pc.py - 1)) == 0;
+  pc.inv_x = 1.0 / pc.px;
+  pc.inv_y = 1.0 / pc.py;
+  pc.finv_x = (float)pc.inv_x;
+  pc.finv_y = (float)pc.inv_y;
+  pc.cell_w = g->geom.dx * g->geom.dy / (double)(pc.px * pc.py);
+  return pc;
+}
+
 }  // namespace
 
 // Shape-order and species dispatch of the particle kernels: the default electron plasma runs
@@ -975,11 +998,11 @@ void launch_plasma_init(const hq_grid_s* g, cudaStream_t s) {
   const double* prof = g->profile.empty() ? nullptr : g->d_profile;
   if (g->multi)
     k_plasma_init<T, true><<<blocks_for(g->np), kThreads, 0, s>>>(plasma_of<T>(g), g->geom, 1, 1, nullptr, 0, 0.0,
-                                                                   0.0, g->sp);
+                                                                   0.0, g->sp, PpcInfo{});
   else
     k_plasma_init<T, false><<<blocks_for(g->np), kThreads, 0, s>>>(
         plasma_of<T>(g), g->geom, g->d.ppc_x, g->d.ppc_y, prof, (int)g->profile.size(), g->d.profile_rmax,
-        g->d.n0_scale, g->sp);
+        g->d.n0_scale, g->sp, ppc_of(g));
 }
 
 template <typename T>
@@ -1040,14 +1063,7 @@ void launch_final_pass(const hq_grid_s* g, int slice, void* dep, void* chi, bool
       return;
     }
   float* ps = psrc_of(g, dep);
-  PpcInfo pc;
-  pc.px = g->d.ppc_x;
-  pc.py = g->d.ppc_y;
-  pc.pow2 = (pc.px & (pc.px - 1)) == 0 && (pc.py & (pc.py - 1)) == 0;
-  pc.inv_x = 1.0 / pc.px;
-  pc.inv_y = 1.0 / pc.py;
-  pc.finv_x = (float)pc.inv_x;
-  pc.finv_y = (float)pc.inv_y;
+  const PpcInfo pc = ppc_of(g);
   HQ_PDISPATCH(g->d.shape_order, g->multi,
                (f4 && C ? launch_pdl(k_final_pass<P, T, C, M, C ? 2 : 0>, nb, kThreads, 0, s, plasma_of<T>(g), g->geom,
                                      gf, bm, d, c, ps, pc, slice, gd, rm, g->sp)
