@@ -44,6 +44,8 @@ struct TensorMaps {
   // fused solve, per N-tile width ([0]: 64, [1]: 32): S_x [nxp][nxp], or the fold matrix
   // [nxp][nxp/2], in boxes of BN rows; the FP32 scale [nyp][nxp] in 128 (x) by BN (y) boxes
   CUtensorMap bx_hi[2], bx_lo[2];
+  CUtensorMap fx_hi, fx_lo, fy_hi, fy_lo;   // the same matrices in 128-row boxes (wide solve)
+  int wide_ctas;                            // its co-resident CTAs
   CUtensorMap by_hi[2], by_lo[2];
   CUtensorMap scale[2];
   CUtensorMap scale_h[2];     // the shifted (Helmholtz) spectral factors, same boxes (explicit solver)
@@ -363,6 +365,8 @@ __global__ void __launch_bounds__(128, 1)
 // 128-byte K block per stage, 4-stage ring), warp 1 lane 0 the MMAs (two per K step:
 // A_hi x [B_hi; B_lo] with N = 2 BN, A_lo x B_hi with N = BN, into a 2 BN-column TMEM
 // accumulator), and all 8 warps the epilogue, each warpgroup half of the columns.
+constexpr int kSolveThreads = 256;
+
 // The caller's sources [nr][ny][nx] (hq_poisson_solve); row and column 0 read zero.
 struct SrcGiven {
   static constexpr int NR = kMaxRhs;
@@ -420,6 +424,41 @@ __device__ __forceinline__ void reset_nodes(const SolveArgs& a, int me, int coun
   for (int o = me; o < nn; o += count) a.sb.reset(o);
 }
 
+// bf16 hi/lo split of 8 values packed for two 16-byte stores.
+__device__ __forceinline__ void split8(const float* v, uint4& hi, uint4& lo) {
+  uint32_t h[4], l[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const __nv_bfloat16 h0 = __float2bfloat16_rn(v[2 * k]), h1 = __float2bfloat16_rn(v[2 * k + 1]);
+    const __nv_bfloat16 l0 = __float2bfloat16_rn(v[2 * k] - __bfloat162float(h0));
+    const __nv_bfloat16 l1 = __float2bfloat16_rn(v[2 * k + 1] - __bfloat162float(h1));
+    h[k] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+    l[k] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+  }
+  hi = make_uint4(h[0], h[1], h[2], h[3]);
+  lo = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
+// Eight consecutive operand elements, split.
+__device__ __forceinline__ void put_run8(__nv_bfloat16* hi, __nv_bfloat16* lo, const float* v) {
+  uint4 h, l;
+  split8(v, h, l);
+  *reinterpret_cast<uint4*>(hi) = h;
+  *reinterpret_cast<uint4*>(lo) = l;
+}
+__device__ __forceinline__ void put_run8(float* hi, float* lo, const float* v) {
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    float h[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) h[k] = round_tf32(v[4 * q + k]);
+    reinterpret_cast<float4*>(hi)[q] = make_float4(h[0], h[1], h[2], h[3]);
+    reinterpret_cast<float4*>(lo)[q] = make_float4(v[4 * q] - h[0], v[4 * q + 1] - h[1], v[4 * q + 2] - h[2], v[4 * q + 3] - h[3]);
+  }
+}
+
+__device__ __forceinline__ void main_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }   // warps 0-7
+
 // Source phase: every thread of the launch takes (row, column) items of the operand writer
 // in turn (consecutive threads along a row), KB items at a time: all their reads are issued
 // before any write, then the sources are evaluated, split into op[0] and the functor's own
@@ -430,8 +469,8 @@ __device__ __forceinline__ void solve_sources(const Geom& gm, const Sink& sink, 
   constexpr int NN = Sink::kFold ? 2 : 1;   // nodes per item
   const int w = visit_width<Sink>(gm);
   const int total = w * gm.ny;
-  const int stride = gridDim.x * blockDim.x;
-  for (int t0 = blockIdx.x * blockDim.x + threadIdx.x; t0 < total; t0 += KB * stride) {
+  const int stride = gridDim.x * kSolveThreads;   // (the first 256 threads of every block)
+  for (int t0 = blockIdx.x * kSolveThreads + threadIdx.x; t0 < total; t0 += KB * stride) {
     int iy[KB][NN], ix[KB][NN];
     typename F::In in[KB][NN];
 #pragma unroll
@@ -468,6 +507,24 @@ __device__ __forceinline__ void solve_sources(const Geom& gm, const Sink& sink, 
     }
   }
 }
+// The sources a launch asks for.
+template <typename E> __device__ __forceinline__ void solve_sources_all(const SolveArgs& a) {
+  const Geom& gm = a.pre == 1 ? a.sm.gm : (a.pre == 2 ? a.sb.gm : a.sc.gm);
+  E* hi = reinterpret_cast<E*>(a.op_hi[0]);
+  E* lo = reinterpret_cast<E*>(a.op_lo[0]);
+  if (a.fold) {
+    const SinkFold<E> sink{hi, lo, a.nx, a.ny};
+    if (a.pre == 1) solve_sources<SinkFold<E>, SrcMain<float>, 3>(gm, sink, a.sm);
+    else if (a.pre == 2) solve_sources<SinkFold<E>, SrcBperp<float>, 2>(gm, sink, a.sb);
+    else solve_sources<SinkFold<E>, SrcGiven, kMaxRhs>(gm, sink, a.sc, a.R);
+  } else {
+    const SinkSplit<E> sink{hi, lo, a.nxp, a.nyp};
+    if (a.pre == 1) solve_sources<SinkSplit<E>, SrcMain<float>, 3>(gm, sink, a.sm);
+    else if (a.pre == 2) solve_sources<SinkSplit<E>, SrcBperp<float>, 2>(gm, sink, a.sb);
+    else solve_sources<SinkSplit<E>, SrcGiven, kMaxRhs>(gm, sink, a.sc, a.R);
+  }
+}
+
 // Bounded mbarrier wait that also gives up once another thread of the CTA has.
 __device__ __forceinline__ bool mbar_wait_a(uint32_t bar, uint32_t parity, int* status, volatile int* abort_f) {
   const long long t0 = clock64();
@@ -537,7 +594,7 @@ __device__ __forceinline__ bool dep_wait(const unsigned long long* c, unsigned l
       return false;
     }
   }
-  asm volatile("fence.proxy.async;" ::: "memory");
+  asm volatile("fence.proxy.async.global;" ::: "memory");
   return true;
 }
 
@@ -549,10 +606,9 @@ __device__ __forceinline__ bool elect_one() {
   return p != 0;
 }
 
-// The fused solve runs 256 threads per CTA (warps 0, 1: TMA producer, MMA issuer; all 8
+// The streamed solve runs 256 threads per CTA (warps 0, 1: TMA producer, MMA issuer; all 8
 // warps: epilogue) on N tiles 64 wide, or 32 wide when that still gives every tile its own
 // CTA (twice the tiles, so more of the SMs take part in each product).
-constexpr int kSolveThreads = 256;
 
 // Shared memory of the solve: the stage ring, the FP32 scale tile of phase 1
 // ([BN n][128 rows]), then the barriers (full, empty, done, scale) and the TMEM slot.
@@ -634,20 +690,7 @@ __global__ void __launch_bounds__(kSolveThreads, 1)
   const unsigned nb0 = a.pre ? 1u : 0u;   // barriers before phase 0
   bool go = true;
   if (a.pre) {
-    const Geom& gm = a.pre == 1 ? a.sm.gm : (a.pre == 2 ? a.sb.gm : a.sc.gm);
-    E* hi0 = reinterpret_cast<E*>(a.op_hi[0]);
-    E* lo0 = reinterpret_cast<E*>(a.op_lo[0]);
-    if (a.fold) {
-      const SinkFold<E> sink{hi0, lo0, a.nx, a.ny};
-      if (a.pre == 1) solve_sources<SinkFold<E>, SrcMain<float>, 3>(gm, sink, a.sm);
-      else if (a.pre == 2) solve_sources<SinkFold<E>, SrcBperp<float>, 2>(gm, sink, a.sb);
-      else solve_sources<SinkFold<E>, SrcGiven, kMaxRhs>(gm, sink, a.sc, a.R);
-    } else {
-      const SinkSplit<E> sink{hi0, lo0, a.nxp, a.nyp};
-      if (a.pre == 1) solve_sources<SinkSplit<E>, SrcMain<float>, 3>(gm, sink, a.sm);
-      else if (a.pre == 2) solve_sources<SinkSplit<E>, SrcBperp<float>, 2>(gm, sink, a.sb);
-      else solve_sources<SinkSplit<E>, SrcGiven, kMaxRhs>(gm, sink, a.sc, a.R);
-    }
+    solve_sources_all<E>(a);
     go = grid_barrier(a.gbar, (unsigned long long)gridDim.x + (unsigned)a.barrier_skew, a.status, abort_f);
   }
   for (int p = 0; p < 4 && go; ++p) {
@@ -822,7 +865,6 @@ __global__ void __launch_bounds__(kSolveThreads, 1)
 // Threads of the resident and cluster solves: warps 0-7 as in the streamed solve, 8-11 fill tensor
 // memory while the others form the sources.
 constexpr int kClThreads = 384;
-__device__ __forceinline__ void main_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }   // warps 0-7
 __device__ __forceinline__ void mma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t b, uint32_t idesc, uint32_t accum) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
@@ -904,21 +946,6 @@ template <int BN> struct RsSmem {
   static constexpr int BYTES = BARS + 256 + 1024 /*alignment*/;
   static constexpr uint32_t TX = 128;                       // tensor-memory columns: accumulator (2 BN), F slice
 };
-
-// bf16 hi/lo split of 8 values packed for two 16-byte stores.
-__device__ __forceinline__ void split8(const float* v, uint4& hi, uint4& lo) {
-  uint32_t h[4], l[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const __nv_bfloat16 h0 = __float2bfloat16_rn(v[2 * k]), h1 = __float2bfloat16_rn(v[2 * k + 1]);
-    const __nv_bfloat16 l0 = __float2bfloat16_rn(v[2 * k] - __bfloat162float(h0));
-    const __nv_bfloat16 l1 = __float2bfloat16_rn(v[2 * k + 1] - __bfloat162float(h1));
-    h[k] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-    l[k] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
-  }
-  hi = make_uint4(h[0], h[1], h[2], h[3]);
-  lo = make_uint4(l[0], l[1], l[2], l[3]);
-}
 
 // Epilogue of one thread's CH consecutive columns (data rows i0 .. i0 + CH - 1 of rhs r) of
 // output slot s.  Modes 0/1 (1: times the 1/lambda factors sc) fold adjacent column pairs into
@@ -1242,7 +1269,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
       }
       kb_run += nk;
       ++tiles_run;
-      if (p < 3) asm volatile("fence.proxy.async;" ::: "memory");
+      if (p < 3) asm volatile("fence.proxy.async.global;" ::: "memory");
       tc_fence_before();
       main_sync();
       tc_fence_after();
@@ -1534,10 +1561,10 @@ __global__ void __launch_bounds__(kClThreads, 1)
       if (a.pre == 1) cl_sources<BN, C::FOLD, SrcMain<float>, 3>(a.sm.gm, a.sm, S, a.R, r, q, buf0);
       else if (a.pre == 2) cl_sources<BN, C::FOLD, SrcBperp<float>, 2>(a.sb.gm, a.sb, S, a.R, r, q, buf0);
       else cl_sources<BN, C::FOLD, SrcGiven, kMaxRhs>(a.sc.gm, a.sc, S, a.R, r, q, buf0);
-      asm volatile("fence.proxy.async;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cluster;" ::: "memory");
       cl_arrive();
       cl_wait();
-      asm volatile("fence.proxy.async;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cluster;" ::: "memory");
     } else {
       solve_sources_any<BN>(a, reinterpret_cast<float*>(basep + C::DATA), ctr_src);   // staged in the data buffers
     }
@@ -1660,10 +1687,10 @@ __global__ void __launch_bounds__(kClThreads, 1)
 #pragma unroll
         for (int c = 0; c < CH; c += 8) put_operand8<BN>(dst, (uint32_t)(r * CPR + tt), row - tt * BN, i0 + c, x + c);
       }
-      asm volatile("fence.proxy.async;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cluster;" ::: "memory");
       cl_arrive();
       cl_wait();
-      asm volatile("fence.proxy.async;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cluster;" ::: "memory");
       tc_fence_after();
     } else {
       // product 1 of several clusters: through global memory, counted per slot block of y
@@ -1671,7 +1698,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
       if (!*abort_f)
         rs_epilogue<CH>(a, 0, s, s, r, i0, x, sc, reinterpret_cast<__nv_bfloat16*>(a.op_hi[1]),
                         reinterpret_cast<__nv_bfloat16*>(a.op_lo[1]));
-      asm volatile("fence.proxy.async;" ::: "memory");
+      asm volatile("fence.proxy.async.global;" ::: "memory");
       main_sync();
       tc_fence_after();
       if (threadIdx.x == 0 && !*abort_f) dep_arrive(ctr_p + 16 * (r * MB + j));
@@ -1687,6 +1714,283 @@ __global__ void __launch_bounds__(kClThreads, 1)
   }
   tc_fence_before();
   main_sync();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+}
+
+// ---------------------------------------------------------------- wide solve
+// The same four products for grids with more than three 128 x 64 tiles per SM (1536^2 with two
+// right-hand sides): 128 x 128 tiles with the roles of the resident solve (A = 128 slots of the
+// fold or sine matrix, B = [X_hi; X_lo] of 128 data rows, N = 256, then A_lo x X_hi with N = 128),
+// both streamed.  Here the products themselves cost something (206 GFLOP at 2048^2, two right-hand
+// sides: 109 us at the measured bf16 rate; a K step reads 20 KB of operands from shared memory, which
+// bounds it at ~340 clocks against 192 of tensor-core work), so loads, MMAs and epilogues run in warps of their own: two
+// accumulators in tensor memory let a tile's epilogue run beside the next one's MMAs, and only the
+// TMA producer waits for the other CTAs between products.
+// Warps 0-7: sources and epilogues; warp 8: TMA producer (3-stage ring of A_hi, A_lo, X_hi, X_lo K
+// blocks, 64 KB); warp 9: MMA issuer.
+constexpr int kWideThreads = 320;
+template <typename E> struct Wide {
+  static constexpr int BN = 128, STAGES = 3, STAGE_BYTES = 4 * A_BYTES;
+  static constexpr int TILE = STAGES * STAGE_BYTES, LD = 65;   // the mixing's staged columns, 128 x 64
+  static constexpr int BARS = TILE + BM * LD * 4;
+  static constexpr int BYTES = BARS + 256 + 1024;
+};
+
+// 32 consecutive data columns i0 .. of slot s into the next operand's row: ns slots, nd data rows per
+// right-hand side; folded, adjacent columns are a pair (see rs_epilogue).
+template <typename E>
+__device__ __forceinline__ void wide_store(E* oh, E* ol, int fold, int r, int orow, int i0, int ns, int nd, const float* x) {
+  const int64_t base = ((int64_t)r * ns + orow) * nd;
+  if (fold) {
+    const int v0 = i0 >> 1, H = nd / 2;
+    float sum[16], dif[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const bool wall = v0 + k == nd / 4;
+      sum[k] = wall ? x[2 * k + 1] : x[2 * k] + x[2 * k + 1];
+      dif[k] = wall ? 0.0f : x[2 * k] - x[2 * k + 1];
+    }
+#pragma unroll
+    for (int k = 0; k < 16; k += 8) {
+      put_run8(oh + base + v0 + k, ol + base + v0 + k, sum + k);
+      put_run8(oh + base + H + v0 + k, ol + base + H + v0 + k, dif + k);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 32; k += 8) put_run8(oh + base + i0 + k, ol + base + i0 + k, x + k);
+  }
+}
+
+template <bool RES, typename E>
+__global__ void __launch_bounds__(kWideThreads, 1)
+    k_dst_solve_wide(const __grid_constant__ CUtensorMap fxh, const __grid_constant__ CUtensorMap fxl,
+                     const __grid_constant__ CUtensorMap fyh, const __grid_constant__ CUtensorMap fyl,
+                     const __grid_constant__ CUtensorMap x0h, const __grid_constant__ CUtensorMap x0l,
+                     const __grid_constant__ CUtensorMap x1h, const __grid_constant__ CUtensorMap x1l, const SolveArgs a) {
+  using W = Wide<E>;
+  using C = Cfg<W::BN, E>;
+  constexpr int BN = W::BN, STAGES = W::STAGES, KE = kb_elems<E>();
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ int s_abort;
+  const uint32_t raw = smem_u32(smem_raw);
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  uint8_t* basep = smem_raw + (base - raw);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(basep + W::BARS);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 5);
+  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES), tfull0 = smem_u32(bars + 2 * STAGES),
+                 tempty0 = smem_u32(bars + 2 * STAGES + 2), drain = smem_u32(bars + 2 * STAGES + 4);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  volatile int* abort_f = &s_abort;
+  if (threadIdx.x == 0) {
+    for (const CUtensorMap* m : {&fxh, &fxl, &fyh, &fyl, &x0h, &x0l, &x1h, &x1l}) prefetch_map(m);
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(full0 + 8 * s, 1);
+      mbar_init(empty0 + 8 * s, 1);
+    }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(tfull0 + 8 * s, 1);
+      mbar_init(tempty0 + 8 * s, kSolveThreads);
+    }
+    mbar_init(drain, 1);
+    s_abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const unsigned nb0 = a.pre ? 1u : 0u;   // barriers before the first product
+  // product p: slots and data rows per right-hand side, tiles (slot block fastest), K blocks
+  struct Geo {
+    int ns, nd, mt, tiles, nk;
+  };
+  auto geo = [&](int p) {
+    Geo g;
+    const bool ax = (p & 1) == 0;
+    g.ns = ax ? a.nxp : a.nyp;
+    g.nd = ax ? a.nyp : a.nxp;
+    g.mt = g.ns / BM;
+    g.tiles = g.mt * (a.R * g.nd / BN);
+    g.nk = (a.fold ? g.ns / 2 : g.ns) / KE;
+    return g;
+  };
+
+  if (warp == 8) {
+    if (lane == 0) {
+      uint32_t it = 0;
+      bool ok = true;
+      for (int p = 0; p < 4 && ok; ++p) {
+        const Geo g = geo(p);
+        const CUtensorMap *fh = p & 1 ? &fyh : &fxh, *fl = p & 1 ? &fyl : &fxl, *xh = p & 1 ? &x1h : &x0h, *xl = p & 1 ? &x1l : &x0l;
+        const unsigned nbar = nb0 + (unsigned)p;   // barriers to pass
+        if (nbar > 0) ok = dep_wait(a.gbar, (unsigned long long)nbar * gridDim.x + (nbar == 1 ? (unsigned)a.barrier_skew : 0u),
+                                    a.status, abort_f);
+        for (int tile = blockIdx.x; ok && tile < g.tiles; tile += gridDim.x) {
+          const int s0 = (tile % g.mt) * BM, c0 = (tile / g.mt) * BN;
+          const int koff = (a.fold && s0 >= g.ns / 2) ? g.ns / 2 : 0;
+          for (int kb = 0; kb < g.nk; ++kb, ++it) {
+            const uint32_t s = it % STAGES, st = base + s * W::STAGE_BYTES, fb = full0 + 8 * s;
+            if (it >= (uint32_t)STAGES && !mbar_wait_a(empty0 + 8 * s, ((it / STAGES) - 1) & 1, a.status, abort_f)) {
+              ok = false;
+              break;
+            }
+            mbar_expect_tx(fb, W::STAGE_BYTES);
+            tma_load_2d(st, fh, kb * KE, s0, fb);
+            tma_load_2d(st + A_BYTES, fl, kb * KE, s0, fb);
+            tma_load_2d(st + 2 * A_BYTES, xh, koff + kb * KE, c0, fb);
+            tma_load_2d(st + 3 * A_BYTES, xl, koff + kb * KE, c0, fb);
+          }
+        }
+      }
+      // every load has landed before the CTA may leave
+      for (uint32_t k = it > (uint32_t)STAGES ? it - STAGES : 0; k < it; ++k)
+        mbar_wait(full0 + 8 * (k % STAGES), (k / STAGES) & 1, a.status);
+    }
+  } else if (warp == 9) {
+    uint32_t it = 0, t = 0;
+    bool ok = true;
+    for (int p = 0; p < 4 && ok; ++p) {
+      const Geo g = geo(p);
+      for (int tile = blockIdx.x; ok && tile < g.tiles; tile += gridDim.x, ++t) {
+        const uint32_t acc = t & 1, d = tmem + acc * (2 * BN);
+        if (t >= 2) ok = __all_sync(0xffffffffu, mbar_wait_a(tempty0 + 8 * acc, ((t >> 1) - 1) & 1, a.status, abort_f));
+        tc_fence_after();
+        for (int kb = 0; ok && kb < g.nk; ++kb, ++it) {
+          const uint32_t s = it % STAGES;
+          ok = __all_sync(0xffffffffu, mbar_wait_a(full0 + 8 * s, (it / STAGES) & 1, a.status, abort_f));
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t st = base + s * W::STAGE_BYTES;
+          const uint64_t ah = desc_k_sw128(st), al = desc_k_sw128(st + A_BYTES), bh = desc_k_sw128(st + 2 * A_BYTES);
+          if (elect_one()) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const uint64_t off = (uint64_t)((k * 32) >> 4);
+              mma_op<E>(d, ah + off, bh + off, C::IDESC2, (kb | k) != 0 ? 1u : 0u);
+              mma_op<E>(d, al + off, bh + off, C::IDESC, 1u);
+            }
+            mma_commit(empty0 + 8 * s);
+          }
+          __syncwarp();
+        }
+        if (elect_one()) mma_commit(tfull0 + 8 * acc);
+        __syncwarp();
+      }
+    }
+    if (elect_one()) mma_commit(drain);
+    __syncwarp();
+    mbar_wait(drain, 0, a.status);
+  } else {
+    if (a.pre) {
+      solve_sources_all<E>(a);
+      asm volatile("fence.proxy.async.global;" ::: "memory");
+      main_sync();
+      if (threadIdx.x == 0) dep_arrive(a.gbar);
+    }
+    float* tilebuf = reinterpret_cast<float*>(basep + W::TILE);
+    const int row = (warp & 3) * 32 + lane, half = warp >> 2;
+    const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    uint32_t t = 0;
+    float d2 = 0.0f, b2 = 0.0f;
+    bool bad = false;
+    // (after an abort the phases run through on waits that fail at once: the named barriers stay
+    // matched, nothing is reported or stored as a result)
+    for (int p = 0; p < 4; ++p) {
+      const Geo g = geo(p);
+      const int mode = p == 3 ? a.final_mode : (p == 1 ? 1 : 0);
+      if (p == 3) pdl_trigger();
+      E* oh = reinterpret_cast<E*>(a.op_hi[(p + 1) & 1]);
+      E* ol = reinterpret_cast<E*>(a.op_lo[(p + 1) & 1]);
+      for (int tile = blockIdx.x; tile < g.tiles; tile += gridDim.x, ++t) {
+        const int s0 = (tile % g.mt) * BM, c0 = (tile / g.mt) * BN, r = c0 / g.nd, i00 = c0 - r * g.nd;
+        const uint32_t acc = t & 1;
+        const int s = s0 + row;
+        mbar_wait_a(tfull0 + 8 * acc, (t >> 1) & 1, a.status, abort_f);
+        tc_fence_after();
+#pragma unroll 1
+        for (int q = 0; q < 2; ++q) {
+          const int cc = half * 64 + q * 32, i0 = i00 + cc;
+          float x[32];
+          tmem_ld_pair<BN, 32>(tl + acc * (2 * BN) + (uint32_t)cc, x);
+          if (q == 1) {
+            // both chunks of this thread are out of the accumulator
+            tc_fence_before();
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty0 + 8 * acc) : "memory");
+          }
+          if (mode <= 1) {
+            if (mode == 1) {   // [nyp][nxp]: this slot's row of the factors
+              const float4* sc = reinterpret_cast<const float4*>(a.scale + (int64_t)s * a.nxp + i0);
+#pragma unroll
+              for (int k = 0; k < 8; ++k) {
+                const float4 f = __ldg(sc + k);
+                x[4 * k] *= f.x;
+                x[4 * k + 1] *= f.y;
+                x[4 * k + 2] *= f.z;
+                x[4 * k + 3] *= f.w;
+              }
+            }
+            // the third product's rows in node order: the last one's columns are consecutive x nodes
+            const int orow = p == 2 && a.fold ? fold_node(s, g.ns) : s;
+            wide_store<E>(oh, ol, a.fold, r, orow, i0, g.ns, g.nd, x);
+            continue;
+          }
+          // result: staged, so that consecutive threads take consecutive nodes of a row
+#pragma unroll
+          for (int k = 0; k < 32; ++k) tilebuf[row * W::LD + half * 32 + k] = x[k];
+          main_sync();
+          constexpr int UN = 16;
+          for (int e0 = threadIdx.x; e0 < BM * 64; e0 += UN * kSolveThreads) {
+            float v[UN], old[UN];
+            int64_t at[UN];
+#pragma unroll
+            for (int k = 0; k < UN; ++k) {
+              const int e = e0 + k * kSolveThreads, rr = e >> 6, jj = e & 63;
+              const int y = a.fold ? fold_node(s0 + rr, a.ny) : s0 + rr, xx = i00 + (jj >> 5) * 64 + q * 32 + (jj & 31);
+              v[k] = tilebuf[rr * W::LD + jj];
+              at[k] = (y < a.ny && xx < a.nx && !*abort_f) ? (int64_t)y * a.nx + xx : -1;
+              if (mode == 3) old[k] = at[k] >= 0 ? a.bm[at[k] * 2 + r] : 0.0f;
+            }
+#pragma unroll
+            for (int k = 0; k < UN; ++k) {
+              if (at[k] < 0) continue;
+              if (mode == 2) {
+                a.out[(int64_t)r * a.ny * a.nx + at[k]] = v[k];
+                continue;
+              }
+              bad |= !isfinite(v[k]);
+              const float nb = a.w * v[k] + (1.0f - a.w) * old[k];
+              a.bm[at[k] * 2 + r] = nb;
+              if constexpr (RES) {
+                const float d = nb - old[k];
+                d2 += d * d;
+                b2 += nb * nb;
+              }
+            }
+          }
+          main_sync();
+        }
+      }
+      if (p < 3) {
+        asm volatile("fence.proxy.async.global;" ::: "memory");
+        main_sync();
+        if (threadIdx.x == 0 && !*abort_f) dep_arrive(a.gbar);
+      }
+    }
+    if (bad) atomicOr(a.status, DEV_NONFINITE);
+    if constexpr (RES) residual_add_main(a.rsum, (double)d2, (double)b2);
+  }
+  tc_fence_before();
+  __syncthreads();
+  // exit arrival: the last CTA through resets the counter for the next launch
+  if (threadIdx.x == 0 && !*abort_f) {
+    const unsigned long long seen = atomicAdd(a.gbar, 1ull);
+    if (seen == (nb0 + 4ull) * gridDim.x - 1ull) atomicExch(a.gbar, 0ull);
+  }
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
 }
 
@@ -1843,6 +2147,11 @@ int dst_tc_init(hq_grid_s* g, std::string& err) {
             !size_solve(k_dst_solve<64, true, __nv_bfloat16>, SolveSmem<64>::BYTES, spare) ||
             !size_solve(k_dst_solve<32, true, __nv_bfloat16>, SolveSmem<32>::BYTES, spare)))
     return 1;
+  if (tf ? !(size_solve(k_dst_solve_wide<false, float>, Wide<float>::BYTES, t.wide_ctas, kWideThreads) &&
+             size_solve(k_dst_solve_wide<true, float>, Wide<float>::BYTES, spare, kWideThreads))
+         : !(size_solve(k_dst_solve_wide<false, __nv_bfloat16>, Wide<__nv_bfloat16>::BYTES, t.wide_ctas, kWideThreads) &&
+             size_solve(k_dst_solve_wide<true, __nv_bfloat16>, Wide<__nv_bfloat16>::BYTES, spare, kWideThreads)))
+    return 1;
   const char* bn = std::getenv("HQ_SOLVE_BN");
   t.wide_only = bn != nullptr && std::atoi(bn) == 64;
   // (the resident fold matrix is bf16: as TF32 words it would need 256 KB of shared memory at 512^2)
@@ -1876,6 +2185,10 @@ int dst_tc_init(hq_grid_s* g, std::string& err) {
   bad |= make_map(enc, &t.a1_lo, g->op_lo[1], kMaxRhs * nxp, nyp, err, 128, tf);
   // S_x, S_y (or the fold matrices, half as wide) as [rows][K]
   const uint64_t kx = g->fold ? nxp / 2 : nxp, ky = g->fold ? nyp / 2 : nyp;
+  bad |= make_map(enc, &t.fx_hi, g->sx_hi, nxp, kx, err, 128, tf);
+  bad |= make_map(enc, &t.fx_lo, g->sx_lo, nxp, kx, err, 128, tf);
+  bad |= make_map(enc, &t.fy_hi, g->sy_hi, nyp, ky, err, 128, tf);
+  bad |= make_map(enc, &t.fy_lo, g->sy_lo, nyp, ky, err, 128, tf);
   for (int i = 0; i < 2; ++i) {
     const uint32_t bn = i == 0 ? 64 : 32;
     bad |= make_map(enc, &t.bx_hi[i], g->sx_hi, nxp, kx, err, bn, tf);
@@ -2015,6 +2328,29 @@ void solve_fused(hq_grid_s* g, int R, int final_mode, int last, cudaStream_t s, 
   auto tiles = [&](int bn) {
     return std::max(R * (g->nyp / BM) * (g->nxp / bn), R * (g->nxp / BM) * (g->nyp / bn));
   };
+  const bool halves = !g->fold || (g->nx % 256 == 0 && g->ny % 256 == 0);   // a slot block lies in one half
+  if (halves && tiles(64) > 3 * t.ctas[0] && !t.wide_only) {
+    // more than three 128 x 64 tiles per CTA: 128 x 128 tiles, pipelined.  2048^2, two right-hand sides:
+    // 295 us with 128 x 64 tiles, 228 us here; 1536^2: 150 and 122; with fewer tiles the last, half
+    // empty wave of large tiles costs more than the overlap gains (1024^2, three: 86 and 92).
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::min(t.wide_ctas, tiles(128)));
+    cfg.blockDim = dim3(kWideThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    auto go = [&](auto* kern, int smem) {
+      cfg.dynamicSmemBytes = (size_t)smem;
+      cudaLaunchKernelEx(&cfg, kern, t.fx_hi, t.fx_lo, t.fy_hi, t.fy_lo, t.a0_hi, t.a0_lo, t.a1_hi, t.a1_lo, a);
+    };
+    using B16 = __nv_bfloat16;
+    if (g->tf32) go(a.rsum ? &k_dst_solve_wide<true, float> : &k_dst_solve_wide<false, float>, Wide<float>::BYTES);
+    else go(a.rsum ? &k_dst_solve_wide<true, B16> : &k_dst_solve_wide<false, B16>, Wide<B16>::BYTES);
+    return;
+  }
   const bool narrow = !t.wide_only && tiles(32) <= t.ctas[1];
   const int v = narrow ? 1 : 0;
   cudaLaunchConfig_t cfg = {};

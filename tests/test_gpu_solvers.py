@@ -57,13 +57,17 @@ def test_poisson_fp64_sizes(hq, nx, ny, nrhs):
 @pytest.mark.parametrize("precision,nx,ny,nrhs", [("fp32", 8, 8, 1), ("fp32", 96, 80, 5), ("fp32", 128, 128, 2),
                                                     ("fp32", 256, 256, 1), ("fp32", 256, 256, 5), ("fp32", 256, 384, 2),
                                                     ("fp32", 512, 512, 1), ("fp32", 512, 512, 4), ("fp32", 512, 512, 5),
-                                                    ("tf32x3", 200, 72, 4), ("tf32x3", 256, 256, 3)])
+                                                    ("fp32", 640, 384, 5), ("fp32", 1500, 1030, 4),
+                                                    ("fp32", 1024, 1280, 4), ("fp32", 2304, 130, 1),
+                                                    ("tf32x3", 200, 72, 4), ("tf32x3", 256, 256, 3),
+                                                    ("tf32x3", 1024, 1536, 4)])
 def test_poisson_fp32_sizes(hq, precision, nx, ny, nrhs):
     """FP32 from the caller's sources to the caller's array in one launch: 3e-5 (bf16x3) and 8e-6
-    (TF32x3), the bars of the parity tests of these operand splits."""
+    (TF32x3), the bars of the parity tests of these operand splits; above 512 cells twice that
+    (the FP32 sums of a rough source grow with the square root of the length)."""
     err, same = solve_case(hq, nx, ny, nrhs, precision)
     print(f"{precision} {nx}x{ny} x {nrhs}: {err:.1e}")
-    assert err <= (3e-5 if precision == "fp32" else 8e-6) and same
+    assert err <= (3e-5 if precision == "fp32" else 8e-6) * (2 if max(nx, ny) > 512 else 1) and same
 
 
 @pytest.mark.parametrize("nx,ny", [(48, 40), (128, 64), (64, 130)])
