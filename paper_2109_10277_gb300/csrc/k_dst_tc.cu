@@ -1606,8 +1606,17 @@ __global__ void __launch_bounds__(kClThreads, 1)
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k) {
             const uint64_t off = (uint64_t)((k * 32) >> 4);
-            mma_bf16_ta(tmem, ta + 8u * k, bh + off, Cfg<BN>::IDESC2, (kb | k) != 0 ? 1u : 0u);
-            mma_bf16_ta(tmem, ta + (uint32_t)(K / 2) + 8u * k, bh + off, Cfg<BN>::IDESC, 1u);
+            const uint32_t on = (kb | k) != 0 ? 1u : 0u;
+            if constexpr (C::LOCAL) {
+              // F_hi X_hi + F_hi X_lo and, apart, F_lo X_hi: the streamed solve's order of additions
+              // (the faster grouping below flips last bits of the splits)
+              mma_bf16_ta(tmem, ta + 8u * k, bh + off, Cfg<BN>::IDESC, on);
+              mma_bf16_ta(tmem, ta + 8u * k, bh + off + (uint64_t)((BN * 128) >> 4), Cfg<BN>::IDESC, 1u);
+              mma_bf16_ta(tmem + BN, ta + (uint32_t)(K / 2) + 8u * k, bh + off, Cfg<BN>::IDESC, on);
+            } else {
+              mma_bf16_ta(tmem, ta + 8u * k, bh + off, Cfg<BN>::IDESC2, on);
+              mma_bf16_ta(tmem, ta + (uint32_t)(K / 2) + 8u * k, bh + off, Cfg<BN>::IDESC, 1u);
+            }
           }
         }
         __syncwarp();

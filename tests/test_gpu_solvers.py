@@ -139,3 +139,27 @@ def test_dependency_wait_times_out(hq, monkeypatch, n):
     for r in range(2):
         assert rel(got[r], O.poisson_solve(O.GridSpec(**g), src[r].double().cpu())) <= 3e-5
     good.close()
+
+
+@pytest.mark.parametrize("order", [1, 2, 3])
+def test_four_particles_per_cell(hq, monkeypatch, order):
+    """FP32, 2 x 2 particles per cell: the passes that take a cell's four particles per thread (from 2^18
+    particles on; here 2^18 at 256 x 256) against the passes that evaluate every particle alone
+    (HQ_NO_F4CACHE=1), a driver strong enough to tear cells apart, walls included.  Within the bf16x3
+    error of a solve (3e-5), which the changed order of the FP32 sums flips in the operand splits."""
+    g = dict(nx=256, ny=256, nzeta=24, xmin=-2.0, xmax=2.0, ymin=-2.0, ymax=2.0, zeta_min=-0.6, zeta_max=0.6,
+             shape_order=order, ppc_x=2, ppc_y=2, n_pc_iter=5)
+    beam = I.random_beam(40_000, 0.15, 0.15, 0.2, 8.0)
+    outs = []
+    for mode in ("0", "1"):
+        monkeypatch.setenv("HQ_NO_F4CACHE", mode)
+        grid = hq.Grid(g, precision="fp32")
+        out = grid.alloc_out(("rho", "jx", "jz", "chi", "ez", "psi", "bx"))
+        grid.sweep([hq.Beam(beam)], out=out)
+        outs.append((out, grid.sync()))
+        grid.close()
+    assert abs(outs[0][1] - outs[1][1]) <= 2   # particles removed, up to roundings at the threshold
+    for k in outs[0][0]:
+        dev = rel(outs[0][0][k], outs[1][0][k])
+        print(f"order {order} {k}: {dev:.1e}")
+        assert dev <= 3e-5, k
