@@ -1330,7 +1330,8 @@ template <int BN, int MODE> struct Cl {
   static constexpr int DATA = 0;
   static constexpr int DATA_BYTES = (DB ? 2 : 1) * BUF > TILE ? (DB ? 2 : 1) * BUF : (TILE + 127) / 128 * 128;
   // LOCAL: staged sources, BN rows (shared by R CTAs, rounded up) of R x 128 floats over R CTAs
-  static constexpr int SRC = DATA + DATA_BYTES, SRC_BYTES = LOCAL ? (BN + kMaxRhs - 1) * 512 : 0;
+  // MODE 1: kSrcRows rows of R x 256 floats (apart from the data buffers: a peer may already exchange)
+  static constexpr int SRC = DATA + DATA_BYTES, SRC_BYTES = LOCAL ? (BN + kMaxRhs - 1) * 512 : kSrcRows * kMaxRhs * 1024;
   static constexpr int BARS = SRC + SRC_BYTES;
   static constexpr int BYTES = BARS + 128 + 1024;
   static constexpr uint32_t TX = 128, TY = TX + K;          // tensor-memory columns: accumulator, x slice, y slice
@@ -1489,8 +1490,15 @@ __global__ void __launch_bounds__(kClThreads, 1)
   const uint32_t buf0 = base + C::DATA, buf1 = C::DB ? buf0 + C::BUF : buf0;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort_f = &s_abort;
-  uint32_t rank;
+  uint32_t rank, cluster_ctas;
   asm("mov.u32 %0, %cluster_ctarank;" : "=r"(rank));
+  asm("mov.u32 %0, %cluster_nctaid.x;" : "=r"(cluster_ctas));
+  if (cluster_ctas != (uint32_t)(C::LOCAL ? a.R * CPR : CPR)) {
+    // not launched in the clusters the exchange addresses (a tool that drops the launch attribute):
+    // report it instead of writing to peers that do not exist
+    if (threadIdx.x == 0) atomicOr(a.status, DEV_TIMEOUT);
+    return;
+  }
   // right-hand side r, x slot block b, position q among the CTAs of (r, b), y slot block j, tile t
   const int q = (int)rank % CPR, j = q / TPB, t = q - j * TPB;
   const int cl = (int)blockIdx.x / CPR;   // MODE > 0: cluster index (clusters of CPR CTAs)
@@ -1519,7 +1527,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
   if (!C::LOCAL && cl >= a.R * MB) {
     // clusters beyond the products' only form sources (256^2, two right-hand sides: 32 CTAs multiply)
     if (warp < 8) {
-      solve_sources_any<BN>(a, reinterpret_cast<float*>(basep + C::DATA), ctr_src);
+      solve_sources_any<BN>(a, reinterpret_cast<float*>(basep + C::SRC), ctr_src);
       if (threadIdx.x == 0) {
         const unsigned long long seen = atomicAdd(a.gbar, 1ull);
         if (seen == gridDim.x - 1ull) {
@@ -1566,7 +1574,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
       cl_wait();
       asm volatile("fence.proxy.async.shared::cluster;" ::: "memory");
     } else {
-      solve_sources_any<BN>(a, reinterpret_cast<float*>(basep + C::DATA), ctr_src);   // staged in the data buffers
+      solve_sources_any<BN>(a, reinterpret_cast<float*>(basep + C::SRC), ctr_src);
     }
   }
   const int row = (warp & 3) * 32 + lane, half = warp >> 2;
