@@ -311,7 +311,7 @@ hq_status solve_fields_impl(hq_grid_s* g, int slice) {
         if (g->fp64) dst_solve_f64(g, 2, s, reinterpret_cast<const double*>(g->scale_h));
         else dst_solve_tc_shifted(g, 2, s);
       }
-      { Prof p(g, HQ_K_FIELD, 4); launch_pcg_iter<T>(g, slice, k, chi_cur, s); }
+      { Prof p(g, HQ_K_FIELD, g->pcg_part ? 3 : 2); launch_pcg_iter<T>(g, slice, k, chi_cur, s); }
     }
     tape_slice_end(g);
     return HQ_OK;
@@ -1082,14 +1082,14 @@ hq_status hq_grid_create(const hq_grid_desc* desc, void* cuda_stream, hq_grid_t*
       HQ_ALLOC(g->xs4, 4 * ts * nn);
       HQ_ALLOC(g->xs1, ts * nn);
     } else {
-      // deterministic mode: per-block partial dot products of the PCG
-      const int64_t nb = std::max<int64_t>((nn + 255) / 256, (int64_t)((g->nx + 127) / 128) * g->ny);
-      HQ_ALLOC(g->pcg_part, 16 * nb);
+      // deterministic mode: per-block partial sums of the PCG
+      HQ_ALLOC(g->pcg_part, 6 * sizeof(double) * pcg_blocks(nn));
     }
     HQ_ALLOC(g->pcg_r, 2 * ts * nn);
-    HQ_ALLOC(g->pcg_p, 2 * ts * nn);
+    HQ_ALLOC(g->pcg_p, 4 * ts * nn);
     HQ_ALLOC(g->pcg_s, sizeof(double) * 4 * kMaxPcg * 2);
-    for (void* p : {g->pcg_r, g->pcg_p}) cudaMemset(p, 0, 2 * ts * nn);
+    cudaMemset(g->pcg_r, 0, 2 * ts * nn);
+    cudaMemset(g->pcg_p, 0, 4 * ts * nn);
     cudaMemset(g->bjp, 0, 4 * ts * nn);
     cudaMemset(g->xs4, 0, 4 * ts * nn);
     cudaMemset(g->xs1, 0, ts * nn);

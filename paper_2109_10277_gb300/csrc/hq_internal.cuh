@@ -233,8 +233,8 @@ struct hq_grid_s {
   void* xs4;           // V4: Fx, Fy, Jxx, Jyy (deposited by the explicit source pass)
   void* xs1;           // Jxy
   void* pcg_r;         // V2: residual r
-  void* pcg_p;         // V2: search direction p
-  double* pcg_s;       // [4][kMaxPcg][2]: r.z, p.Ap per iteration and right-hand side
+  void* pcg_p;         // V2 [2][nnode]: search direction p, by iteration parity
+  double* pcg_s;       // [4][kMaxPcg][2]: dot products per iteration and right-hand side
   double* pcg_part;    // deterministic mode: per-block partial dot products (else null)
   void* scale_h;       // the preconditioner's spectral factors 1/(lambda - c), like f32_scale / f64_scale
   void* gf;            // kGF per node (gather fields ExmBy, EypBx, Ez, Bz of the current slice)
@@ -388,6 +388,9 @@ void launch_beam_moments(const hq_beam_view& v, double* m, cudaStream_t s);   //
 template <typename T> void launch_explicit_src(const hq_grid_s* g, cudaStream_t s);
 template <typename T> void launch_pcg_init(const hq_grid_s* g, int slice, const void* cur, const void* chi_cur, void* prev,
                                            void* chi_prev, cudaStream_t s);
+// blocks of the PCG's sums (256 threads): two nodes per thread, so that the blocks' own sums cost less than the
+// nodes', and at most four blocks per SM
+inline unsigned pcg_blocks(int64_t nn) { return (unsigned)std::min<int64_t>((nn + 511) / 512, 4 * 152); }
 template <typename T> void launch_pcg_iter(const hq_grid_s* g, int slice, int k, const void* chi_cur, cudaStream_t s);
 // adjoint (k_adjoint.cu)
 template <typename T> void launch_adj_final(const hq_grid_s* g, const SnapView<T>& s, const void* gf, int slice,

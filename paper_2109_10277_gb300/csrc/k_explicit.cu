@@ -14,8 +14,11 @@
 // FP32 mode), starting from the guess 2 B(i-1) - B(i-2), a fixed number of iterations.
 //
 // Kernels: the source pass over the plasma particles, and per-node PCG steps (the residual and
-// direction vectors are V2 records (Bx, By); the scalars r.z and p.Ap are FP64 sums per
-// iteration and right-hand side, accumulated with one atomic per block).
+// direction vectors are V2 records (Bx, By); the dot products are FP64 sums per iteration and
+// right-hand side, accumulated with one atomic per block).
+#include <algorithm>
+#include <type_traits>
+
 #include "hq_internal.cuh"
 
 namespace hq {
@@ -119,16 +122,10 @@ __global__ void __launch_bounds__(kThreads) k_explicit_src(Plasma<T> pl, Geom gm
 }
 
 // ---------------------------------------------------------------- PCG on (chi - L) B = -rhs
-// A v = chi v - L v at interior node (iy, ix) (wall nodes read 0; every PCG vector is 0 there).
+// chi v - L v from the node's value c and its four neighbours.
 template <typename T>
-__device__ __forceinline__ V2<T> apply_A(const V2<T>* __restrict__ v, const T* __restrict__ chi, const Geom& gm, int iy,
-                                         int ix) {
-  const int nx = gm.nx;
-  const int64_t o = (int64_t)iy * nx + ix;
-  const V2<T> c = v[o], l = v[o - 1], d = v[o - nx];
-  const V2<T> r = ix + 1 < nx ? v[o + 1] : V2<T>{T(0), T(0)};
-  const V2<T> u = iy + 1 < gm.ny ? v[o + nx] : V2<T>{T(0), T(0)};
-  const T k = chi[o];
+__device__ __forceinline__ V2<T> stencil_A(const Geom& gm, T k, const V2<T>& c, const V2<T>& l, const V2<T>& r,
+                                           const V2<T>& d, const V2<T>& u) {
   if constexpr (sizeof(T) == 8) {
     const double dx2 = gm.dx * gm.dx, dy2 = gm.dy * gm.dy;
     return V2<T>{k * c.a - ((r.a - 2.0 * c.a + l.a) / dx2 + (u.a - 2.0 * c.a + d.a) / dy2),
@@ -140,50 +137,54 @@ __device__ __forceinline__ V2<T> apply_A(const V2<T>* __restrict__ v, const T* _
   }
 }
 
-// Block sum of two FP64 values, one atomic per block and value.
-// Block sum of two FP64 values: one atomic per block and value into out, or (part non-null:
-// deterministic FP64 mode) the block's pair stored at part[2 * block] for k_ordered_sum2.
-__device__ __forceinline__ void block_sum2(double a, double b, double* out, double* part_out = nullptr) {
-  __shared__ double part[2][32];
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_down_sync(0xffffffffu, a, o);
-    b += __shfl_down_sync(0xffffffffu, b, o);
-  }
-  const int w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  if ((threadIdx.x & 31) == 0) {
-    part[0][w] = a;
-    part[1][w] = b;
-  }
-  __syncthreads();
-  if (threadIdx.x < 2) {
-    double t = 0.0;
-    for (int k = 0; k < nw; ++k) t += part[threadIdx.x][k];
-    if (part_out) part_out[2 * (blockIdx.y * gridDim.x + blockIdx.x) + threadIdx.x] = t;
-    else if (t != 0.0) atomicAdd(out + threadIdx.x, t);
-  }
+// A v = chi v - L v at interior node (iy, ix), v(o) the vector at node o (wall nodes read 0; every PCG
+// vector is 0 there).
+template <typename T, typename F>
+__device__ __forceinline__ V2<T> apply_A(F&& v, const T* __restrict__ chi, const Geom& gm, int iy, int ix, const V2<T>& c) {
+  const int nx = gm.nx;
+  const int64_t o = (int64_t)iy * nx + ix;
+  const V2<T> z{T(0), T(0)}, l = v(o - 1), d = v(o - nx);
+  const V2<T> r = ix + 1 < nx ? v(o + 1) : z, u = iy + 1 < gm.ny ? v(o + nx) : z;
+  return stencil_A<T>(gm, chi[o], c, l, r, d, u);
 }
 
-// out[c] = sum over the nb block pairs of part[2 b + c] in a fixed order (one block of 256
-// threads: strided partial sums in increasing b, then a fixed tree): the deterministic mode's
-// dot products.
-__global__ void k_ordered_sum2(const double* __restrict__ part, int nb, double* out) {
-  __shared__ double red[2][256];
-  double a = 0.0, b = 0.0;
-  for (int i = threadIdx.x; i < nb; i += 256) {
-    a += part[2 * i];
-    b += part[2 * i + 1];
-  }
-  red[0][threadIdx.x] = a;
-  red[1][threadIdx.x] = b;
+// Block sums of N FP64 values, block of 256 threads: one atomic per block and value into out[i], or
+// (part non-null: deterministic FP64 mode) the block's sums stored at part[N * block] for k_ordered_sum.
+// The values change hands through shared memory, a warp per value: the FP64 pipe takes a warp
+// instruction per 16 clocks of an SM, and N shuffle trees in each of the eight warps are 240 of them for
+// N = 6, against 78.
+constexpr int kSumThreads = 256;
+template <int N>
+__device__ __forceinline__ void block_sum(const double* v, double* const* out, double* part_out) {
+  __shared__ double part[N][kSumThreads];
+#pragma unroll
+  for (int i = 0; i < N; ++i) part[i][threadIdx.x] = v[i];
+  __syncthreads();
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (w >= N) return;
+  double t = 0.0;
+  for (int k = lane; k < kSumThreads; k += 32) t += part[w][k];
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+  if (lane) return;
+  if (part_out) part_out[(int64_t)N * blockIdx.x + w] = t;
+  else if (t != 0.0) atomicAdd(out[w >> 1] + (w & 1), t);
+}
+
+// Sum c = blockIdx.x of the nb blocks' partial sums part[N b + c] in a fixed order (256 threads: strided
+// partial sums in increasing b, then a fixed tree): the deterministic mode's dot products.
+struct PcgSums { double* out[3]; };   // r.z, z.Az, p.Az: a pair (the right-hand sides) each
+__global__ void k_ordered_sum(const double* __restrict__ part, int nb, PcgSums sums) {
+  __shared__ double red[256];
+  double a = 0.0;
+  const int c = blockIdx.x;
+  for (int i = threadIdx.x; i < nb; i += 256) a += part[(int64_t)gridDim.x * i + c];
+  red[threadIdx.x] = a;
   __syncthreads();
   for (int h = 128; h > 0; h >>= 1) {
-    if (threadIdx.x < h) {
-      red[0][threadIdx.x] += red[0][threadIdx.x + h];
-      red[1][threadIdx.x] += red[1][threadIdx.x + h];
-    }
+    if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
     __syncthreads();
   }
-  if (threadIdx.x < 2) out[threadIdx.x] = red[threadIdx.x][0];
+  if (threadIdx.x == 0) sums.out[c >> 1][c & 1] = red[0];
 }
 
 // Per-node right-hand side of the two Helmholtz-like equations and the initial residual
@@ -222,7 +223,7 @@ template <typename T> struct PcgInit {
       const T ty = s.b + dxc(fxy, iy, ix, nx, i2x) + dyc(fyy, iy, ix, gm.ny, i2y) + (bp.b - bn.b) * i2z;
       const T rx = -dyc(jz, iy, ix, gm.ny, i2y) + ty;
       const T ry = dxc(jz, iy, ix, nx, i2x) - tx;
-      const V2<T> ax = apply_A<T>(x, chi, gm, iy, ix);
+      const V2<T> ax = apply_A<T>([&](int64_t i) { return x[i]; }, chi, gm, iy, ix, x[o]);
       v[0] = -rx - ax.a;
       v[1] = -ry - ax.b;
     }
@@ -240,82 +241,133 @@ __global__ void k_pcg_init(PcgInit<T> f, Sink sink) {
   visit_nodes<2, T>(f.gm, sink, 2, f);
 }
 
-// z = P r = -(solved) (the shifted solve gives (L - c)^{-1} r); rz[k] += r . z.  Iteration 0 also
-// clears the consumed source records.
+// An iteration takes two node passes, with one reduction between them.  z = P r = -(solved) (the shifted
+// solve gives (L - c)^{-1} r); with the last direction p' the new one is p = z + beta p', beta =
+// (r.z) / (r.z)', and p.Ap = z.Az + 2 beta p'.Az + beta^2 p'.Ap', so that r.z, z.Az and p'.Az are all
+// that the node sums have to give: beta is not needed before they are complete.  Forming p first and
+// p.Ap from it took four passes (r.z; p; p.Ap; x and r) with a full drain between each two; at 256^2,
+// where a pass is launch and latency and not its bytes, a slice (six iterations) took 241 us with four
+// launches, 240 with one cooperative launch and three grid barriers, and takes 219 with two.  (The expanded form stays a
+// sum of squares: p'.Az is measured, not taken to be -beta p'.Ap', so that a residual at the rounding
+// floor cannot turn p.Ap negative by cancellation.)
+
+// First pass: the three sums.  Iteration 0 also clears the consumed source records.
 template <typename T>
-__global__ void k_pcg_z(const T* __restrict__ solved, const V2<T>* __restrict__ r, double* rz, int64_t nn, int first,
-                        V4<T>* xs4, T* xs1, V2<T>* bjp, V2<T>* bjn, double* part) {
-  const int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double a = 0.0, b = 0.0;
-  if (o < nn) {
-    const V2<T> q = r[o];
-    a = -(double)q.a * (double)solved[o];
-    b = -(double)q.b * (double)solved[nn + o];
-    if (first) {
+__global__ void __launch_bounds__(kSumThreads) k_pcg_dots(const T* __restrict__ solved, const V2<T>* __restrict__ r,
+                                                  const V2<T>* __restrict__ p_old, const T* __restrict__ chi, Geom gm,
+                                                  PcgSums sums, double* part, V4<T>* xs4, T* xs1, V2<T>* bjp, V2<T>* bjn) {
+  pdl_trigger();
+  pdl_wait();
+  const int nx = gm.nx;
+  const int64_t nn = (int64_t)nx * gm.ny;
+  double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  const auto z = [&](int64_t i) { return V2<T>{-solved[i], -solved[nn + i]}; };
+  for (int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o < nn; o += (int64_t)gridDim.x * blockDim.x) {
+    const int iy = (int)(o / nx), ix = (int)(o - (int64_t)iy * nx);
+    const V2<T> zo = z(o), q = r[o];
+    v[0] += (double)q.a * (double)zo.a;
+    v[1] += (double)q.b * (double)zo.b;
+    if (ix > 0 && iy > 0) {
+      const V2<T> az = apply_A<T>(z, chi, gm, iy, ix, zo);
+      v[2] += (double)zo.a * (double)az.a;
+      v[3] += (double)zo.b * (double)az.b;
+      if (p_old) {
+        const V2<T> pp = p_old[o];
+        v[4] += (double)pp.a * (double)az.a;
+        v[5] += (double)pp.b * (double)az.b;
+      }
+    }
+    if (!p_old) {
       xs4[o] = V4<T>{T(0), T(0), T(0), T(0)};
       xs1[o] = T(0);
       bjp[o] = V2<T>{T(0), T(0)};
       bjn[o] = V2<T>{T(0), T(0)};
     }
   }
-  block_sum2(a, b, rz, part);
+  block_sum<6>(v, sums.out, part);
 }
 
-// p = z + beta p, beta = rz[k] / rz[k-1] (0 on the first iteration or a zero denominator).
-template <typename T>
-__global__ void k_pcg_p(const T* __restrict__ solved, V2<T>* p, const double* __restrict__ rz_k,
-                        const double* __restrict__ rz_km1, int64_t nn) {
-  const int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= nn) return;
-  double be[2] = {0.0, 0.0};
-  if (rz_km1)
-    for (int c = 0; c < 2; ++c) be[c] = rz_km1[c] != 0.0 ? rz_k[c] / rz_km1[c] : 0.0;
-  const V2<T> q = p[o];
-  p[o] = V2<T>{T(-solved[o] + be[0] * q.a), T(-solved[nn + o] + be[1] * q.b)};
+// z + beta p rounded to T, beta in 64 bits.  FP32: beta = bh + bl, the product and the sum with their
+// rounding errors (Dekker's and Knuth's error-free forms), since a node needs its neighbours' values
+// too: ten of these per node in FP64 (two conversions, a product and a rounding each, 16 clocks a warp
+// instruction), with shuffle trees in the sums, made a slice of 256^2 take 276 us instead of 219.
+__device__ __forceinline__ double axpy_rn(double z, double b, double p) { return z + b * p; }
+struct Beta32 { float h, l; };
+__device__ __forceinline__ float axpy_rn(float z, const Beta32& b, float p) {
+  const float m = __fmul_rn(b.h, p), e = __fmaf_rn(b.l, p, __fmaf_rn(b.h, p, -m));
+  const float t = __fadd_rn(z, m), u = __fsub_rn(t, z);
+  const float d = __fadd_rn(__fsub_rn(z, __fsub_rn(t, u)), __fsub_rn(m, u));
+  return __fadd_rn(t, __fadd_rn(d, e));
 }
 
-// pq[k] += p . (A p)
-template <typename T>
-__global__ void k_pcg_q(const V2<T>* __restrict__ p, const T* __restrict__ chi, Geom gm, double* pq, double* part) {
-  const int ix = blockIdx.x * blockDim.x + threadIdx.x, iy = blockIdx.y;
-  double a = 0.0, b = 0.0;
-  if (ix < gm.nx && ix > 0 && iy > 0) {
-    const V2<T> ap = apply_A<T>(p, chi, gm, iy, ix);
-    const V2<T> q = p[(int64_t)iy * gm.nx + ix];
-    a = (double)q.a * (double)ap.a;
-    b = (double)q.b * (double)ap.b;
-  }
-  block_sum2(a, b, pq, part);
-}
-
-// x += alpha p, r -= alpha A p with alpha = rz[k] / pq[k] (0 for a zero denominator); the new r
-// goes to the operand writer as the next preconditioner solve's sources.
+// Second pass: p = z + beta p' (into the other buffer: the neighbours' p' are still read), x += alpha p,
+// r -= alpha A p, alpha = (r.z) / (p.Ap) (a zero denominator gives a zero factor); the new r goes to the
+// operand writer as the next preconditioner solve's sources.
 template <typename T> struct PcgStep {
   static constexpr int NR = 2;
-  const V2<T>* p;
+  const T* solved;
+  const V2<T>* p_old;        // null: first iteration
+  V2<T>* p;
   const T* chi;
   V2<T>* x;
   V2<T>* r;
-  const double* rz;
-  const double* pq;
+  PcgSums sums;              // r.z, z.Az, p'.Az
+  const double* rz_prev;     // (r.z)', p'.Ap'
+  const double* pq_prev;
+  double* pq;                // p.Ap, kept for the next iteration
   Geom gm;
+  T al[2];
+  std::conditional_t<sizeof(T) == 8, double, Beta32> be[2];
+  // alpha and beta, by two threads of the block (two divisions each: FP64 work worth doing once)
+  __device__ void scalars(bool keep) {
+    __shared__ double ab[2][2];
+    const int c = threadIdx.x;
+    if (c < 2) {
+      const double rz = sums.out[0][c], b = p_old && rz_prev[c] != 0.0 ? rz / rz_prev[c] : 0.0;
+      double d = sums.out[1][c];
+      if (p_old) d += b * (2.0 * sums.out[2][c] + b * pq_prev[c]);
+      ab[0][c] = d != 0.0 ? rz / d : 0.0;
+      ab[1][c] = b;
+      if (keep) pq[c] = d;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      al[i] = T(ab[0][i]);
+      const double b = ab[1][i];
+      if constexpr (sizeof(T) == 8) be[i] = b;
+      else be[i] = Beta32{(float)b, (float)(b - (double)(float)b)};
+    }
+  }
   __device__ void operator()(int iy, int ix, T* v) const {
-    const int64_t o = (int64_t)iy * gm.nx + ix;
+    const int64_t o = (int64_t)iy * gm.nx + ix, nn = (int64_t)gm.nx * gm.ny;
     v[0] = v[1] = T(0);
+    const auto dir = [&](int64_t i) {
+      V2<T> q{-solved[i], -solved[nn + i]};
+      if (p_old) {
+        const V2<T> w = p_old[i];
+        q = V2<T>{axpy_rn(q.a, be[0], w.a), axpy_rn(q.b, be[1], w.b)};
+      }
+      return q;
+    };
+    const V2<T> pp = dir(o);
+    p[o] = pp;
     if (ix > 0 && iy > 0) {
-      const V2<T> ap = apply_A<T>(p, chi, gm, iy, ix);
-      const T al0 = T(pq[0] != 0.0 ? rz[0] / pq[0] : 0.0), al1 = T(pq[1] != 0.0 ? rz[1] / pq[1] : 0.0);
-      const V2<T> pp = p[o], xx = x[o], rr = r[o];
-      x[o] = V2<T>{xx.a + al0 * pp.a, xx.b + al1 * pp.b};
-      v[0] = rr.a - al0 * ap.a;
-      v[1] = rr.b - al1 * ap.b;
+      const V2<T> ap = apply_A<T>(dir, chi, gm, iy, ix, pp);
+      const V2<T> xx = x[o], rr = r[o];
+      x[o] = V2<T>{xx.a + al[0] * pp.a, xx.b + al[1] * pp.b};
+      v[0] = rr.a - al[0] * ap.a;
+      v[1] = rr.b - al[1] * ap.b;
       r[o] = V2<T>{v[0], v[1]};
     }
   }
 };
 
 template <typename T, typename Sink>
-__global__ void k_pcg_x(PcgStep<T> f, Sink sink) {
+__global__ void k_pcg_step(PcgStep<T> f, Sink sink) {
+  pdl_trigger();
+  pdl_wait();
+  f.scalars(blockIdx.x == 0 && blockIdx.y == 0);
   visit_nodes<2, T>(f.gm, sink, 2, f);
 }
 
@@ -327,7 +379,7 @@ inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t
 
 }  // namespace
 
-// pcg_s layout: [which][k][rhs], which 0: r.z, 1: p.Ap
+// pcg_s layout: [which][k][rhs], which 0: r.z, 1: p.Ap, 2: z.Az, 3: p'.Az
 inline double* pcg_at(const hq_grid_s* g, int which, int k) { return g->pcg_s + ((size_t)which * kMaxPcg + k) * 2; }
 
 template <typename T>
@@ -365,23 +417,20 @@ void launch_pcg_init(const hq_grid_s* g, int slice, const void* cur, const void*
 
 template <typename T>
 void launch_pcg_iter(const hq_grid_s* g, int slice, int k, const void* chi_cur, cudaStream_t s) {
-  const int64_t nn = g->nnode;
   const T* solved = reinterpret_cast<const T*>(g->solved);
   const T* chi = reinterpret_cast<const T*>(chi_cur);
   V2<T>* r = reinterpret_cast<V2<T>*>(g->pcg_r);
-  V2<T>* p = reinterpret_cast<V2<T>*>(g->pcg_p);
-  double* part = g->pcg_part;   // deterministic mode: per-block partial dot products
-  const unsigned nbz = blocks_for(nn, 256);
-  k_pcg_z<T><<<nbz, 256, 0, s>>>(solved, r, pcg_at(g, 0, k), nn, k == 0, reinterpret_cast<V4<T>*>(g->xs4),
-                                 reinterpret_cast<T*>(g->xs1), reinterpret_cast<V2<T>*>(bjp_at(g, slice + 1)),
-                                 reinterpret_cast<V2<T>*>(g->bjn), part);
-  if (part) k_ordered_sum2<<<1, 256, 0, s>>>(part, (int)nbz, pcg_at(g, 0, k));
-  k_pcg_p<T><<<blocks_for(nn, 256), 256, 0, s>>>(solved, p, pcg_at(g, 0, k), k > 0 ? pcg_at(g, 0, k - 1) : nullptr, nn);
-  const dim3 g2((unsigned)((g->nx + 127) / 128), (unsigned)g->ny);
-  k_pcg_q<T><<<g2, 128, 0, s>>>(p, chi, g->geom, pcg_at(g, 1, k), part);
-  if (part) k_ordered_sum2<<<1, 256, 0, s>>>(part, (int)(g2.x * g2.y), pcg_at(g, 1, k));
-  PcgStep<T> f{p, chi, reinterpret_cast<V2<T>*>(g->bm), r, pcg_at(g, 0, k), pcg_at(g, 1, k), g->geom};
-  with_sink<T>(g, [&](auto sink) { k_pcg_x<T, decltype(sink)><<<src_grid(g), 128, 0, s>>>(f, sink); });
+  V2<T>* p = reinterpret_cast<V2<T>*>(g->pcg_p) + (k & 1) * (int64_t)g->nnode;   // the two directions, by parity
+  const V2<T>* p_old = k > 0 ? reinterpret_cast<V2<T>*>(g->pcg_p) + (~k & 1) * (int64_t)g->nnode : nullptr;
+  const PcgSums sums{{pcg_at(g, 0, k), pcg_at(g, 2, k), pcg_at(g, 3, k)}};
+  double* part = g->pcg_part;   // deterministic mode: per-block partial sums
+  const unsigned nb = pcg_blocks(g->nnode);
+  launch_pdl(k_pcg_dots<T>, nb, kSumThreads, 0, s, solved, r, p_old, chi, g->geom, sums, part, reinterpret_cast<V4<T>*>(g->xs4),
+             reinterpret_cast<T*>(g->xs1), reinterpret_cast<V2<T>*>(bjp_at(g, slice + 1)), reinterpret_cast<V2<T>*>(g->bjn));
+  if (part) k_ordered_sum<<<6, 256, 0, s>>>(part, (int)nb, sums);
+  PcgStep<T> f{solved, p_old, p, chi, reinterpret_cast<V2<T>*>(g->bm), r, sums, k > 0 ? pcg_at(g, 0, k - 1) : nullptr,
+               k > 0 ? pcg_at(g, 1, k - 1) : nullptr, pcg_at(g, 1, k), g->geom, {}, {}};
+  with_sink<T>(g, [&](auto sink) { launch_pdl(k_pcg_step<T, decltype(sink)>, src_grid(g), 128, 0, s, f, sink); });
 }
 
 template void launch_explicit_src<float>(const hq_grid_s*, cudaStream_t);

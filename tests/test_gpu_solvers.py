@@ -163,3 +163,26 @@ def test_four_particles_per_cell(hq, monkeypatch, order):
         dev = rel(outs[0][0][k], outs[1][0][k])
         print(f"order {order} {k}: {dev:.1e}")
         assert dev <= 3e-5, k
+
+
+@pytest.mark.parametrize("precision,nx,ny,nz,iters", [("fp64", 17, 64, 12, 1), ("fp64", 40, 23, 12, 6),
+                                                      ("fp64", 650, 490, 3, 4), ("fp32", 72, 40, 12, 2),
+                                                      ("fp32", 64, 64, 12, 40), ("fp32", 650, 490, 3, 4)])
+def test_explicit_sizes(hq, precision, nx, ny, nz, iters):
+    """Explicit B_perp against the oracle: one and many PCG iterations (40 in FP32 iterate long past the
+    rounding floor, where the dot products cancel), odd extents, and more nodes than one round of the
+    dot products' blocks takes (608 x 512).  FP64 1e-9 (eps 1e-16, gathers and PCG over a few slices at a
+    condition number of 1e4-1e5), FP32 1e-3: the bar of a recorded field of an FP32 sweep."""
+    g = dict(nx=nx, ny=ny, nzeta=nz, xmin=-4.0, xmax=4.0, ymin=-4.0, ymax=4.0, zeta_min=-0.6, zeta_max=0.6,
+             n_pc_iter=iters, bperp_solver="explicit")
+    beam = I.random_beam(20_000, 0.4, 0.4, 0.3, 0.5)
+    ref = O.sweep(O.GridSpec(**g), [O.as_beam(beam)], record=("bx", "by", "ez"))
+    grid = hq.Grid(g, precision=precision)
+    out = grid.alloc_out(("bx", "by", "ez"))
+    grid.sweep([hq.Beam(beam)], out=out)
+    assert grid.sync() == 0
+    grid.close()
+    for k in out:
+        dev = rel(out[k], ref.fields[k])
+        print(f"{precision} {nx}x{ny} {iters} iterations {k}: {dev:.1e}")
+        assert dev <= (1e-9 if precision == "fp64" else 1e-3), k
