@@ -648,7 +648,7 @@ hq_status adjoint_impl(hq_grid_s* g, const hq_beam_view* beams, int nb, int witn
                      sn.alive, reinterpret_cast<const T*>(sn.hist), f32 ? sn.hsum : nullptr, f32 ? sn.cell : nullptr,
                      f32 ? sn.fx : nullptr, f32 ? sn.fy : nullptr, f32 ? sn.opp : nullptr};
       const void* gf = a->tape_gf[t];
-      cudaMemsetAsync(a->jtot, 0, 2 * ts * nn, s);
+      if (npc == 0) cudaMemsetAsync(a->jtot, 0, 2 * ts * nn, s);   // (else the first pc_post writes it)
       if (seeds) {
         Prof p(g, HQ_K_FIELD, 1);
         launch_adj_seed<T>(g, *seeds, i, a->tbar, a->fbar_b, dcur, s);
@@ -665,23 +665,24 @@ hq_status adjoint_impl(hq_grid_s* g, const hq_beam_view* beams, int nb, int witn
       char* bb = reinterpret_cast<char*>(a->bbar);
       { Prof p(g, HQ_K_FIELD, 1); launch_adj_bstart<T>(g, a->fbar_b, a->carry[i % 3], bb + (size_t)npc * brec, s); }
       for (int m = npc; m >= 1; --m) {
-        { Prof p(g, HQ_K_FIELD, 1); launch_adj_pc_pre<T>(g, bb + (size_t)m * brec, bb + (size_t)(m - 1) * brec, s); }
+        char *bm = bb + (size_t)m * brec, *bm1 = bm - brec;
+        { Prof p(g, HQ_K_FIELD, 1); launch_adj_pc_pre<T>(g, bm, s); }
         dst_solve(g, 2);
-        { Prof p(g, HQ_K_FIELD, 1); launch_adj_pc_post<T>(g, dcur, dprev, a->jbar, a->jtot, s); }
+        {
+          Prof p(g, HQ_K_FIELD, 1);
+          launch_adj_pc_post<T>(g, dcur, dprev, a->jbar, a->jtot, bm, bm1, m == npc, s);
+        }
         {
           Prof p(g, HQ_K_TRIAL, 1);
           launch_adj_trial<T>(g, sv, gf, reinterpret_cast<char*>(a->tape_b[t]) + (size_t)(m - 1) * brec, i, a->jbar, av,
-                              a->tbar, bb + (size_t)(m - 1) * brec, a->wbar_p, s);
+                              a->tbar, bm1, a->wbar_p, s);
         }
       }
       {
         Prof p(g, HQ_K_FIELD, 1);
-        launch_adj_guess<T>(g, bb, i >= 1 ? a->carry[(i - 1) % 3] : nullptr, i >= 2 ? a->carry[(i - 2) % 3] : nullptr, s);
-      }
-      {
-        Prof p(g, HQ_K_FIELD, 1);
         const void* sp = seeds && seeds->psi ? static_cast<const char*>(seeds->psi) + (size_t)i * nn * ts : nullptr;
-        launch_adj_main_pre<T>(g, a->tbar, sp, s);
+        launch_adj_main_pre<T>(g, a->tbar, sp, bb, i >= 1 ? a->carry[(i - 1) % 3] : nullptr,
+                               i >= 2 ? a->carry[(i - 2) % 3] : nullptr, s);
       }
       dst_solve(g, 3);
       { Prof p(g, HQ_K_FIELD, 1); launch_adj_main_post<T>(g, dcur, a->rho_ion_bar, a->tbar, s); }
@@ -690,12 +691,13 @@ hq_status adjoint_impl(hq_grid_s* g, const hq_beam_view* beams, int nb, int witn
         Prof p(g, HQ_K_BEAM, 1);
         launch_adj_beam<T>(g, b, beams[b], i, dcur, a->jtot, wbar_b[b], s);
       }
-      // rotate: slice i's record becomes "next" for slice i-1; the old next is cleared for i-2
+      // rotate: slice i's record becomes "next" for slice i-1; the old next is i-2's, written by the
+      // next slice's first pc_post
       void* old_next = dnext;
       dnext = dcur;
       dcur = dprev;
       dprev = old_next;
-      cudaMemsetAsync(dprev, 0, 4 * ts * nn, s);
+      if (npc == 0) cudaMemsetAsync(dprev, 0, 4 * ts * nn, s);
     }
   }
   { Prof p(g, HQ_K_OTHER, 1); launch_adj_init<T>(g, dnext, a->rho_ion_bar, a->wbar_p, s); }

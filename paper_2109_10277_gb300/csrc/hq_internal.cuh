@@ -400,10 +400,11 @@ template <typename T> void launch_adj_trial(const hq_grid_s* g, const SnapView<T
                                            int slice, const void* jbar, const AdjView<T>& a, void* tbar, void* bbar_m1,
                                            double* wbar_p, cudaStream_t st);
 template <typename T> void launch_adj_bstart(const hq_grid_s* g, void* fbar_b, void* carry, void* bbar_n, cudaStream_t st);
-template <typename T> void launch_adj_pc_pre(const hq_grid_s* g, const void* bbar_m, void* bbar_m1, cudaStream_t st);
-template <typename T> void launch_adj_pc_post(const hq_grid_s* g, void* dcur, void* dprev, void* jbar, void* jtot, cudaStream_t st);
-template <typename T> void launch_adj_guess(const hq_grid_s* g, const void* b0, void* c1, void* c2, cudaStream_t st);
-template <typename T> void launch_adj_main_pre(const hq_grid_s* g, const void* tbar, const void* seed_psi, cudaStream_t st);
+template <typename T> void launch_adj_pc_pre(const hq_grid_s* g, const void* bbar_m, cudaStream_t st);
+template <typename T> void launch_adj_pc_post(const hq_grid_s* g, void* dcur, void* dprev, void* jbar, void* jtot,
+                                              const void* bbar_m, void* bbar_m1, int first, cudaStream_t st);
+template <typename T> void launch_adj_main_pre(const hq_grid_s* g, const void* tbar, const void* seed_psi, const void* b0,
+                                               void* c1, void* c2, cudaStream_t st);
 template <typename T> void launch_adj_seed(const hq_grid_s* g, const hq_field_out& seeds, int slice, void* tbar,
                                            void* fbar_b, void* dcur, cudaStream_t st);
 template <typename T> void launch_adj_main_post(const hq_grid_s* g, void* dcur, void* rho_ion_bar, void* tbar,

@@ -274,6 +274,8 @@ template <int P, typename T>
 __global__ void __launch_bounds__(kThreads)
     k_adj_final(SnapView<T> s, const T* __restrict__ gf, Geom gm, int slice, double guard,
                 const V4<T>* __restrict__ dbar_next, AdjView<T> a, T* tbar, V2<T>* fbar_b, double* wbar_p) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= s.n || !s.alive[p]) return;
   const int64_t n = s.n;
@@ -384,6 +386,8 @@ template <int P, typename T>
 __global__ void __launch_bounds__(kThreads)
     k_adj_trial(SnapView<T> s, const T* __restrict__ gf, const V2<T>* __restrict__ bm, Geom gm, int slice, double guard,
                 const V2<T>* __restrict__ jbar, AdjView<T> a, T* tbar, V2<T>* bbar_m1, double* wbar_p) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= s.n || !s.alive[p]) return;
   const int64_t n = s.n;
@@ -510,6 +514,8 @@ __global__ void __launch_bounds__(kThreads)
 // (cleared for the next slice).
 template <typename T>
 __global__ void k_adj_bstart(V2<T>* fbar_b, V2<T>* carry, V2<T>* bbar_n, int64_t nn) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= nn) return;
   const V2<T> c = carry[o], f = fbar_b[o];
@@ -518,23 +524,30 @@ __global__ void k_adj_bstart(V2<T>* fbar_b, V2<T>* carry, V2<T>* bbar_n, int64_t
   fbar_b[o] = V2<T>{T(0), T(0)};
 }
 
-// Mixing B^m = w Bs + (1-w) B^(m-1): the solve gets w Bbar^m, Bbar^(m-1) starts at (1-w) Bbar^m.
+// Mixing B^m = w Bs + (1-w) B^(m-1): the solve gets w Bbar^m, and Bbar^(m-1) starts at (1-w) Bbar^m
+// (k_adj_pc_post).  The reverse sweep's node passes are a few microseconds of launch and latency each,
+// so they launch early (programmatic dependent launch), share what can be shared, and write rather than
+// clear and add: a gradient of 48 slices of 256^2 took 28.7 ms with plain launches, two memsets and a
+// guess kernel more per slice, and takes 27.2.  (This pass inside the solve's source phase: the same.)
 template <typename T, typename Sink>
-__global__ void k_adj_pc_pre(const V2<T>* __restrict__ bbar_m, V2<T>* bbar_m1, T w, Geom gm, Sink sink) {
+__global__ void k_adj_pc_pre(const V2<T>* __restrict__ bbar_m, T w, Geom gm, Sink sink) {
+  pdl_trigger();
+  pdl_wait();
   visit_nodes<2, T>(gm, sink, 2, [&](int iy, int ix, T* v) {
-    const int64_t o = (int64_t)iy * gm.nx + ix;
-    const V2<T> b = bbar_m[o];
-    bbar_m1[o] = V2<T>{(T(1) - w) * b.a, (T(1) - w) * b.b};
+    const V2<T> b = bbar_m[(int64_t)iy * gm.nx + ix];
     v[0] = w * b.a;
     v[1] = w * b.b;
   });
 }
 
 // Sources Bx = -dy Jz + (Jy(i-1) - Jy(i+1))/2dz, By = dx Jz - (Jx(i-1) - Jx(i+1))/2dz,
-// transposed: res = L^-1 of the mixed B adjoints.
+// transposed: res = L^-1 of the mixed B adjoints.  A slice's first iteration writes the records that
+// only these add to (slice i-1's, the sum of the trial currents' adjoints), the others add.
 template <typename T>
 __global__ void k_adj_pc_post(const T* __restrict__ res, V4<T>* dcur, V4<T>* dprev, V2<T>* jbar, V2<T>* jbar_tot,
-                              Geom gm) {
+                              const V2<T>* __restrict__ bbar_m, V2<T>* bbar_m1, T w1, int first, Geom gm) {
+  pdl_trigger();
+  pdl_wait();
   const int ix = blockIdx.x * blockDim.x + threadIdx.x, iy = blockIdx.y;
   if (ix >= gm.nx) return;
   const int nx = gm.nx;
@@ -552,34 +565,38 @@ __global__ void k_adj_pc_post(const T* __restrict__ res, V4<T>* dcur, V4<T>* dpr
     jxn = a1 * i2z;
     jyn = -a0 * i2z;
   }
+  const V2<T> b = bbar_m[o];
+  bbar_m1[o] = V2<T>{w1 * b.a, w1 * b.b};
   dcur[o].d += jz;
-  dprev[o].b += jxp;
-  dprev[o].c += jyp;
   jbar[o] = V2<T>{jxn, jyn};
-  const V2<T> t = jbar_tot[o];
-  jbar_tot[o] = V2<T>{t.a + jxn, t.b + jyn};
-}
-
-// Guess B^0 = 2 B(i-1) - B(i-2): carries for the two previous slices.
-template <typename T>
-__global__ void k_adj_guess(const V2<T>* __restrict__ b0, V2<T>* c1, V2<T>* c2, int64_t nn) {
-  const int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= nn) return;
-  const V2<T> b = b0[o];
-  if (c1) { c1[o].a += T(2) * b.a; c1[o].b += T(2) * b.b; }
-  if (c2) { c2[o].a -= b.a; c2[o].b -= b.b; }
+  if (first) {
+    dprev[o] = V4<T>{T(0), jxp, jyp, T(0)};
+    jbar_tot[o] = V2<T>{jxn, jyn};
+  } else {
+    dprev[o].b += jxp;
+    dprev[o].c += jyp;
+    const V2<T> t = jbar_tot[o];
+    jbar_tot[o] = V2<T>{t.a + jxn, t.b + jyn};
+  }
 }
 
 // psi_bar = Dx tbar0 + Dy tbar1 (ExmBy = -Dx psi, EypBx = -Dy psi), with Ez_bar, Bz_bar: tbar
 // holds the adjoints of the gathered ExmBy, EypBx, Ez, Bz (witness, final and trial passes).
+// Also the guess B^0 = 2 B(i-1) - B(i-2): carries for the two previous slices.
 template <typename T, typename Sink>
-__global__ void k_adj_main_pre(const T* __restrict__ tbar, const T* __restrict__ seed_psi, Geom gm, Sink sink) {
+__global__ void k_adj_main_pre(const T* __restrict__ tbar, const T* __restrict__ seed_psi, const V2<T>* __restrict__ b0,
+                               V2<T>* c1, V2<T>* c2, Geom gm, Sink sink) {
+  pdl_trigger();
+  pdl_wait();
   const int nx = gm.nx;
   auto f0 = [&](int y, int x) { return tbar[((int64_t)y * nx + x) * 4 + 0]; };
   auto f1 = [&](int y, int x) { return tbar[((int64_t)y * nx + x) * 4 + 1]; };
   visit_nodes<3, T>(gm, sink, 3, [&](int iy, int ix, T* v) {
     const int64_t o = (int64_t)iy * nx + ix;
     v[0] = v[1] = v[2] = T(0);
+    const V2<T> b = b0[o];
+    if (c1) { c1[o].a += T(2) * b.a; c1[o].b += T(2) * b.b; }
+    if (c2) { c2[o].a -= b.a; c2[o].b -= b.b; }
     if (ix > 0 && iy > 0) {
       v[0] = dxc(f0, iy, ix, nx, gsel<T>(gm.inv2dx, gm.f_inv2dx)) + dyc(f1, iy, ix, gm.ny, gsel<T>(gm.inv2dy, gm.f_inv2dy));
       if (seed_psi) v[0] += seed_psi[o];   // the caller's dL/dpsi of this slice
@@ -593,6 +610,8 @@ __global__ void k_adj_main_pre(const T* __restrict__ tbar, const T* __restrict__
 // tbar of this slice is consumed: cleared for the next slice.
 template <typename T>
 __global__ void k_adj_main_post(const T* __restrict__ res, V4<T>* dcur, T* rho_ion_bar, V4<T>* tbar, Geom gm) {
+  pdl_trigger();
+  pdl_wait();
   const int ix = blockIdx.x * blockDim.x + threadIdx.x, iy = blockIdx.y;
   if (ix >= gm.nx) return;
   const int nx = gm.nx;
@@ -650,6 +669,8 @@ template <int P, typename T>
 __global__ void k_adj_beam(hq_beam_view v, const int32_t* __restrict__ off, const int32_t* __restrict__ perm, int slice,
                            int nz, Geom gm, const V4<T>* __restrict__ dcur, const V2<T>* __restrict__ jtot,
                            double* wbar) {
+  pdl_trigger();
+  pdl_wait();
   const int a0 = off[slice], a1 = off[slice + 1];
   const int b0 = slice + 1 < nz ? off[slice + 1] : 0, b1 = slice + 1 < nz ? off[slice + 2] : 0;
   const int na = a1 - a0, nb = b1 - b0;
@@ -677,6 +698,8 @@ template <int P, typename T>
 __global__ void k_adj_witness(hq_beam_view v, const int32_t* __restrict__ off, const int32_t* __restrict__ perm,
                               int slice, Geom gm, const T* __restrict__ gf, double sb0, double sb1, double sb2, T* tbar,
                               double* wbar) {
+  pdl_trigger();
+  pdl_wait();
   const int a0 = off[slice], a1 = off[slice + 1];
   for (int t = a0 + blockIdx.x * blockDim.x + threadIdx.x; t < a1; t += gridDim.x * blockDim.x) {
     const int p = perm[t];
@@ -783,7 +806,7 @@ template <typename T>
 void launch_adj_final(const hq_grid_s* g, const SnapView<T>& s, const void* gf, int slice, const void* dbar_next,
                       const AdjView<T>& a, void* tbar, void* fbar_b, double* wbar_p, cudaStream_t st) {
   HQ_SHAPE_SWITCH(g->d.shape_order,
-                  (k_adj_final<P, T><<<blocks_for(s.n), kThreads, 0, st>>>(
+                  (launch_pdl(k_adj_final<P, T>, blocks_for(s.n), kThreads, 0, st,
                       s, reinterpret_cast<const T*>(gf), g->geom, slice, g->d.psi_guard,
                       reinterpret_cast<const V4<T>*>(dbar_next), a, reinterpret_cast<T*>(tbar),
                       reinterpret_cast<V2<T>*>(fbar_b), wbar_p)));
@@ -793,41 +816,38 @@ void launch_adj_trial(const hq_grid_s* g, const SnapView<T>& s, const void* gf, 
                       const void* jbar, const AdjView<T>& a, void* tbar, void* bbar_m1, double* wbar_p,
                       cudaStream_t st) {
   HQ_SHAPE_SWITCH(g->d.shape_order,
-                  (k_adj_trial<P, T><<<blocks_for(s.n), kThreads, 0, st>>>(
+                  (launch_pdl(k_adj_trial<P, T>, blocks_for(s.n), kThreads, 0, st,
                       s, reinterpret_cast<const T*>(gf), reinterpret_cast<const V2<T>*>(bm), g->geom, slice,
                       g->d.psi_guard, reinterpret_cast<const V2<T>*>(jbar), a, reinterpret_cast<T*>(tbar),
                       reinterpret_cast<V2<T>*>(bbar_m1), wbar_p)));
 }
 template <typename T>
 void launch_adj_bstart(const hq_grid_s* g, void* fbar_b, void* carry, void* bbar_n, cudaStream_t st) {
-  k_adj_bstart<T><<<blocks_for(g->nnode), kThreads, 0, st>>>(reinterpret_cast<V2<T>*>(fbar_b),
-                                                           reinterpret_cast<V2<T>*>(carry),
-                                                           reinterpret_cast<V2<T>*>(bbar_n), g->nnode);
+  launch_pdl(k_adj_bstart<T>, blocks_for(g->nnode), kThreads, 0, st, reinterpret_cast<V2<T>*>(fbar_b),
+             reinterpret_cast<V2<T>*>(carry), reinterpret_cast<V2<T>*>(bbar_n), g->nnode);
 }
 template <typename T>
-void launch_adj_pc_pre(const hq_grid_s* g, const void* bbar_m, void* bbar_m1, cudaStream_t st) {
+void launch_adj_pc_pre(const hq_grid_s* g, const void* bbar_m, cudaStream_t st) {
   with_sink<T>(g, [&](auto sink) {
-    k_adj_pc_pre<T, decltype(sink)><<<src_grid(g), 128, 0, st>>>(
-        reinterpret_cast<const V2<T>*>(bbar_m), reinterpret_cast<V2<T>*>(bbar_m1), T(g->d.pc_mix), g->geom, sink);
+    launch_pdl(k_adj_pc_pre<T, decltype(sink)>, src_grid(g), 128, 0, st, reinterpret_cast<const V2<T>*>(bbar_m),
+               T(g->d.pc_mix), g->geom, sink);
   });
 }
 template <typename T>
-void launch_adj_pc_post(const hq_grid_s* g, void* dcur, void* dprev, void* jbar, void* jtot, cudaStream_t st) {
-  k_adj_pc_post<T><<<grid2d(g), 128, 0, st>>>(reinterpret_cast<const T*>(g->solved), reinterpret_cast<V4<T>*>(dcur),
-                                             reinterpret_cast<V4<T>*>(dprev), reinterpret_cast<V2<T>*>(jbar),
-                                             reinterpret_cast<V2<T>*>(jtot), g->geom);
+void launch_adj_pc_post(const hq_grid_s* g, void* dcur, void* dprev, void* jbar, void* jtot, const void* bbar_m,
+                        void* bbar_m1, int first, cudaStream_t st) {
+  launch_pdl(k_adj_pc_post<T>, grid2d(g), 128, 0, st, reinterpret_cast<const T*>(g->solved),
+             reinterpret_cast<V4<T>*>(dcur), reinterpret_cast<V4<T>*>(dprev), reinterpret_cast<V2<T>*>(jbar),
+             reinterpret_cast<V2<T>*>(jtot), reinterpret_cast<const V2<T>*>(bbar_m), reinterpret_cast<V2<T>*>(bbar_m1),
+             T(1) - T(g->d.pc_mix), first, g->geom);
 }
 template <typename T>
-void launch_adj_guess(const hq_grid_s* g, const void* b0, void* c1, void* c2, cudaStream_t st) {
-  k_adj_guess<T><<<blocks_for(g->nnode), kThreads, 0, st>>>(reinterpret_cast<const V2<T>*>(b0),
-                                                          reinterpret_cast<V2<T>*>(c1), reinterpret_cast<V2<T>*>(c2),
-                                                          g->nnode);
-}
-template <typename T>
-void launch_adj_main_pre(const hq_grid_s* g, const void* tbar, const void* seed_psi, cudaStream_t st) {
+void launch_adj_main_pre(const hq_grid_s* g, const void* tbar, const void* seed_psi, const void* b0, void* c1, void* c2,
+                         cudaStream_t st) {
   with_sink<T>(g, [&](auto sink) {
-    k_adj_main_pre<T, decltype(sink)><<<src_grid(g), 128, 0, st>>>(reinterpret_cast<const T*>(tbar),
-                                                                   reinterpret_cast<const T*>(seed_psi), g->geom, sink);
+    launch_pdl(k_adj_main_pre<T, decltype(sink)>, src_grid(g), 128, 0, st, reinterpret_cast<const T*>(tbar),
+               reinterpret_cast<const T*>(seed_psi), reinterpret_cast<const V2<T>*>(b0), reinterpret_cast<V2<T>*>(c1),
+               reinterpret_cast<V2<T>*>(c2), g->geom, sink);
   });
 }
 
@@ -872,27 +892,24 @@ void launch_adj_seed(const hq_grid_s* g, const hq_field_out& sd, int slice, void
 }
 template <typename T>
 void launch_adj_main_post(const hq_grid_s* g, void* dcur, void* rho_ion_bar, void* tbar, cudaStream_t st) {
-  k_adj_main_post<T><<<grid2d(g), 128, 0, st>>>(reinterpret_cast<const T*>(g->solved), reinterpret_cast<V4<T>*>(dcur),
-                                               reinterpret_cast<T*>(rho_ion_bar), reinterpret_cast<V4<T>*>(tbar),
-                                               g->geom);
+  launch_pdl(k_adj_main_post<T>, grid2d(g), 128, 0, st, reinterpret_cast<const T*>(g->solved),
+             reinterpret_cast<V4<T>*>(dcur), reinterpret_cast<T*>(rho_ion_bar), reinterpret_cast<V4<T>*>(tbar), g->geom);
 }
 template <typename T>
 void launch_adj_beam(const hq_grid_s* g, int b, const hq_beam_view& v, int slice, const void* dcur, const void* jtot,
                      double* wbar, cudaStream_t st) {
   const BeamBins& bb = g->bins[b];
   HQ_SHAPE_SWITCH(g->d.shape_order,
-                  (k_adj_beam<P, T><<<kSliceBlocks, kThreads, 0, st>>>(v, bb.offset, bb.perm, slice, g->nz, g->geom,
-                                                                       reinterpret_cast<const V4<T>*>(dcur),
-                                                                       reinterpret_cast<const V2<T>*>(jtot), wbar)));
+                  (launch_pdl(k_adj_beam<P, T>, kSliceBlocks, kThreads, 0, st, v, bb.offset, bb.perm, slice, g->nz,
+                              g->geom, reinterpret_cast<const V4<T>*>(dcur), reinterpret_cast<const V2<T>*>(jtot), wbar)));
 }
 template <typename T>
 void launch_adj_witness(const hq_grid_s* g, int b, const hq_beam_view& v, int slice, const void* gf, const double* sb,
                         void* tbar, double* wbar, cudaStream_t st) {
   const BeamBins& bb = g->bins[b];
   HQ_SHAPE_SWITCH(g->d.shape_order,
-                  (k_adj_witness<P, T><<<kSliceBlocks, kThreads, 0, st>>>(v, bb.offset, bb.perm, slice, g->geom,
-                                                                          reinterpret_cast<const T*>(gf), sb[0], sb[1],
-                                                                          sb[2], reinterpret_cast<T*>(tbar), wbar)));
+                  (launch_pdl(k_adj_witness<P, T>, kSliceBlocks, kThreads, 0, st, v, bb.offset, bb.perm, slice, g->geom,
+                              reinterpret_cast<const T*>(gf), sb[0], sb[1], sb[2], reinterpret_cast<T*>(tbar), wbar)));
 }
 template <typename T>
 void launch_adj_init(const hq_grid_s* g, const void* d0, const void* rho_ion_bar, double* wbar_p, cudaStream_t st) {
@@ -914,11 +931,12 @@ void launch_adj_params(const hq_grid_s* g, const double* wbar_p, double* dn0, do
   template void launch_adj_trial<T>(const hq_grid_s*, const SnapView<T>&, const void*, const void*, int, const void*, \
                                     const AdjView<T>&, void*, void*, double*, cudaStream_t);                         \
   template void launch_adj_bstart<T>(const hq_grid_s*, void*, void*, void*, cudaStream_t);                           \
-  template void launch_adj_pc_pre<T>(const hq_grid_s*, const void*, void*, cudaStream_t);                            \
-  template void launch_adj_pc_post<T>(const hq_grid_s*, void*, void*, void*, void*, cudaStream_t);                   \
-  template void launch_adj_guess<T>(const hq_grid_s*, const void*, void*, void*, cudaStream_t);                      \
-  template void launch_adj_main_pre<T>(const hq_grid_s*, const void*, const void*, cudaStream_t);                    \
-  template void launch_adj_seed<T>(const hq_grid_s*, const hq_field_out&, int, void*, void*, void*, cudaStream_t);    \
+  template void launch_adj_pc_pre<T>(const hq_grid_s*, const void*, cudaStream_t);                                   \
+  template void launch_adj_pc_post<T>(const hq_grid_s*, void*, void*, void*, void*, const void*, void*, int,        \
+                                      cudaStream_t);                                                                 \
+  template void launch_adj_main_pre<T>(const hq_grid_s*, const void*, const void*, const void*, void*, void*,       \
+                                       cudaStream_t);                                                                \
+  template void launch_adj_seed<T>(const hq_grid_s*, const hq_field_out&, int, void*, void*, void*, cudaStream_t);   \
   template void launch_adj_main_post<T>(const hq_grid_s*, void*, void*, void*, cudaStream_t);                        \
   template void launch_adj_beam<T>(const hq_grid_s*, int, const hq_beam_view&, int, const void*, const void*,        \
                                    double*, cudaStream_t);                                                           \

@@ -186,3 +186,19 @@ def test_explicit_sizes(hq, precision, nx, ny, nz, iters):
         dev = rel(out[k], ref.fields[k])
         print(f"{precision} {nx}x{ny} {iters} iterations {k}: {dev:.1e}")
         assert dev <= (1e-9 if precision == "fp64" else 1e-3), k
+
+
+@pytest.mark.parametrize("precision,iters", [("fp64", 0), ("fp64", 1), ("fp64", 3), ("fp32", 1)])
+def test_adjoint_iterations(hq, precision, iters):
+    """Gradients with no, one and several predictor-corrector iterations (the reverse sweep's first
+    iteration of a slice writes records that the others add to; none leaves them to be cleared), at the
+    bars of the adjoint tests."""
+    from test_gpu_adjoint import case, gpu_grads, oracle_grads
+    g, d, w = case(nz=16)
+    g["n_pc_iter"] = iters
+    ref = oracle_grads(g, d, w, "mean")
+    got = gpu_grads(hq, g, d, w, "mean", precision, 5)
+    tol = 1e-5 if precision == "fp64" else 1e-3
+    errs = [rel(got[1], ref[1]), rel(got[2], ref[2]), abs(got[3] - ref[3]) / abs(ref[3]), rel(got[4], ref[4])]
+    print(precision, iters, [f"{e:.1e}" for e in errs])
+    assert max(errs) <= tol
