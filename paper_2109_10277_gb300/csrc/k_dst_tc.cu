@@ -2091,12 +2091,25 @@ template <typename K> struct Sized {   // a kernel, its shared memory and where 
 template <typename K> Sized(K, int, int*) -> Sized<K>;
 template <int BN, int MODE, bool RES> auto* cl_kernel() { return &k_dst_solve_cl<BN, MODE, RES>; }
 
+// No two CTAs of solve kernels may share an SM, of one launch or of launches on different streams: most
+// of them allocate all of tensor memory and then wait for other CTAs, so that two launches could each
+// hold what the other waits for.  Each takes more than half an SM's registers or shared memory.
+template <typename K> bool alone_on_sm(K kern, int threads, int smem) {
+  cudaFuncAttributes fa;
+  if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return 2 * fa.numRegs * threads > 65536 || 2 * smem > 228 * 1024;
+}
+
 // Right-hand sides whose clusters fit the GPU at once (0: none).
 template <int BN, int MODE, bool RES> int cl_capacity(int* most = nullptr) {
   using C = Cl<BN, MODE>;
   auto kern = cl_kernel<BN, MODE, RES>();
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::BYTES) != cudaSuccess ||
-      cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+      cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      !alone_on_sm(kern, kClThreads, C::BYTES)) {
     cudaGetLastError();
     return 0;
   }
@@ -2144,7 +2157,8 @@ int dst_tc_init(hq_grid_s* g, std::string& err) {
   auto size_solve = [&](auto kern, int smem, int& ctas, int threads = kSolveThreads) {
     int per_sm = 0;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess || per_sm < 1) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess || per_sm < 1 ||
+        !alone_on_sm(kern, threads, smem)) {
       err = "cannot size the cooperative DST solve";
       return false;
     }
