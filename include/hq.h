@@ -32,7 +32,8 @@
  *   HQ_NO_FOLD=1   FP32 DST-I without the folded (half-K) products
  *   HQ_SOLVE_BN=64 FP32 solves always on 128 x 64 tiles (no 128 x 32 tiles)
  *   HQ_NO_RS=1     FP32 square grids of 256 or 512 cells: the solve streams the fold matrix
- *                  per tile instead of keeping each CTA's slice of it in tensor memory; also as HQ_NO_CLUSTER=1
+ *                  per tile instead of keeping each CTA's slice of it in tensor memory; also as
+ *                  HQ_NO_CLUSTER=1
  *   HQ_NO_CLUSTER=1  FP32 (bf16x3) grids of up to 128 x 128 and of 256 x 256 cells: the solve's
  *                  operands go through global memory between all its products (by default
  *                  through the shared memory of a thread-block cluster where they can)
