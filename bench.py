@@ -39,7 +39,8 @@ CLOCK_QUERY = ("index,clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.ac
                "clocks_event_reasons.hw_slowdown,clocks_event_reasons.hw_thermal_slowdown,"
                "clocks_event_reasons.sw_thermal_slowdown,clocks_event_reasons.sw_power_cap")
 # algorithmic bytes per particle of the FP32 particle passes (particle streams read + written)
-BYTES_TRIAL = 49    # ux, uy, w (12) + AB5 history sum (20) + cell/frac/1+Psi cache (16) + alive (1)
+BYTES_TRIAL = 49    # mean of five: the first reads ux, uy, w (12), AB5 history sum (20), cell/frac/1+Psi cache (16),
+                    # alive (1) and writes the trial cache (36) and the gathered fields (16); the others read the cache
 BYTES_FINAL = 221   # reads: x, y, Psi (24), ux, uy, w (12), AB5 history 4x5x4 (80), cache (16), alive (1);
                     # writes: x, y, Psi (24), ux, uy (8), f_i (20), history sum (20), cache (16)
 
@@ -205,8 +206,8 @@ def run_reference(args):
 # (profiles/: k_dst_solve_rs R = 3, R = 2 of the first and of the later predictor-corrector
 # iterations weighted 1:1:4 as in a slice; the trial pass's first and later iterations 1:4;
 # the final pass)
-NCU_TRAFFIC = {"dst": (6.902016e6 + 16.344832e6 + 4 * 7.961856e6) / 6, "trial": (21.229824e6 + 4 * 21.23648e6) / 5,
-               "final": 46.436608e6 + 4.096e3}
+NCU_TRAFFIC = {"dst": (6.911232e6 + 16.355072e6 + 4 * 7.967744e6) / 6, "trial": (21.232896e6 + 4 * 13.637312e6) / 5,
+               "final": 46.438144e6 + 118.784e3}
 
 
 def dst_flops_per_sweep(g: dict) -> float:
