@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "../../include/hq.h"
+#include "solve_order.h"
 
 namespace hq {
 
@@ -544,27 +545,6 @@ __device__ __forceinline__ void pc_residual_add(double* rs, double d2, double b2
     if (t != 0.0) atomicAdd(rs + 2 * lane + threadIdx.x, t);
   }
   __syncthreads();
-}
-
-// Folded DST-I order (Sec. 3.2 solver).  With S_jk = sin(pi j k / n),
-// S_{n-j,k} = -(-1)^k S_jk: odd k see only x_j + x_{n-j}, even k only x_j - x_{n-j},
-// so after folding the node pairs (j, n-j) every output needs n/2 terms.  The folded
-// solver keeps each grid index in "slot order", pair u on slots 2u, 2u+1: pairs
-// 0 .. n/4-1 are (1, n-1), (3, n-3), ...; pair n/4 is (0, n/2); the rest (2, n-2),
-// (4, n-4), ...  Slots 0 .. n/2-1 thus hold the odd indices.  n must be a multiple of 4.
-__host__ __device__ __forceinline__ void fold_pair(int u, int n, int& a, int& b) {
-  if (u < n / 4) {
-    a = 2 * u + 1;
-    b = n - a;
-  } else {
-    a = 2 * (u - n / 4);
-    b = a == 0 ? n / 2 : n - a;
-  }
-}
-__host__ __device__ __forceinline__ int fold_node(int s, int n) {
-  int a, b;
-  fold_pair(s >> 1, n, a, b);
-  return (s & 1) ? b : a;
 }
 
 }  // namespace hq

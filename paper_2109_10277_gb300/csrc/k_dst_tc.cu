@@ -935,8 +935,10 @@ __device__ __forceinline__ void fill_tmem(const uint4* __restrict__ f, int block
 // adjacent columns of one thread (no shuffle), and each thread stores its row of the next
 // operand as contiguous 16-byte runs.  The third product writes its rows in node order, so
 // the last one's output columns are consecutive x nodes.
-// Between the products a tile waits for its own producers only (dependency counters: the 16 tiles
-// that wrote its rows at n = 512) instead of a barrier of the whole grid.
+// Between the products a tile waits for its producers only instead of a barrier of the whole grid
+// (dependency counters, rs_wait: the 16 tiles of the slot block that wrote its rows at n = 512; for the
+// last product, whose rows are nodes and come from two or three slot blocks, all 64 of its right-hand
+// side).
 template <int BN> struct RsSmem {
   static constexpr int KB_MAX = 4;                          // folded K = n/2 <= 256
   static constexpr int STAGE = 2 * BN * BK * 2;             // X_hi + X_lo rows of one K block
@@ -1130,7 +1132,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
   const bool tiles = nt0 < NT;               // a CTA beyond the tiles only forms sources
   const int NTR = n / BN;                    // data-row tiles per right-hand side
   unsigned long long* ctr_src = a.gbar + 16; // [NTR]: source rows of a data tile formed
-  unsigned long long* ctr_p = ctr_src + 16 * NTR;   // [3][R][MB]: product p's rows of a slot block written
+  unsigned long long* ctr_p = ctr_src + 16 * NTR;   // [rs_counters]: rows of a product's output written
 
   if (threadIdx.x == 0) {
     for (const CUtensorMap* m : {&x0h, &x0l, &x1h, &x1l, &x2h, &x2l}) prefetch_map(m);
@@ -1181,14 +1183,15 @@ __global__ void __launch_bounds__(kClThreads, 1)
       const int c0 = nt * BN;
       if (warp == 0 && lane == 0) {
         // data-tile producer: the whole folded K of BN rows, one stage per 64-wide K block, once
-        // the rows' producers have reported (the source rows of the tile, or every data tile's
-        // product with the slot block that holds these rows)
+        // the rows' producers have reported (the source rows of the tile, or the tiles of the product
+        // before that wrote them: rs_wait)
         bool ok = true;
         const int r_ = c0 / n, row0 = c0 - r_ * n;
-        if (p > 0)
-          ok = dep_wait(ctr_p + 16 * (((p - 1) * a.R + r_) * MB + row0 / BM),
-                        (unsigned long long)NTR + (p == 1 && !a.pre ? (unsigned)a.barrier_skew : 0u), a.status, abort_f);
-        else if (a.pre)
+        if (p > 0) {
+          const RsWait w = rs_wait(p, a.R, MB, NTR, r_, row0);
+          ok = dep_wait(ctr_p + 16 * w.counter,
+                        (unsigned long long)w.target + (p == 1 && !a.pre ? (unsigned)a.barrier_skew : 0u), a.status, abort_f);
+        } else if (a.pre)
           ok = dep_wait(ctr_src + 16 * (row0 / BN), (unsigned long long)(BN / kSrcRows) + (unsigned)a.barrier_skew, a.status,
                         abort_f);
         for (int kb = 0; ok && kb < nk; ++kb) {
@@ -1251,7 +1254,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
       {
         float x[CH];
         tmem_ld_pair<BN, CH>(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(half * CH), x);
-        const int orow = p == 2 ? fold_node(s, n) : s;
+        const int orow = rs_out_row(p, s, n);
         if (mode == 3) {
           // predictor-corrector mixing into bm[node][r]: the tile goes through shared memory (the
           // drained stage ring) so that a warp updates consecutive nodes of one row
@@ -1274,7 +1277,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
       main_sync();
       tc_fence_after();
       if (*abort_f) break;
-      if (p < 3 && threadIdx.x == 0) dep_arrive(ctr_p + 16 * ((p * a.R + r) * MB + mb));
+      if (p < 3 && threadIdx.x == 0) dep_arrive(ctr_p + 16 * rs_arrival(p, a.R, MB, r, mb));
     }
     if (*abort_f) break;
   }
@@ -1285,7 +1288,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
   if (threadIdx.x == 0 && !*abort_f) {
     const unsigned long long seen = atomicAdd(a.gbar, 1ull);
     if (seen == gridDim.x - 1ull) {
-      for (int i = 0; i < NTR + 3 * a.R * MB; ++i) ctr_src[16 * i] = 0ull;
+      for (int i = 0; i < NTR + rs_counters(a.R, MB); ++i) ctr_src[16 * i] = 0ull;
       atomicExch(a.gbar, 0ull);
     }
   }
