@@ -660,6 +660,14 @@ __global__ void __launch_bounds__(kThreads) k_trial_lin4(TrialCache<float> tc, i
     k[1] = q.y * f;
     k[2] = q.z * f;
     k[3] = q.w * f;
+    // what a particle that does not deposit left in the cache need not be finite, and a zero weight or current
+    // would not keep it out of the window's sums
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+      if (idx[p].y == kNoTrial) {
+        e[p] = te[p] = a[p] = make_float2(0.0f, 0.0f);
+        k[p] = 0.0f;
+      }
   }
   // windows at the particles and at the trial positions, over the particles that deposit
   int gx = 1 << 20, gy = 1 << 20, tx = 1 << 20, ty = 1 << 20, gx1 = -2, gy1 = -2, tx1 = -2, ty1 = -2;
@@ -1156,7 +1164,8 @@ __global__ void __launch_bounds__(kThreads) k_deposit4(Plasma<float> pl, int64_t
   const float4 fx4 = reinterpret_cast<const float4*>(pl.fx)[g], fy4 = reinterpret_cast<const float4*>(pl.fy)[g];
   const float4 q4 = reinterpret_cast<const float4*>(pl.tc.qt)[g];
   const int cell[4] = {c4.x, c4.y, c4.z, c4.w};
-  const float fx[4] = {fx4.x, fx4.y, fx4.z, fx4.w}, fy[4] = {fy4.x, fy4.y, fy4.z, fy4.w}, ch[4] = {q4.x, q4.y, q4.z, q4.w};
+  const float fx[4] = {fx4.x, fx4.y, fx4.z, fx4.w}, fy[4] = {fy4.x, fy4.y, fy4.z, fy4.w};
+  float ch[4] = {q4.x, q4.y, q4.z, q4.w};
   float4 v[4];
   int ix[4], iy[4], gx = 1 << 20, gy = 1 << 20, gx1 = -2, gy1 = -2;
   float ex[4], ey[4];
@@ -1168,6 +1177,11 @@ __global__ void __launch_bounds__(kThreads) k_deposit4(Plasma<float> pl, int64_t
     if (live[p]) {
       gx = min(gx, ix[p]); gx1 = max(gx1, ix[p]);
       gy = min(gy, iy[p]); gy1 = max(gy1, iy[p]);
+    } else {
+      // a removed particle's values need not be finite (1 / (1 + Psi) of a step that landed on zero): a
+      // zero weight would not keep them out of the window's sums
+      v[p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      ch[p] = ex[p] = ey[p] = 0.0f;
     }
   }
   if (gx1 == -2) return;
@@ -1188,9 +1202,6 @@ __global__ void __launch_bounds__(kThreads) k_deposit4(Plasma<float> pl, int64_t
   for (int p = 0; p < 4; ++p) {
     window_weights<P>(ex[p], live[p] ? ix[p] - gx : 0, wx[p]);
     window_weights<P>(ey[p], live[p] ? iy[p] - gy : 0, wy[p]);
-    if (!live[p])
-#pragma unroll
-      for (int a = 0; a < W; ++a) wx[p][a] = 0.0f;
   }
 #pragma unroll
   for (int b = 0; b < W; ++b)
