@@ -47,7 +47,11 @@
  *   HQ_NO_F4CACHE=1  every predictor-corrector trial pass and the final pass evaluate everything
  *                  (by default the first trial pass of a slice keeps per particle what does
  *                  not depend on B_perp, and the later passes of the slice gather Bx, By alone:
- *                  the same values up to rounding)
+ *                  the same values up to rounding).  That
+ *                  takes 52 bytes of device memory per plasma particle in FP32 and 128 in FP64 (with
+ *                  the predictor-corrector), which are given up where they do not fit when the grid
+ *                  is created or when the library allocates later; set the switch where a caller's
+ *                  own allocations need them
  *   HQ_NO_SRCCACHE=1  FP32: every B_perp source phase of the predictor-corrector forms all its
  *                  terms from the records (by default the first iteration of a slice keeps
  *                  the part that does not depend on the trial J_perp, and the others add the

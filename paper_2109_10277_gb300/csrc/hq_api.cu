@@ -52,21 +52,58 @@ int64_t round_up(int64_t v, int64_t m) { return (v + m - 1) / m * m; }
 
 void adj_free(hq_grid_s* g);
 
-void free_all(hq_grid_s* g) {
+// The trial cache (HQ_NO_F4CACHE=0) is memory that the solver can do without, so it never makes an
+// allocation fail that would succeed without it: it is taken last when a grid is created, left out
+// when it does not fit, and given back when a later allocation of the library does not.
+void free_trial_cache(hq_grid_s* g) {
   auto F = [](void* p) { if (p) cudaFree(p); };
   auto free_tc = [&](auto& t) {
     F(t.idx); F(t.e); F(t.te); F(t.a); F(t.qt); F(t.f4); F(t.rate); F(t.tg); F(t.tx); F(t.ty); F(t.tpsi);
+    t = {};
   };
+  free_tc(g->p64.tc);
+  free_tc(g->p32.tc);
+}
+// Bytes per particle: FP32 52, FP64 128.
+void alloc_trial_cache(hq_grid_s* g) {
+  const size_t np = (size_t)g->np;
+  auto alloc_tc = [&](auto& t, size_t z) {
+    bool ok = dalloc(&t.idx, 8 * np) == cudaSuccess && dalloc(&t.e, 2 * z * np) == cudaSuccess &&
+              dalloc(&t.te, 2 * z * np) == cudaSuccess && dalloc(&t.a, 2 * z * np) == cudaSuccess &&
+              dalloc(&t.qt, z * np) == cudaSuccess;
+    if (z == 4) return ok && dalloc(&t.f4, 16 * np) == cudaSuccess;
+    return ok && dalloc(&t.rate, 32 * np) == cudaSuccess && dalloc(&t.tg, z * np) == cudaSuccess &&
+           dalloc(&t.tx, 8 * np) == cudaSuccess && dalloc(&t.ty, 8 * np) == cudaSuccess &&
+           dalloc(&t.tpsi, 8 * np) == cudaSuccess;
+  };
+  if (g->fp64 ? alloc_tc(g->p64.tc, 8) : alloc_tc(g->p32.tc, 4)) return;
+  cudaGetLastError();
+  free_trial_cache(g);
+  g->no_f4 = 1;
+}
+// Gives the trial cache back (false: there is none); every pass evaluates everything from then on.
+bool release_trial_cache(hq_grid_s* g) {
+  cudaGetLastError();
+  if (!g->p64.tc.idx && !g->p32.tc.idx) return false;
+  cudaStreamSynchronize(g->stream);   // (a sweep's second stream is joined to it)
+  graph_free(g);
+  free_trial_cache(g);
+  g->no_f4 = 1;
+  g->f4_slice = -1;
+  return true;
+}
+
+void free_all(hq_grid_s* g) {
+  auto F = [](void* p) { if (p) cudaFree(p); };
+  free_trial_cache(g);
   for (hq::Plasma<double>* p : {&g->p64}) {
     F(p->x); F(p->y); F(p->psi); F(p->ux); F(p->uy); F(p->w); F(p->alive); F(p->hist);
-    free_tc(p->tc);
   }
   {
     hq::Plasma<float>& p = g->p32;
     if (!g->fp64) {
       // x, y, psi, alive are shared with p64 storage (freed above); free the typed arrays
       F(p.ux); F(p.uy); F(p.w); F(p.hist); F(p.cell); F(p.fx); F(p.fy); F(p.opp); F(p.hsum);
-      free_tc(p.tc);
     }
   }
   if (g->det_arena) {
@@ -429,7 +466,7 @@ hq_status check_launch(hq_grid_s* g) {
 
 
 // ---------------------------------------------------------------- checkpointed forward and adjoint
-hq_status adj_alloc(hq_grid_s* g, int k) {
+hq_status adj_alloc_once(hq_grid_s* g, int k) {
   AdjStore* a = adj_of(g);
   if (a && a->k == k) return HQ_OK;
   adj_free(g);
@@ -480,6 +517,11 @@ hq_status adj_alloc(hq_grid_s* g, int k) {
   }
   return HQ_OK;
 }
+hq_status adj_alloc(hq_grid_s* g, int k) {
+  hq_status st = adj_alloc_once(g, k);
+  if (st == HQ_ERR_OOM && release_trial_cache(g)) st = adj_alloc_once(g, k);
+  return st;
+}
 
 void ckpt_copy(hq_grid_s* g, int seg, bool save) {
   AdjStore* a = adj_of(g);
@@ -502,18 +544,29 @@ void ckpt_copy(hq_grid_s* g, int seg, bool save) {
   }
 }
 
+// Bin storage for n particles.
+hq_status bins_alloc(hq_grid_s* g, BeamBins& bb, int64_t n) {
+  if (bb.cap >= n) return HQ_OK;
+  if (bb.bin) cudaFree(bb.bin);
+  if (bb.perm) cudaFree(bb.perm);
+  bb.bin = bb.perm = nullptr;
+  bb.cap = 0;
+  auto get = [&](int32_t** p) {
+    cudaError_t e = dalloc(p, sizeof(int32_t) * n);
+    if (e == cudaErrorMemoryAllocation && release_trial_cache(g)) e = dalloc(p, sizeof(int32_t) * n);
+    return e;
+  };
+  HQ_CUDA(g, get(&bb.bin));
+  HQ_CUDA(g, get(&bb.perm));
+  bb.cap = n;
+  return HQ_OK;
+}
+
 // Binds view `v` to bin slot k: counting sort of its particles by slice at their current zeta.
 hq_status bind_view(hq_grid_s* g, int k, const hq_beam_view& v) {
   BeamBins& bb = g->bins[k];
-  if (bb.cap < v.n) {
-    if (bb.bin) cudaFree(bb.bin);
-    if (bb.perm) cudaFree(bb.perm);
-    bb.bin = bb.perm = nullptr;
-    bb.cap = 0;
-    HQ_CUDA(g, dalloc(&bb.bin, sizeof(int32_t) * v.n));
-    HQ_CUDA(g, dalloc(&bb.perm, sizeof(int32_t) * v.n));
-    bb.cap = v.n;
-  }
+  const hq_status st = bins_alloc(g, bb, v.n);
+  if (st != HQ_OK) return st;
   g->bound[k] = v;
   Prof p(g, HQ_K_BEAM, v.n > 0 ? 3 : 1);
   launch_beam_bin(g, k, v, g->stream);
@@ -817,15 +870,8 @@ void graph_free(hq_grid_s* g) {
 // Beam bin storage for the beams of a sweep, allocated ahead of a stream capture.
 hq_status reserve_bins(hq_grid_s* g, const hq_beam_view* beams, int nb) {
   for (int b = 0; b < nb; ++b) {
-    BeamBins& bb = g->bins[b];
-    if (bb.cap >= beams[b].n) continue;
-    if (bb.bin) cudaFree(bb.bin);
-    if (bb.perm) cudaFree(bb.perm);
-    bb.bin = bb.perm = nullptr;
-    bb.cap = 0;
-    HQ_CUDA(g, dalloc(&bb.bin, sizeof(int32_t) * beams[b].n));
-    HQ_CUDA(g, dalloc(&bb.perm, sizeof(int32_t) * beams[b].n));
-    bb.cap = beams[b].n;
+    const hq_status st = bins_alloc(g, g->bins[b], beams[b].n);
+    if (st != HQ_OK) return st;
   }
   return HQ_OK;
 }
@@ -1013,21 +1059,6 @@ hq_status hq_grid_create(const hq_grid_desc* desc, void* cuda_stream, hq_grid_t*
   }
   const char* nf4 = std::getenv("HQ_NO_F4CACHE");
   g->no_f4 = nf4 && nf4[0] == '1';
-  if (!g->explicit_b && !g->no_f4 && d.n_pc_iter > 0) {
-    auto alloc_tc = [&](auto& t, size_t z) -> hq_status {
-      HQ_ALLOC(t.idx, 8 * np); HQ_ALLOC(t.e, 2 * z * np); HQ_ALLOC(t.te, 2 * z * np); HQ_ALLOC(t.a, 2 * z * np);
-      HQ_ALLOC(t.qt, z * np);
-      if (z == 4) {
-        HQ_ALLOC(t.f4, 16 * np);
-      } else {
-        HQ_ALLOC(t.rate, 32 * np);
-        HQ_ALLOC(t.tg, z * np); HQ_ALLOC(t.tx, 8 * np); HQ_ALLOC(t.ty, 8 * np); HQ_ALLOC(t.tpsi, 8 * np);
-      }
-      return HQ_OK;
-    };
-    const hq_status st = g->fp64 ? alloc_tc(g->p64.tc, 8) : alloc_tc(g->p32.tc, 4);
-    if (st != HQ_OK) return st;   // (everything is freed)
-  }
   if (d.resort_every > 0) {
     HQ_ALLOC(g->porigin, 4 * np);
     g->p64.origin = g->p32.origin = g->porigin;
@@ -1304,6 +1335,7 @@ hq_status hq_grid_create(const hq_grid_desc* desc, void* cuda_stream, hq_grid_t*
       cudaMemcpy(g->c0, f.data(), 4 * nn, cudaMemcpyHostToDevice);
     }
   }
+  if (!g->explicit_b && !g->no_f4 && d.n_pc_iter > 0) alloc_trial_cache(g);
   cudaError_t e = cudaStreamSynchronize(g->stream);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
