@@ -21,6 +21,7 @@ thread_local std::string g_global_err;
 hq_status fail(hq_grid_s* g, hq_status st, const std::string& msg) {
   if (g) g->err = msg;
   else g_global_err = msg;
+  if (st == HQ_ERR_OOM || st == HQ_ERR_CUDA) cudaGetLastError();   // reported here, not again by the next call's check
   return st;
 }
 

@@ -99,3 +99,32 @@ def test_adjoint_takes_the_cache_back(hq):
     for a, b, c in zip(got, again, ref):
         assert float((a - c).abs().max()) <= 1e-9 * float(c.abs().max())
         assert float((b - c).abs().max()) <= 1e-9 * float(c.abs().max())
+
+
+def test_refused_allocation_is_reported_once(hq):
+    """A grid, and a reverse sweep's storage, that do not fit are refused with HQ_ERR_OOM; the calls after
+    that succeed once there is room."""
+    g = I.scaled_grid(I.grid_params("linear64"), 256, 256, 4, ppc_x=4, ppc_y=4, zeta_min=-0.2, zeta_max=0.2)
+    beam = hq.Beam(I.random_beam(2_000, 0.4, 0.4, 0.1, 0.5))
+    start = free_bytes()
+    grid = hq.Grid(g, precision="fp64")
+    need = start - free_bytes()
+    grid.close()
+    filler = leave(need // 4)
+    with pytest.raises(hq.HQError) as e:
+        hq.Grid(g, precision="fp64")
+    assert e.value.status == 3
+    del filler
+    torch.cuda.empty_cache()
+    grid = hq.Grid(g, precision="fp64")
+    sums = torch.zeros(3, dtype=torch.float64, device="cuda")
+    filler = leave(need // 2)
+    with pytest.raises(hq.HQError) as e:
+        grid.forward_ckpt([beam], 0, sums, 1)
+    assert e.value.status == 3
+    del filler
+    torch.cuda.empty_cache()
+    grid.sweep([beam])
+    grid.forward_ckpt([beam], 0, sums, 1)
+    assert grid.sync() == 0
+    grid.close()
