@@ -367,6 +367,14 @@ __global__ void __launch_bounds__(128, 1)
 // accumulator), and all 8 warps the epilogue, each warpgroup half of the columns.
 constexpr int kSolveThreads = 256;
 
+// No two CTAs of solve kernels may share an SM, of one launch or of launches on different streams: most
+// of them allocate all of tensor memory and then wait for other CTAs, so that two launches could each
+// hold what the other waits for.  Each therefore takes more than half of an SM's 228 KB of shared memory
+// (1 KB of it the system's, per CTA), whether it needs that much or not.
+constexpr int kAloneBytes = 116 * 1024;
+constexpr int alone_bytes(int need) { return need > kAloneBytes ? need : kAloneBytes; }
+static_assert(2 * (kAloneBytes + 1024) > 228 * 1024, "two solve CTAs would fit one SM");
+
 // The caller's sources [nr][ny][nx] (hq_poisson_solve); row and column 0 read zero.
 struct SrcGiven {
   static constexpr int NR = kMaxRhs;
@@ -617,7 +625,7 @@ template <int BN> struct SolveSmem {
   static constexpr int RING = STAGES * Cfg<BN>::STAGE_BYTES;
   static constexpr int SCALE = RING;
   static constexpr int BARS = SCALE + BN * BM * 4;
-  static constexpr int BYTES = BARS + 256 + 1024 /*alignment*/;
+  static constexpr int BYTES = alone_bytes(BARS + 256 + 1024 /*alignment*/);
 };
 
 template <int BN, bool RES, typename E>
@@ -945,7 +953,7 @@ template <int BN> struct RsSmem {
   static constexpr int RING = 0;
   static constexpr int TILE = BM * (BN + 1) * 4;            // the mixing's staged tile
   static constexpr int BARS = KB_MAX * STAGE > TILE ? KB_MAX * STAGE : TILE;
-  static constexpr int BYTES = BARS + 256 + 1024 /*alignment*/;
+  static constexpr int BYTES = alone_bytes(BARS + 256 + 1024 /*alignment*/);
   static constexpr uint32_t TX = 128;                       // tensor-memory columns: accumulator (2 BN), F slice
 };
 
@@ -1336,7 +1344,7 @@ template <int BN, int MODE> struct Cl {
   // MODE 1: kSrcRows rows of R x 256 floats (apart from the data buffers: a peer may already exchange)
   static constexpr int SRC = DATA + DATA_BYTES, SRC_BYTES = LOCAL ? (BN + kMaxRhs - 1) * 512 : kSrcRows * kMaxRhs * 1024;
   static constexpr int BARS = SRC + SRC_BYTES;
-  static constexpr int BYTES = BARS + 128 + 1024;
+  static constexpr int BYTES = alone_bytes(BARS + 128 + 1024);
   static constexpr uint32_t TX = 128, TY = TX + K;          // tensor-memory columns: accumulator, x slice, y slice
   // cluster barriers of a launch (each thread arrives at and waits for every one): the start, the
   // end of each exchange, and where a peer's buffer has to be drained first
@@ -1753,7 +1761,7 @@ template <typename E> struct Wide {
   static constexpr int BN = 128, STAGES = 3, STAGE_BYTES = 4 * A_BYTES;
   static constexpr int TILE = STAGES * STAGE_BYTES, LD = 65;   // the mixing's staged columns, 128 x 64
   static constexpr int BARS = TILE + BM * LD * 4;
-  static constexpr int BYTES = BARS + 256 + 1024;
+  static constexpr int BYTES = alone_bytes(BARS + 256 + 1024);
 };
 
 // 32 consecutive data columns i0 .. of slot s into the next operand's row: ns slots, nd data rows per
@@ -2094,25 +2102,12 @@ template <typename K> struct Sized {   // a kernel, its shared memory and where 
 template <typename K> Sized(K, int, int*) -> Sized<K>;
 template <int BN, int MODE, bool RES> auto* cl_kernel() { return &k_dst_solve_cl<BN, MODE, RES>; }
 
-// No two CTAs of solve kernels may share an SM, of one launch or of launches on different streams: most
-// of them allocate all of tensor memory and then wait for other CTAs, so that two launches could each
-// hold what the other waits for.  Each takes more than half an SM's registers or shared memory.
-template <typename K> bool alone_on_sm(K kern, int threads, int smem) {
-  cudaFuncAttributes fa;
-  if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return 2 * fa.numRegs * threads > 65536 || 2 * smem > 228 * 1024;
-}
-
 // Right-hand sides whose clusters fit the GPU at once (0: none).
 template <int BN, int MODE, bool RES> int cl_capacity(int* most = nullptr) {
   using C = Cl<BN, MODE>;
   auto kern = cl_kernel<BN, MODE, RES>();
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::BYTES) != cudaSuccess ||
-      cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-      !alone_on_sm(kern, kClThreads, C::BYTES)) {
+      cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -2160,8 +2155,7 @@ int dst_tc_init(hq_grid_s* g, std::string& err) {
   auto size_solve = [&](auto kern, int smem, int& ctas, int threads = kSolveThreads) {
     int per_sm = 0;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess || per_sm < 1 ||
-        !alone_on_sm(kern, threads, smem)) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess || per_sm < 1) {
       err = "cannot size the cooperative DST solve";
       return false;
     }
