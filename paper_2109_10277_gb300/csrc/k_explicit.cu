@@ -20,6 +20,7 @@
 #include <type_traits>
 
 #include "hq_internal.cuh"
+#include "pcg_scalars.h"
 
 namespace hq {
 
@@ -247,9 +248,7 @@ __global__ void k_pcg_init(PcgInit<T> f, Sink sink) {
 // that the node sums have to give: beta is not needed before they are complete.  Forming p first and
 // p.Ap from it took four passes (r.z; p; p.Ap; x and r) with a full drain between each two; at 256^2,
 // where a pass is launch and latency and not its bytes, a slice (six iterations) took 241 us with four
-// launches, 240 with one cooperative launch and three grid barriers, and takes 219 with two.  (The expanded form stays a
-// sum of squares: p'.Az is measured, not taken to be -beta p'.Ap', so that a residual at the rounding
-// floor cannot turn p.Ap negative by cancellation.)
+// launches, 240 with one cooperative launch and three grid barriers, and takes 219 with two.
 
 // First pass: the three sums.  Iteration 0 also clears the consumed source records.
 template <typename T>
@@ -323,12 +322,12 @@ template <typename T> struct PcgStep {
     __shared__ double ab[2][2];
     const int c = threadIdx.x;
     if (c < 2) {
-      const double rz = sums.out[0][c], b = p_old && rz_prev[c] != 0.0 ? rz / rz_prev[c] : 0.0;
-      double d = sums.out[1][c];
-      if (p_old) d += b * (2.0 * sums.out[2][c] + b * pq_prev[c]);
-      ab[0][c] = d != 0.0 ? rz / d : 0.0;
-      ab[1][c] = b;
-      if (keep) pq[c] = d;
+      // (the terms' rounding grows with A's condition: a direction 1e-4 of them in FP32, 1e-12 in FP64, is lost)
+      const PcgScalars t = pcg_scalars(!p_old, sums.out[0][c], sums.out[1][c], sums.out[2][c], p_old ? rz_prev[c] : 0.0,
+                                       p_old ? pq_prev[c] : 0.0, sizeof(T) == 8 ? 1e-12 : 1e-4);
+      ab[0][c] = t.alpha;
+      ab[1][c] = t.beta;
+      if (keep) pq[c] = t.pq;
     }
     __syncthreads();
 #pragma unroll
