@@ -322,9 +322,9 @@ template <typename T> struct PcgStep {
     __shared__ double ab[2][2];
     const int c = threadIdx.x;
     if (c < 2) {
-      // (the terms' rounding grows with A's condition: a direction 1e-4 of them in FP32, 1e-12 in FP64, is lost)
+      // (the terms' rounding grows with A's condition: a direction 2^-13 of them in FP32, 2^-40 in FP64, is lost)
       const PcgScalars t = pcg_scalars(!p_old, sums.out[0][c], sums.out[1][c], sums.out[2][c], p_old ? rz_prev[c] : 0.0,
-                                       p_old ? pq_prev[c] : 0.0, sizeof(T) == 8 ? 1e-12 : 1e-4);
+                                       p_old ? pq_prev[c] : 0.0, sizeof(T) == 8 ? 40 : 13);
       ab[0][c] = t.alpha;
       ab[1][c] = t.beta;
       if (keep) pq[c] = t.pq;
