@@ -1658,7 +1658,7 @@ hq_status hq_poisson_solve(hq_grid_t g, const void* src, void* dst, int32_t nrhs
   }
   {
     Prof p(g, HQ_K_FIELD, 1);
-    launch_src_copy<float>(g, src, nrhs, s);
+    launch_src_copy(g, static_cast<const float*>(src), nrhs, s);
   }
   dst_solve(g, nrhs);
   HQ_CUDA(g, cudaMemcpyAsync(dst, g->solved, (size_t)nrhs * g->nnode * g->tsize, cudaMemcpyDeviceToDevice, s));

@@ -333,7 +333,7 @@ template <typename T> void launch_src_main(const hq_grid_s* g, const void* dep, 
 // ion background (it receives the next slice's deposit)
 template <typename T> void launch_src_bperp(const hq_grid_s* g, const void* dep_cur, void* dep_prev, void* chi_prev,
                                             int reset_prev, cudaStream_t s);
-template <typename T> void launch_src_copy(const hq_grid_s* g, const void* src, int nrhs, cudaStream_t s);
+void launch_src_copy(const hq_grid_s* g, const float* src, int nrhs, cudaStream_t s);
 // finish_main also sets the B_perp guess 2 B(i-1) - B(i-2) (first: slice 0, B(-1) = 0) and
 // moves B(i-1) into bprev1
 template <typename T> void launch_finish_main(const hq_grid_s* g, const void* res, int first, cudaStream_t s);

@@ -42,11 +42,13 @@ __global__ void k_src_bperp(SrcBperp<T> src, Sink sink) {
   visit_nodes<2, T>(src.gm, sink, 2, src);
 }
 
-template <typename T, typename Sink>
-__global__ void k_src_copy(const T* __restrict__ src, int nrhs, Geom gm, Sink sink) {
-  visit_nodes<kMaxRhs, T>(gm, sink, nrhs, [&](int iy, int ix, T* v) {
+// The caller's sources (FP32 hq_poisson_solve into an array that is not 16-byte aligned, or with
+// HQ_SEPARATE_SRC=1; all other solves read them themselves).
+template <typename Sink>
+__global__ void k_src_copy(const float* __restrict__ src, int nrhs, Geom gm, Sink sink) {
+  visit_nodes<kMaxRhs, float>(gm, sink, nrhs, [&](int iy, int ix, float* v) {
     for (int r = 0; r < kMaxRhs; ++r)
-      v[r] = (r < nrhs && ix > 0 && iy > 0) ? src[((int64_t)r * gm.ny + iy) * gm.nx + ix] : T(0);
+      v[r] = (r < nrhs && ix > 0 && iy > 0) ? src[((int64_t)r * gm.ny + iy) * gm.nx + ix] : 0.0f;
   });
 }
 
@@ -161,11 +163,8 @@ void launch_src_bperp(const hq_grid_s* g, const void* cur, void* prev, void* chi
                src_bperp_of<T>(g, cur, prev, chi_prev, reset_prev), sink);
   });
 }
-template <typename T>
-void launch_src_copy(const hq_grid_s* g, const void* src, int nrhs, cudaStream_t s) {
-  with_sink<T>(g, [&](auto sink) {
-    k_src_copy<T, decltype(sink)><<<src_grid(g), 128, 0, s>>>(reinterpret_cast<const T*>(src), nrhs, g->geom, sink);
-  });
+void launch_src_copy(const hq_grid_s* g, const float* src, int nrhs, cudaStream_t s) {
+  with_sink<float>(g, [&](auto sink) { k_src_copy<<<src_grid(g), 128, 0, s>>>(src, nrhs, g->geom, sink); });
 }
 template <typename T>
 void launch_finish_main(const hq_grid_s* g, const void* res, int first, cudaStream_t s) {
@@ -215,7 +214,6 @@ void launch_fx_decode(const hq_grid_s* g, void* rec, int64_t n, double* dst, cud
   template void launch_reset_dep<T>(const hq_grid_s*, void*, void*, cudaStream_t);             \
   template void launch_src_main<T>(const hq_grid_s*, const void*, cudaStream_t);               \
   template void launch_src_bperp<T>(const hq_grid_s*, const void*, void*, void*, int, cudaStream_t); \
-  template void launch_src_copy<T>(const hq_grid_s*, const void*, int, cudaStream_t);          \
   template void launch_finish_main<T>(const hq_grid_s*, const void*, int, cudaStream_t);       \
   template void launch_finish_bperp<T>(const hq_grid_s*, const void*, cudaStream_t);           \
   template void launch_store<T>(const hq_grid_s*, const hq_field_out*, int64_t, const void*, const void*, cudaStream_t); \
