@@ -93,8 +93,8 @@ typedef enum {
      rounded to TF32, lo = the remainder, read by the tensor core truncated to TF32): ~21
      significant bits per operand against bf16x3's 16, at twice the operand bytes and twice
      the tensor-core instructions (K = 8 per instruction); every grid shape takes the solve
-     that streams the sine/fold matrices (the resident-matrix solve would need 256 KB of
-     shared memory at 512^2) */
+     that streams the sine/fold matrices (as TF32 words the matrix that the resident solve
+     keeps would fill tensor memory at 512^2) */
   HQ_PREC_FP32_TF32X3 = 2
 } hq_precision;
 

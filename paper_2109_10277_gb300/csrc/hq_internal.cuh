@@ -390,7 +390,8 @@ template <typename T> void launch_explicit_src(const hq_grid_s* g, cudaStream_t 
 template <typename T> void launch_pcg_init(const hq_grid_s* g, int slice, const void* cur, const void* chi_cur, void* prev,
                                            void* chi_prev, cudaStream_t s);
 // blocks of the PCG's sums (256 threads): two nodes per thread, so that the blocks' own sums cost less than the
-// nodes', and at most four blocks per SM
+// nodes', and at most four blocks for each of a GB300's 152 SMs (a constant: the deterministic mode's order of
+// summation, and so its result, is the same on every device)
 inline unsigned pcg_blocks(int64_t nn) { return (unsigned)std::min<int64_t>((nn + 511) / 512, 4 * 152); }
 template <typename T> void launch_pcg_iter(const hq_grid_s* g, int slice, int k, const void* chi_cur, cudaStream_t s);
 // adjoint (k_adjoint.cu)

@@ -2182,7 +2182,7 @@ int dst_tc_init(hq_grid_s* g, std::string& err) {
     return 1;
   const char* bn = std::getenv("HQ_SOLVE_BN");
   t.wide_only = bn != nullptr && std::atoi(bn) == 64;
-  // (the resident fold matrix is bf16: as TF32 words it would need 256 KB of shared memory at 512^2)
+  // (the resident fold matrix is bf16: as TF32 words, hi and lo, it would fill tensor memory at 512^2)
   t.rs = dst_tc_resident(g);
   auto size_rs = [&](auto... kern) { return (size_solve(kern.k, kern.smem, *kern.ctas, kClThreads) && ...); };
   if (t.rs && !(g->nx == 512 ? size_rs(Sized{rs_kernel<64, 512, false>(), RsSmem<64>::BYTES, &t.rs_ctas[0]},

@@ -582,9 +582,10 @@ template <int P, typename T, bool MS>
 __global__ void __launch_bounds__(kThreads) k_trial_lin(TrialCache<T> tc, int64_t n, Geom gm, const T* __restrict__ bm, V2<T>* tj, SpeciesTab tab) {
   pdl_trigger();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  // FP32: the launch before is the cooperative solve, which started after the trial pass that
-  // filled the cache had ended: the cache is read while that solve drains.  (The FP64 solve's
-  // launches overlap their predecessors: wait first.)
+  // FP32: the launch before is a solve, and no FP32 solve is launched early (none has the
+  // programmatic-serialization attribute): it started after the trial pass that filled the cache
+  // had ended, so the cache is read while that solve drains.  (The FP64 solve's launches overlap
+  // their predecessors: wait first; an FP32 solve launched early would need that here too.)
   if constexpr (sizeof(T) == 8) pdl_wait();
   const bool in = p < n;
   const int2 idx = in ? tc.idx[p] : make_int2(0, kNoTrial);
@@ -947,10 +948,10 @@ __device__ __forceinline__ void deposit_ion_src(float* ps, const Geom& gm, const
 // ---------------------------------------------------------------- final pass
 // Gather with the converged fields of slice i, store f_i in the AB5 history,
 // advance to slice i+1, apply the removal rule and deposit rho, J, chi there.
-// Resident CTAs the FP32 final pass is compiled for: the pass is memory-latency bound, and a
-// 48-register budget (64 for the cubic shape) keeps 30 % more warps resident than its unconstrained
-// 62 (70) registers allow: 3 % of the blowout512 sweep.  The linear shape would spill at 48: 56
-// (262144 particles: 32.6 -> 27.6 us).
+// Resident CTAs the FP32 final pass is compiled for: the pass is memory-latency bound, and a register
+// budget keeps more warps resident than its unconstrained 62 (cubic: 70) registers allow.  Quadratic
+// shape, 96 slices of 512^2: 21.85 ms at 48 registers (with 32 bytes of spills) and at 56 (without), 22.14
+// at 64.  Linear, 262144 particles: 32.6 us at 48, 27.6 at 56.  Cubic: 64.
 template <int P, typename T> constexpr int final_min_blocks() {
   return sizeof(T) == 4 ? 65536 / ((P == 3 ? 64 : P == 2 ? 48 : 56) * kThreads) : 1;
 }
