@@ -25,8 +25,8 @@
 // n <= 64 (dst_direct): the folded sums directly, one thread per output and row.  A 64 x 64 sweep
 // of 64 slices: 25.9 ms before, 19.3 ms with the fast transform, 11.1 ms with the direct sums.
 //
-// Other n: k_dst_gemm64, the sine sums as a tiled product over the folded pairs (x_j + x_{n-j}
-// for odd k, x_j - x_{n-j} for even k: half the terms).  The FP32 path uses tensor cores instead.
+// Other n: k_dst_sums64, the sine sums over the folded pairs (x_j + x_{n-j} for odd k,
+// x_j - x_{n-j} for even k: half the terms).  The FP32 path uses tensor cores instead.
 #include <atomic>
 
 #include "hq_internal.cuh"
@@ -148,7 +148,7 @@ __device__ __forceinline__ void dst_pair(double2* A, double2* B, const double2* 
 
 // n <= 64 (any n): the folded sine sums directly, one thread per output and row: the fast
 // transform would leave most lanes of its one warp idle and runs 4 times as long.  On return
-// B[k] = X_k.  T: tab (see k_dst_gemm64) in shared memory; tp >= 2 n threads.
+// B[k] = X_k.  T: tab (see k_dst_sums64) in shared memory; tp >= 2 n threads.
 __device__ __forceinline__ void dst_direct(double2* A, double2* B, const double* T, int n, int tid, int tp) {
   const int H = n >> 1, He = (n - 1) >> 1;
   for (int j = 1 + tid; j <= He; j += tp) {
@@ -332,69 +332,64 @@ __global__ void k_dst_rows(RowsArgs a, Load ld, Store st) {
 // ---------------------------------------------------------------- rows of any length
 // out[k] = sum_j in[j] sin(pi j k / n), folded: tab[0][j-1][i] = sin(pi j (2i+1) / n) weighs
 // x_j + x_{n-j} (x_{n/2} alone once), tab[1][j-1][i] = sin(pi j (2i+2) / n) weighs x_j - x_{n-j};
-// j = 1..H, H = n/2.  A CTA forms 32 rows x 64 outputs of one parity, 4 x 4 per thread.
-constexpr int GR = 32, GK = 64, GJ = 16;
-__global__ void __launch_bounds__(128) k_dst_gemm64(const double* __restrict__ in, double* __restrict__ out, int n, int M,
-                                                    const double* __restrict__ tab, const double* __restrict__ scale,
-                                                    int transposed) {
-  __shared__ double xs[GJ][GR + 2];
-  __shared__ double ts[GJ][GK];
-  pdl_trigger();
+// j = 1..H, H = n/2.  A warp forms 32 outputs of one parity of one row, a lane each: the table's
+// values are read along a row of it, those of the folded row from shared memory (one for all lanes).
+//
+// What bounds it: the FP64 pipe, which takes a warp's multiply-add in 16 clocks of an SM, so that a
+// multiply-add's two operands come fast enough without being kept for a second row, and what counts
+// is that the warps are spread evenly: tiles of 32 rows x 64 outputs (a block of 16 multiply-adds per
+// thread from registers) left most SMs idle up to 200 cells and the last wave nearly empty beyond, 2 and
+// 4 rows per warp are up to 1.7 and 2.5 times as slow as one and never more than 2 % faster.  Solves:
+//                                          100^2, 1 rhs  16 x 400, 1  400^2, 2  409^2, 3  1000^2, 1
+//   a thread per output, n terms                    54 us        134        2094      1439      10715
+//   the tiles                                      176           424        1570      2419       6567
+//   this kernel                                     23            36         536       826       3662
+constexpr int kSumRows = 4, kSumChunk = 256;   // rows (warps) of a block, folded terms staged at a time
+__global__ void __launch_bounds__(32 * kSumRows) k_dst_sums64(const double* __restrict__ in, double* __restrict__ out, int n,
+                                                              int M, const double* __restrict__ tab,
+                                                              const double* __restrict__ scale, int transposed) {
+  __shared__ alignas(16) double xs[kSumRows][kSumChunk];
   pdl_wait();
-  const int H = n / 2, nt = (H + GK - 1) / GK;
-  const int par = blockIdx.y / nt, i0 = (blockIdx.y - par * nt) * GK, m0 = blockIdx.x * GR, r = blockIdx.z;
-  const double* src = in + (int64_t)r * M * n;
-  const double* tb = tab + (int64_t)par * H * H;
-  const int tr = threadIdx.x & 7, tk = threadIdx.x >> 3;   // rows 4 tr.., outputs tk + 16 c
-  double acc[4][4];
-#pragma unroll
-  for (int x = 0; x < 4; ++x)
-#pragma unroll
-    for (int y = 0; y < 4; ++y) acc[x][y] = 0.0;
-  for (int j0 = 0; j0 < H; j0 += GJ) {
-    for (int t = threadIdx.x; t < GR * GJ; t += 128) {
-      const int row = t / GJ, jj = t - row * GJ, j = j0 + jj + 1, m = m0 + row;
-      double v = 0.0;
-      if (m < M && j <= H) {
-        const double a = src[(int64_t)m * n + j], b = src[(int64_t)m * n + n - j];
-        v = 2 * j == n ? (par ? 0.0 : a) : (par ? a - b : a + b);
+  const int H = n / 2, nt = (H + 31) / 32, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int par = blockIdx.y / nt, i = (blockIdx.y - par * nt) * 32 + lane, m = blockIdx.x * kSumRows + w, r = blockIdx.z;
+  if (m < M) {
+    const double* src = in + ((int64_t)r * M + m) * n;
+    const double* t = tab + (int64_t)par * H * H + (i < H ? i : H - 1);
+    double* x = xs[w];
+    double acc0 = 0.0, acc1 = 0.0;
+    for (int j0 = 0; j0 < H; j0 += kSumChunk) {
+      const int kc = H - j0 < kSumChunk ? H - j0 : kSumChunk;
+      __syncwarp();
+      for (int jj = lane; jj < kc; jj += 32) {
+        const int j = j0 + jj + 1;
+        const double a = src[j], b = src[n - j];
+        x[jj] = 2 * j == n ? (par ? 0.0 : a) : (par ? a - b : a + b);
       }
-      xs[jj][row] = v;
-    }
-    for (int t = threadIdx.x; t < GJ * GK; t += 128) {
-      const int jj = t / GK, i = t - jj * GK;
-      ts[jj][i] = (j0 + jj < H && i0 + i < H) ? tb[(int64_t)(j0 + jj) * H + i0 + i] : 0.0;
-    }
-    __syncthreads();
+      __syncwarp();
+      int jj = 0;
+#pragma unroll 1
+      for (; jj + 8 <= kc; jj += 8, t += 8 * (int64_t)H) {
+        double s[8];
 #pragma unroll
-    for (int jj = 0; jj < GJ; ++jj) {
-      double x[4], s[4];
+        for (int c = 0; c < 8; ++c) s[c] = t[(int64_t)c * H];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        x[c] = xs[jj][4 * tr + c];
-        s[c] = ts[jj][tk + 16 * c];
+        for (int c = 0; c < 8; c += 2) {
+          const double2 v = *reinterpret_cast<const double2*>(x + jj + c);
+          acc0 = fma(v.x, s[c], acc0);
+          acc1 = fma(v.y, s[c + 1], acc1);
+        }
       }
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc[a][c] = fma(x[a], s[c], acc[a][c]);
+      for (; jj < kc; ++jj, t += H) acc0 = fma(x[jj], t[0], acc0);
     }
-    __syncthreads();
-  }
-  auto put = [&](int m, int k, double v) {
-    if (transposed) out[((int64_t)r * n + k) * M + m] = v;
-    else out[((int64_t)r * M + m) * n + k] = v;
-  };
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int m = m0 + 4 * tr + a;
-    if (m >= M) continue;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int k = 2 * (i0 + tk + 16 * c) + 1 + par;
-      if (k < n) put(m, k, scale ? acc[a][c] * scale[(int64_t)m * n + k] : acc[a][c]);
-    }
-    if (par == 0 && i0 == 0 && tk == 0) put(m, 0, 0.0);
+    pdl_trigger();
+    auto put = [&](int k, double v) {
+      if (transposed) out[((int64_t)r * n + k) * M + m] = v;
+      else out[((int64_t)r * M + m) * n + k] = v;
+    };
+    const int k = 2 * i + 1 + par;
+    const double v = acc0 + acc1;
+    if (k < n) put(k, scale ? v * scale[(int64_t)m * n + k] : v);
+    if (blockIdx.y == 0 && lane == 0) put(0, 0.0);
   }
 }
 
@@ -402,7 +397,7 @@ bool is_pow2(int n) { return n > 0 && (n & (n - 1)) == 0; }
 int ilog2(int n) { int l = 0; while ((1 << l) < n) ++l; return l; }
 
 // Rows of up to kDirect points: direct sums; longer ones of a power of two: the fast algorithm;
-// both in k_dst_rows.  The rest: k_dst_gemm64.
+// both in k_dst_rows.  The rest: k_dst_sums64.
 constexpr int kDirect = 64;
 bool rows_direct(int n) { return n <= kDirect; }
 bool rows_ok(int n) { return rows_direct(n) || is_pow2(n); }
@@ -413,9 +408,15 @@ size_t rows_smem(int n, int P) {
   return sizeof(double2) * 2 * P * (size_t)n + tab;
 }
 
+// Whether the kernel of rows of length n lets the next launch in only when its blocks are about to store
+// (k_dst_rows of more than kDirect points, k_dst_sums64) and not when they begin (direct sums): the blocks of a
+// long pass that are let in then crowd the SMs that have room (two right-hand sides of 200 x 16: 25 -> 76 us,
+// five of 37 x 128: 32 -> 115 us), so that within a solve one is launched plainly behind direct sums.
+bool rows_late(int n) { return !rows_direct(n); }
+
 template <int P, bool TWICE, bool DIRECT, typename Load, typename Store>
 void rows_launch_d(const hq_grid_s* g, int n, int M, int R, const double* tab, const double* scale, const Load& ld,
-                   const Store& st, cudaStream_t s) {
+                   const Store& st, bool late, cudaStream_t s) {
   auto kern = k_dst_rows<Load, Store, P, TWICE, DIRECT>;
   static std::atomic<unsigned long long> done{0};   // devices whose shared-memory limit is raised
   const unsigned long long bit = 1ull << (g->dev & 63);
@@ -426,28 +427,31 @@ void rows_launch_d(const hq_grid_s* g, int n, int M, int R, const double* tab, c
   // threads per pair: one radix-4 group each per pass, or one output and row each
   const int tp = DIRECT ? (2 * n + 31) / 32 * 32 : (n / 4 > 256 ? 256 : n / 4);
   RowsArgs a{n, DIRECT ? 0 : ilog2(n), M, tab, scale};
-  launch_pdl(kern, dim3((unsigned)((M + 1) / 2), (unsigned)(R / P)), dim3((unsigned)(tp * P)), rows_smem(n, P), s, a, ld,
-             st);
+  const dim3 grid((unsigned)((M + 1) / 2), (unsigned)(R / P));
+  if (DIRECT || late) launch_pdl(kern, grid, dim3((unsigned)(tp * P)), rows_smem(n, P), s, a, ld, st);
+  else kern<<<grid, tp * P, rows_smem(n, P), s>>>(a, ld, st);
 }
 template <int P, bool TWICE, typename Load, typename Store>
 void rows_launch(const hq_grid_s* g, int n, int M, int R, const double* tw, const double* tab, const double* scale,
-                 const Load& ld, const Store& st, cudaStream_t s) {
-  if (rows_direct(n)) rows_launch_d<P, TWICE, true>(g, n, M, R, tab, scale, ld, st, s);
-  else rows_launch_d<P, TWICE, false>(g, n, M, R, tw, scale, ld, st, s);
+                 const Load& ld, const Store& st, bool late, cudaStream_t s) {
+  if (rows_direct(n)) rows_launch_d<P, TWICE, true>(g, n, M, R, tab, scale, ld, st, late, s);
+  else rows_launch_d<P, TWICE, false>(g, n, M, R, tw, scale, ld, st, late, s);
 }
 
-// One transform along rows of length n ([R][M][n]): transposed or in place order.
+// One transform along rows of length n ([R][M][n]): transposed or in place order.  late: rows_late of the launch
+// before in the solve.
 void one_pass(const hq_grid_s* g, const double* in, double* out, int n, int M, int R, const double* tw, const double* tab,
-              const double* scale, bool transposed, cudaStream_t s) {
+              const double* scale, bool transposed, bool late, cudaStream_t s) {
   if (rows_ok(n)) {
     const LoadRows<1> ld{in, transposed};   // (the transposed pass reads the caller's sources)
-    if (transposed) rows_launch<1, false>(g, n, M, R, tw, tab, nullptr, ld, StoreT{out}, s);
-    else rows_launch<1, false>(g, n, M, R, tw, tab, nullptr, ld, StoreN{out}, s);
+    if (transposed) rows_launch<1, false>(g, n, M, R, tw, tab, nullptr, ld, StoreT{out}, late, s);
+    else rows_launch<1, false>(g, n, M, R, tw, tab, nullptr, ld, StoreN{out}, late, s);
     return;
   }
-  const int nt = (n / 2 + GK - 1) / GK;
-  launch_pdl(k_dst_gemm64, dim3((unsigned)((M + GR - 1) / GR), (unsigned)(2 * nt), (unsigned)R), dim3(128), (size_t)0, s,
-             in, out, n, M, tab, scale, transposed ? 1 : 0);
+  const dim3 grid((unsigned)((M + kSumRows - 1) / kSumRows), (unsigned)(2 * ((n / 2 + 31) / 32)), (unsigned)R);
+  const int tr = transposed ? 1 : 0;
+  if (late) launch_pdl(k_dst_sums64, grid, dim3(32 * kSumRows), (size_t)0, s, in, out, n, M, tab, scale, tr);
+  else k_dst_sums64<<<grid, 32 * kSumRows, 0, s>>>(in, out, n, M, tab, scale, tr);
 }
 
 // Along y of b = [R][nx][ny], forward, scaled and backward; the result [R][ny][nx] is in the
@@ -455,17 +459,17 @@ void one_pass(const hq_grid_s* g, const double* in, double* out, int n, int M, i
 const double* y_both(const hq_grid_s* g, double* a, double* b, int R, const double* scale, cudaStream_t s) {
   const int nx = g->nx, ny = g->ny;
   if (rows_ok(ny)) {
-    rows_launch<1, true>(g, ny, nx, R, g->tw_y, g->sin_y, scale, LoadRows<1>{b, false}, StoreT{a}, s);
+    rows_launch<1, true>(g, ny, nx, R, g->tw_y, g->sin_y, scale, LoadRows<1>{b, false}, StoreT{a}, rows_late(nx), s);
     return a;
   }
-  one_pass(g, b, a, ny, nx, R, g->tw_y, g->sin_y, scale, false, s);
-  one_pass(g, a, b, ny, nx, R, g->tw_y, g->sin_y, nullptr, true, s);
+  one_pass(g, b, a, ny, nx, R, g->tw_y, g->sin_y, scale, false, rows_late(nx), s);
+  one_pass(g, a, b, ny, nx, R, g->tw_y, g->sin_y, nullptr, true, true, s);
   return b;
 }
 
 }  // namespace
 
-// Sine sums of the tiled product (see k_dst_gemm64): [2][n/2][n/2] values sin(pi j k / n).
+// Sine table of the folded sums (see k_dst_sums64): [2][n/2][n/2] values sin(pi j k / n).
 std::vector<double> dst_f64_table(int n, double (*sin_jk)(int64_t, int64_t, int)) {
   const int H = n / 2;
   std::vector<double> t(2 * (size_t)H * H, 0.0);
@@ -498,18 +502,19 @@ void dst_solve_f64(hq_grid_s* g, int R, cudaStream_t s, const double* scale, con
   if (!src) src = g->f64_a;
   if (!dst) dst = reinterpret_cast<double*>(g->solved);
   const int nx = g->nx, ny = g->ny;
-  one_pass(g, src, g->f64_b, nx, ny, R, g->tw_x, g->sin_x, nullptr, true, s);   // (s S_x)^T      [R][nx][ny]
-  const double* q = y_both(g, g->f64_a, g->f64_b, R, scale, s);                 // [R][ny][nx]
-  one_pass(g, q, dst, nx, ny, R, g->tw_x, g->sin_x, nullptr, false, s);
+  one_pass(g, src, g->f64_b, nx, ny, R, g->tw_x, g->sin_x, nullptr, true, rows_ok(nx), s);   // (s S_x)^T [R][nx][ny]
+  const double* q = y_both(g, g->f64_a, g->f64_b, R, scale, s);                        // [R][ny][nx]
+  one_pass(g, q, dst, nx, ny, R, g->tw_x, g->sin_x, nullptr, false, rows_late(ny), s);
 }
 
 // psi, Ez, Bz of the deposit record dep -> g->solved, sources formed by the first pass.
 void dst_f64_main(hq_grid_s* g, const void* dep, cudaStream_t s) {
   using F = SrcMain<double>;
   rows_launch<3, false>(g, g->nx, g->ny, 3, g->tw_x, g->sin_x, nullptr, LoadSource<F>{src_main_of<double>(g, dep)}, StoreT{g->f64_b},
-                        s);
+                        true, s);
   const double* q = y_both(g, g->f64_a, g->f64_b, 3, g->f64_scale, s);
-  one_pass(g, q, reinterpret_cast<double*>(g->solved), g->nx, g->ny, 3, g->tw_x, g->sin_x, nullptr, false, s);
+  one_pass(g, q, reinterpret_cast<double*>(g->solved), g->nx, g->ny, 3, g->tw_x, g->sin_x, nullptr, false,
+           rows_late(g->ny), s);
 }
 
 // One predictor-corrector iteration: B_perp sources (which clear the trial J_perp and, on the
@@ -517,10 +522,11 @@ void dst_f64_main(hq_grid_s* g, const void* dep, cudaStream_t s) {
 void dst_f64_bmix(hq_grid_s* g, const void* cur, void* prev, void* chi_prev, int last, cudaStream_t s) {
   using F = SrcBperp<double>;
   rows_launch<2, false>(g, g->nx, g->ny, 2, g->tw_x, g->sin_x, nullptr,
-                        LoadSource<F>{src_bperp_of<double>(g, cur, prev, chi_prev, last)}, StoreT{g->f64_b}, s);
+                        LoadSource<F>{src_bperp_of<double>(g, cur, prev, chi_prev, last)}, StoreT{g->f64_b}, true, s);
   const double* q = y_both(g, g->f64_a, g->f64_b, 2, g->f64_scale, s);
   rows_launch<2, false>(g, g->nx, g->ny, 2, g->tw_x, g->sin_x, nullptr, LoadRows<2>{q, false},
-                        StoreMix{reinterpret_cast<V2<double>*>(g->bm), g->d.pc_mix, g->d_status, g->pc_rsum}, s);
+                        StoreMix{reinterpret_cast<V2<double>*>(g->bm), g->d.pc_mix, g->d_status, g->pc_rsum},
+                        rows_late(g->ny), s);
 }
 
 }  // namespace hq

@@ -139,3 +139,15 @@ def test_poisson_into_an_unaligned_array(hq, precision, nx, ny, nrhs):
     dev = float(torch.linalg.norm((got - ref).double()) / torch.linalg.norm(ref.double()))
     print(f"{precision} {nx}x{ny} x {nrhs}: {dev:.1e}")
     assert dev <= (3e-5 if precision == "fp32" else 8e-6)
+
+
+@pytest.mark.parametrize("nx,ny,nrhs", [(65, 65, 1), (67, 70, 4), (409, 37, 1), (37, 128, 5), (514, 66, 2), (516, 520, 1),
+                                        (96, 1030, 3), (24, 100, 3)])
+def test_fp64_sums_of_any_length(hq, nx, ny, nrhs):
+    """FP64 rows of other lengths than powers of two, at the edges of the kernel's blocks (four rows, 32
+    outputs of a parity, 256 folded terms) and behind direct sums, against the oracle's dense sine sums:
+    1e-12, the bar of a single linear operation."""
+    from test_gpu_solvers import solve_case
+    err, same = solve_case(hq, nx, ny, nrhs, "fp64")
+    print(f"fp64 {nx}x{ny} x {nrhs}: {err:.1e}")
+    assert err <= 1e-12 and same
