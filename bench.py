@@ -583,7 +583,7 @@ def dst_comparator(hq, I, stream):
     grid.close()
     return {"case": "Dirichlet solve, 512x512, 3 right-hand sides, FP32 data",
             "tensor_core_dst_us": us_ours, "cufft_dst_us": us_lib, "rel_l2_between": agree,
-            "note": "tensor-core path: one fused cooperative launch (plus the source copy kernel); cuFFT path: "
+            "note": "tensor-core path: one fused cooperative launch from the caller's sources to its array; cuFFT path: "
                     "torch.fft rfft of the odd extension, 4 batched transforms + elementwise ops"}
 
 

@@ -61,6 +61,7 @@ struct TensorMaps {
   int cl_mode;
   int cl_rhs[2];
   int cl_max;   // resident clusters of mode 1
+  bool all_smem;   // a solve kernel of this grid does not exclude others by its registers (see alone_by_registers)
 };
 
 namespace {
@@ -369,11 +370,15 @@ constexpr int kSolveThreads = 256;
 
 // No two CTAs of solve kernels may share an SM, of one launch or of launches on different streams: most
 // of them allocate all of tensor memory and then wait for other CTAs, so that two launches could each
-// hold what the other waits for.  Each therefore takes more than half of an SM's 228 KB of shared memory
-// (1 KB of it the system's, per CTA), whether it needs that much or not.
-constexpr int kAloneBytes = 116 * 1024;
-constexpr int alone_bytes(int need) { return need > kAloneBytes ? need : kAloneBytes; }
-static_assert(2 * (kAloneBytes + 1024) > 228 * 1024, "two solve CTAs would fit one SM");
+// hold what the other waits for.  Two CTAs that take more than half of its registers each never do, and
+// the solve kernels take 127 to 168 registers in 256 to 384 threads.  Should a build give one of them less,
+// the grids that use it request (nearly) all of the shared memory for their launches, which leaves no room
+// for a CTA that has any.  (Shared memory above one half for all of them, without the look at the
+// registers, made a 512^2 sweep with the explicit solver 1.2 % slower: the SMs' split between L1 and shared
+// memory changes between the solves and the node kernels.)
+constexpr bool alone_by_registers(int regs, int threads) { return 2 * regs * threads > 65536; }
+constexpr int kSmemAll = 226 * 1024;
+static_assert(kSmemAll + 2 * 1024 >= 228 * 1024, "1 KB for the system per CTA: room for another CTA would be left");
 
 // The caller's sources [nr][ny][nx] (hq_poisson_solve); row and column 0 read zero.
 struct SrcGiven {
@@ -625,7 +630,7 @@ template <int BN> struct SolveSmem {
   static constexpr int RING = STAGES * Cfg<BN>::STAGE_BYTES;
   static constexpr int SCALE = RING;
   static constexpr int BARS = SCALE + BN * BM * 4;
-  static constexpr int BYTES = alone_bytes(BARS + 256 + 1024 /*alignment*/);
+  static constexpr int BYTES = BARS + 256 + 1024 /*alignment*/;
 };
 
 template <int BN, bool RES, typename E>
@@ -953,7 +958,7 @@ template <int BN> struct RsSmem {
   static constexpr int RING = 0;
   static constexpr int TILE = BM * (BN + 1) * 4;            // the mixing's staged tile
   static constexpr int BARS = KB_MAX * STAGE > TILE ? KB_MAX * STAGE : TILE;
-  static constexpr int BYTES = alone_bytes(BARS + 256 + 1024 /*alignment*/);
+  static constexpr int BYTES = BARS + 256 + 1024 /*alignment*/;
   static constexpr uint32_t TX = 128;                       // tensor-memory columns: accumulator (2 BN), F slice
 };
 
@@ -1344,7 +1349,7 @@ template <int BN, int MODE> struct Cl {
   // MODE 1: kSrcRows rows of R x 256 floats (apart from the data buffers: a peer may already exchange)
   static constexpr int SRC = DATA + DATA_BYTES, SRC_BYTES = LOCAL ? (BN + kMaxRhs - 1) * 512 : kSrcRows * kMaxRhs * 1024;
   static constexpr int BARS = SRC + SRC_BYTES;
-  static constexpr int BYTES = alone_bytes(BARS + 128 + 1024);
+  static constexpr int BYTES = BARS + 128 + 1024;
   static constexpr uint32_t TX = 128, TY = TX + K;          // tensor-memory columns: accumulator, x slice, y slice
   // cluster barriers of a launch (each thread arrives at and waits for every one): the start, the
   // end of each exchange, and where a peer's buffer has to be drained first
@@ -1761,7 +1766,7 @@ template <typename E> struct Wide {
   static constexpr int BN = 128, STAGES = 3, STAGE_BYTES = 4 * A_BYTES;
   static constexpr int TILE = STAGES * STAGE_BYTES, LD = 65;   // the mixing's staged columns, 128 x 64
   static constexpr int BARS = TILE + BM * LD * 4;
-  static constexpr int BYTES = alone_bytes(BARS + 256 + 1024);
+  static constexpr int BYTES = BARS + 256 + 1024;
 };
 
 // 32 consecutive data columns i0 .. of slot s into the next operand's row: ns slots, nd data rows per
@@ -2094,23 +2099,28 @@ int dst_tc_cluster_mode(const hq_grid_s* g) {
 
 namespace {
 template <int BN, int N, bool RES> auto* rs_kernel() { return &k_dst_solve_rs<BN, N, RES>; }
-template <typename K> struct Sized {   // a kernel, its shared memory and where its co-resident CTA count goes
-  K k;
-  int smem;
-  int* ctas;
-};
-template <typename K> Sized(K, int, int*) -> Sized<K>;
 template <int BN, int MODE, bool RES> auto* cl_kernel() { return &k_dst_solve_cl<BN, MODE, RES>; }
 
+static_assert(SolveSmem<64>::BYTES <= kSmemAll && SolveSmem<32>::BYTES <= kSmemAll && Wide<float>::BYTES <= kSmemAll &&
+                  RsSmem<64>::BYTES <= kSmemAll && Cl<64, 0>::BYTES <= kSmemAll && Cl<32, 1>::BYTES <= kSmemAll,
+              "a solve kernel needs more than a launch can request");
+template <typename K> bool by_registers(K kern, int threads) {
+  cudaFuncAttributes fa;
+  if (cudaFuncGetAttributes(&fa, kern) == cudaSuccess) return alone_by_registers(fa.numRegs, threads);
+  cudaGetLastError();
+  return false;
+}
+
 // Right-hand sides whose clusters fit the GPU at once (0: none).
-template <int BN, int MODE, bool RES> int cl_capacity(int* most = nullptr) {
+template <int BN, int MODE, bool RES> int cl_capacity(bool& all_smem, int* most = nullptr) {
   using C = Cl<BN, MODE>;
   auto kern = cl_kernel<BN, MODE, RES>();
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::BYTES) != cudaSuccess ||
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAll) != cudaSuccess ||
       cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
+  all_smem |= !by_registers(kern, kClThreads);
   int best = 0;
   for (int R = 1; R <= kMaxRhs; ++R) {
     const int cs = C::LOCAL ? R * C::CPR : C::CPR, need = C::LOCAL ? 1 : R * C::MB;
@@ -2118,7 +2128,7 @@ template <int BN, int MODE, bool RES> int cl_capacity(int* most = nullptr) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(cs * need));
     cfg.blockDim = dim3(kClThreads);
-    cfg.dynamicSmemBytes = C::BYTES;
+    cfg.dynamicSmemBytes = kSmemAll;   // (one CTA per SM, whatever it requests)
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)cs;
@@ -2152,58 +2162,55 @@ int dst_tc_init(hq_grid_s* g, std::string& err) {
     err = "cannot read the SM count";
     return 1;
   }
-  auto size_solve = [&](auto kern, int smem, int& ctas, int threads = kSolveThreads) {
+  g->tmaps = new TensorMaps();
+  TensorMaps& t = *g->tmaps;
+  t.all_smem = false;
+  auto size_solve = [&](auto kern, int& ctas, int threads = kSolveThreads) {
     int per_sm = 0;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess || per_sm < 1) {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAll) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, kSmemAll) != cudaSuccess || per_sm < 1) {
       err = "cannot size the cooperative DST solve";
       return false;
     }
-    ctas = per_sm * sms;
+    t.all_smem |= !by_registers(kern, threads);
+    ctas = sms;   // one CTA per SM
     return true;
   };
-  g->tmaps = new TensorMaps();
-  TensorMaps& t = *g->tmaps;
   int spare = 0;   // the residual-accumulating instances (the last P-C iteration): same resources
   const bool tf = g->tf32 != 0;
-  if (tf ? (!size_solve(k_dst_solve<64, false, float>, SolveSmem<64>::BYTES, t.ctas[0]) ||
-            !size_solve(k_dst_solve<32, false, float>, SolveSmem<32>::BYTES, t.ctas[1]) ||
-            !size_solve(k_dst_solve<64, true, float>, SolveSmem<64>::BYTES, spare) ||
-            !size_solve(k_dst_solve<32, true, float>, SolveSmem<32>::BYTES, spare))
-         : (!size_solve(k_dst_solve<64, false, __nv_bfloat16>, SolveSmem<64>::BYTES, t.ctas[0]) ||
-            !size_solve(k_dst_solve<32, false, __nv_bfloat16>, SolveSmem<32>::BYTES, t.ctas[1]) ||
-            !size_solve(k_dst_solve<64, true, __nv_bfloat16>, SolveSmem<64>::BYTES, spare) ||
-            !size_solve(k_dst_solve<32, true, __nv_bfloat16>, SolveSmem<32>::BYTES, spare)))
-    return 1;
-  if (tf ? !(size_solve(k_dst_solve_wide<false, float>, Wide<float>::BYTES, t.wide_ctas, kWideThreads) &&
-             size_solve(k_dst_solve_wide<true, float>, Wide<float>::BYTES, spare, kWideThreads))
-         : !(size_solve(k_dst_solve_wide<false, __nv_bfloat16>, Wide<__nv_bfloat16>::BYTES, t.wide_ctas, kWideThreads) &&
-             size_solve(k_dst_solve_wide<true, __nv_bfloat16>, Wide<__nv_bfloat16>::BYTES, spare, kWideThreads)))
+  using B16 = __nv_bfloat16;
+  if (tf ? !(size_solve(k_dst_solve<64, false, float>, t.ctas[0]) && size_solve(k_dst_solve<32, false, float>, t.ctas[1]) &&
+             size_solve(k_dst_solve<64, true, float>, spare) && size_solve(k_dst_solve<32, true, float>, spare) &&
+             size_solve(k_dst_solve_wide<false, float>, t.wide_ctas, kWideThreads) &&
+             size_solve(k_dst_solve_wide<true, float>, spare, kWideThreads))
+         : !(size_solve(k_dst_solve<64, false, B16>, t.ctas[0]) && size_solve(k_dst_solve<32, false, B16>, t.ctas[1]) &&
+             size_solve(k_dst_solve<64, true, B16>, spare) && size_solve(k_dst_solve<32, true, B16>, spare) &&
+             size_solve(k_dst_solve_wide<false, B16>, t.wide_ctas, kWideThreads) &&
+             size_solve(k_dst_solve_wide<true, B16>, spare, kWideThreads)))
     return 1;
   const char* bn = std::getenv("HQ_SOLVE_BN");
   t.wide_only = bn != nullptr && std::atoi(bn) == 64;
   // (the resident fold matrix is bf16: as TF32 words, hi and lo, it would fill tensor memory at 512^2)
   t.rs = dst_tc_resident(g);
-  auto size_rs = [&](auto... kern) { return (size_solve(kern.k, kern.smem, *kern.ctas, kClThreads) && ...); };
-  if (t.rs && !(g->nx == 512 ? size_rs(Sized{rs_kernel<64, 512, false>(), RsSmem<64>::BYTES, &t.rs_ctas[0]},
-                                       Sized{rs_kernel<32, 512, false>(), RsSmem<32>::BYTES, &t.rs_ctas[1]},
-                                       Sized{rs_kernel<64, 512, true>(), RsSmem<64>::BYTES, &spare},
-                                       Sized{rs_kernel<32, 512, true>(), RsSmem<32>::BYTES, &spare})
-                             : size_rs(Sized{rs_kernel<64, 256, false>(), RsSmem<64>::BYTES, &t.rs_ctas[0]},
-                                       Sized{rs_kernel<32, 256, false>(), RsSmem<32>::BYTES, &t.rs_ctas[1]},
-                                       Sized{rs_kernel<64, 256, true>(), RsSmem<64>::BYTES, &spare},
-                                       Sized{rs_kernel<32, 256, true>(), RsSmem<32>::BYTES, &spare})))
+  auto size_rs = [&](auto* w0, auto* n0, auto* w1, auto* n1) {
+    return size_solve(w0, t.rs_ctas[0], kClThreads) && size_solve(n0, t.rs_ctas[1], kClThreads) &&
+           size_solve(w1, spare, kClThreads) && size_solve(n1, spare, kClThreads);
+  };
+  if (t.rs && !(g->nx == 512 ? size_rs(rs_kernel<64, 512, false>(), rs_kernel<32, 512, false>(), rs_kernel<64, 512, true>(),
+                                       rs_kernel<32, 512, true>())
+                             : size_rs(rs_kernel<64, 256, false>(), rs_kernel<32, 256, false>(), rs_kernel<64, 256, true>(),
+                                       rs_kernel<32, 256, true>())))
     return 1;
   t.cl_mode = dst_tc_cluster_mode(g);
   t.cl_rhs[0] = t.cl_rhs[1] = t.cl_max = 0;
   if (t.cl_mode == 0) {
-    t.cl_rhs[0] = std::min(cl_capacity<32, 0, false>(), cl_capacity<32, 0, true>());
-    t.cl_rhs[1] = cl_capacity<64, 0, false>();
+    t.cl_rhs[0] = std::min(cl_capacity<32, 0, false>(t.all_smem), cl_capacity<32, 0, true>(t.all_smem));
+    t.cl_rhs[1] = cl_capacity<64, 0, false>(t.all_smem);
   } else if (t.cl_mode == 2) {
-    t.cl_rhs[0] = std::min(cl_capacity<32, 2, false>(), cl_capacity<32, 2, true>());
-    t.cl_rhs[1] = cl_capacity<64, 2, false>();
+    t.cl_rhs[0] = std::min(cl_capacity<32, 2, false>(t.all_smem), cl_capacity<32, 2, true>(t.all_smem));
+    t.cl_rhs[1] = cl_capacity<64, 2, false>(t.all_smem);
   } else if (t.cl_mode == 1) {
-    t.cl_rhs[0] = std::min(cl_capacity<32, 1, false>(&t.cl_max), cl_capacity<32, 1, true>());
+    t.cl_rhs[0] = std::min(cl_capacity<32, 1, false>(t.all_smem, &t.cl_max), cl_capacity<32, 1, true>(t.all_smem));
   }
   const uint64_t nxp = g->nxp, nyp = g->nyp;
   int bad = 0;
@@ -2277,6 +2284,7 @@ void solve_fused(hq_grid_s* g, int R, int final_mode, int last, cudaStream_t s, 
   if (pre == 1) a.sm = src_main_of<float>(g, dep_cur);
   if (pre == 2) a.sb = src_bperp_of<float>(g, dep_cur, dep_prev, chi_prev, last);
   if (pre == 3) a.sc = SrcGiven{src, g->geom, R};
+  const auto smem_of = [&](int need) { return (size_t)(t.all_smem ? kSmemAll : need); };
   auto late_reset = [&]() {
     if (pre == 2 && a.sb.reset_prev && a.sb.mode == 2) {
       a.sb.reset_prev = 0;
@@ -2304,7 +2312,7 @@ void solve_fused(hq_grid_s* g, int R, int final_mode, int last, cudaStream_t s, 
     cfg.attrs = at;
     cfg.numAttrs = local ? 1 : 2;
     auto go = [&](auto* kern, int smem) {
-      cfg.dynamicSmemBytes = (size_t)smem;
+      cfg.dynamicSmemBytes = smem_of(smem);
       cudaLaunchKernelEx(&cfg, kern, t.rx_hi[0][v], t.rx_lo[0][v], t.rx_hi[1][v], t.rx_lo[1][v],
                          static_cast<const uint4*>(g->fxt), static_cast<const uint4*>(g->fyt), a);
     };
@@ -2335,7 +2343,7 @@ void solve_fused(hq_grid_s* g, int R, int final_mode, int last, cudaStream_t s, 
     // (at least a CTA per kSrcRows source rows: 256^2, two right-hand sides has 32 tiles)
     cfg.gridDim = dim3((unsigned)std::min(std::max(tiles_v, pre ? n / kSrcRows : 0), t.rs_ctas[v] / MB * MB));
     cfg.blockDim = dim3(kClThreads);
-    cfg.dynamicSmemBytes = narrow ? RsSmem<32>::BYTES : RsSmem<64>::BYTES;
+    cfg.dynamicSmemBytes = smem_of(narrow ? RsSmem<32>::BYTES : RsSmem<64>::BYTES);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -2371,7 +2379,7 @@ void solve_fused(hq_grid_s* g, int R, int final_mode, int last, cudaStream_t s, 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     auto go = [&](auto* kern, int smem) {
-      cfg.dynamicSmemBytes = (size_t)smem;
+      cfg.dynamicSmemBytes = smem_of(smem);
       cudaLaunchKernelEx(&cfg, kern, t.fx_hi, t.fx_lo, t.fy_hi, t.fy_lo, t.a0_hi, t.a0_lo, t.a1_hi, t.a1_lo, a);
     };
     using B16 = __nv_bfloat16;
@@ -2384,7 +2392,7 @@ void solve_fused(hq_grid_s* g, int R, int final_mode, int last, cudaStream_t s, 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)std::min(t.ctas[v], tiles(narrow ? 32 : 64)));
   cfg.blockDim = dim3(kSolveThreads);
-  cfg.dynamicSmemBytes = narrow ? SolveSmem<32>::BYTES : SolveSmem<64>::BYTES;
+  cfg.dynamicSmemBytes = smem_of(narrow ? SolveSmem<32>::BYTES : SolveSmem<64>::BYTES);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
