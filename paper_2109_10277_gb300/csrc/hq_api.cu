@@ -360,7 +360,7 @@ hq_status solve_fields_impl(hq_grid_s* g, int slice) {
     g->pc_rsum = last && g->d_pcres ? g->d_pcres + 2 * kResLanes * (int64_t)slice : nullptr;   // (opt-in)
     tape_b_iterate(g, m);
     g->pc_iter = m;   // the B_perp sources of iteration 0 keep their invariant part for the others
-    { Prof p(g, HQ_K_TRIAL, 1); launch_trial_pass<T>(g, slice, m, s); }
+    { Prof p(g, HQ_K_TRIAL, trial_launches(g, m)); launch_trial_pass<T>(g, slice, m, s); }
     if (m == 0) g->f4_slice = g->no_f4 ? -1 : slice;   // the final pass may reuse it
     if (g->det) launch_fx_decode(g, g->tj, 2 * g->nnode, nullptr, s);
     if (fused_src) {
@@ -398,7 +398,7 @@ hq_status solve_fields_impl(hq_grid_s* g, int slice) {
 // last predictor-corrector source kernel of that slice reset to the ion background.
 template <typename T>
 void final_pass(hq_grid_s* g, int slice_from, int parity) {
-  Prof p(g, HQ_K_FINAL, 1);
+  Prof p(g, HQ_K_FINAL, final_launches(g, g->f4_slice == slice_from));
   launch_final_pass<T>(g, slice_from, g->dep[parity], g->chi[parity], g->f4_slice == slice_from, g->stream);
   if (g->det) {
     launch_fx_decode(g, g->dep[parity], 4 * g->nnode, nullptr, g->stream);

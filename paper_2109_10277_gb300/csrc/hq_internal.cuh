@@ -324,6 +324,8 @@ inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 template <typename T> void launch_plasma_init(const hq_grid_s* g, cudaStream_t s);
 template <typename T> void launch_deposit_initial(const hq_grid_s* g, void* dep, void* chi, int ion_only, cudaStream_t s);
 template <typename T> void launch_trial_pass(const hq_grid_s* g, int slice, int iter, cudaStream_t s);
+int trial_launches(const hq_grid_s* g, int iter);   // kernel launches of a trial pass, and of a final pass
+int final_launches(const hq_grid_s* g, bool f4);
 template <typename T> void launch_final_pass(const hq_grid_s* g, int slice, void* dep, void* chi, bool f4,
                                              cudaStream_t s);
 // fields

@@ -1300,6 +1300,11 @@ void launch_species_c0(const hq_grid_s* g, double* out, cudaStream_t s) {
   }
 }
 
+// (quads, their order-3 final pass: two kernels in the slice's first trial pass and in the final pass)
+bool quads_final(const hq_grid_s* g, bool f4) { return f4 && quads(g) && g->d.shape_order == 3; }
+int trial_launches(const hq_grid_s* g, int iter) { return iter == 0 && quads(g) ? 2 : 1; }
+int final_launches(const hq_grid_s* g, bool f4) { return quads_final(g, f4) ? 2 : 1; }
+
 template <typename T>
 void launch_trial_pass(const hq_grid_s* g, int slice, int iter, cudaStream_t s) {
   const unsigned nb = blocks_for(g->np);
@@ -1348,7 +1353,7 @@ void launch_final_pass(const hq_grid_s* g, int slice, void* dep, void* chi, bool
   float* ps = psrc_of(g, dep);
   const PpcInfo pc = ppc_of(g);
   if constexpr (C)
-    if (f4 && quads(g) && g->d.shape_order == 3) {   // (lower orders: 95 -> 107, 103 -> 116 us at 2^20 particles)
+    if (quads_final(g, f4)) {   // (lower orders: 95 -> 107, 103 -> 116 us at 2^20 particles)
       const unsigned n4 = blocks_for(g->np / 4);
       auto go = [&](auto* fin, auto* dep4) {
         launch_pdl(fin, nb, kThreads, 0, s, g->p32, g->geom, gf, bm, d, c, ps, pc, slice, gd, rm, g->sp);

@@ -151,3 +151,22 @@ def test_fp64_sums_of_any_length(hq, nx, ny, nrhs):
     err, same = solve_case(hq, nx, ny, nrhs, "fp64")
     print(f"fp64 {nx}x{ny} x {nrhs}: {err:.1e}")
     assert err <= 1e-12 and same
+
+
+@pytest.mark.parametrize("n,ppc,order,trial,final", [(256, 2, 3, 2, 2), (256, 2, 2, 2, 1), (128, 2, 3, 1, 1), (256, 1, 3, 1, 1)])
+def test_profiled_launches(hq, n, ppc, order, trial, final):
+    """hq_profile_read counts every kernel launch: with four particles per cell in one thread a slice's first
+    trial pass is two kernels, and so is the cubic final pass."""
+    nz, iters = 4, 3
+    g = I.scaled_grid(I.grid_params("linear64"), n, n, nz, ppc_x=ppc, ppc_y=ppc, shape_order=order, n_pc_iter=iters,
+                      zeta_min=-0.2, zeta_max=0.2)
+    grid = hq.Grid(g, precision="fp32")
+    beams = [hq.Beam(I.random_beam(2_000, 0.4, 0.4, 0.1, 0.5))]
+    grid.profile(True)
+    grid.sweep(beams)
+    prof = grid.profile_read()
+    grid.profile(False)
+    grid.sync()
+    grid.close()
+    assert prof["trial"][1] == nz * (iters - 1 + trial)
+    assert prof["final"][1] == nz * final
