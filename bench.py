@@ -206,8 +206,8 @@ def run_reference(args):
 # (profiles/: k_dst_solve_rs R = 3, R = 2 of the first and of the later predictor-corrector
 # iterations weighted 1:1:4 as in a slice; the trial pass's first and later iterations 1:4;
 # the final pass)
-NCU_TRAFFIC = {"dst": (6.911232e6 + 16.355072e6 + 4 * 7.967744e6) / 6, "trial": (21.232896e6 + 4 * 13.637312e6) / 5,
-               "final": 46.438144e6 + 118.784e3}
+NCU_TRAFFIC = {"dst": (6.909952e6 + 16.348416e6 + 4 * 7.971328e6) / 6, "trial": (21.23264e6 + 4 * 13.637248e6) / 5,
+               "final": 46.43712e6 + 83.968e3}
 
 
 def dst_flops_per_sweep(g: dict) -> float:
