@@ -170,3 +170,37 @@ def test_profiled_launches(hq, n, ppc, order, trial, final):
     grid.close()
     assert prof["trial"][1] == nz * (iters - 1 + trial)
     assert prof["final"][1] == nz * final
+
+
+@pytest.mark.parametrize("n,nrhs", [(512, 2), (512, 5), (256, 5), (256, 2)])
+def test_solves_beside_other_work(hq, n, nrhs):
+    """FP32 solves whose products wait for single tiles, on one stream, beside a sweep on another that takes
+    some of the SMs, so that a product's tiles end far apart: every result is bit for bit that of the solve
+    alone (the sums of a solve have a fixed order)."""
+    g = dict(nx=n, ny=n, nzeta=2, xmin=-4.0, xmax=4.0, ymin=-4.0, ymax=4.0, zeta_min=0.0, zeta_max=1.0)
+    src = [torch.randn(nrhs, n, n, device="cuda", generator=torch.Generator(device="cuda").manual_seed(k)) for k in range(4)]
+    torch.cuda.synchronize()
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    with torch.cuda.stream(s1):
+        grid = hq.Grid(g, precision="fp32")
+        ref = [grid.poisson_solve(s) for s in src]
+        grid.sync()
+    with torch.cuda.stream(s2):
+        other = hq.Grid(I.scaled_grid(I.grid_params("linear64"), 96, 96, 48), precision="fp32")
+        beams = [hq.Beam(I.random_beam(20_000, 0.4, 0.4, 1.0, 0.5))]
+        other.sweep(beams)
+        other.sync()
+    torch.cuda.synchronize()
+    got = []
+    for _ in range(6):
+        with torch.cuda.stream(s2):
+            other.sweep(beams)
+        with torch.cuda.stream(s1):
+            got += [grid.poisson_solve(s) for _ in range(10) for s in src]
+    assert grid.sync() == 0
+    other.sync()
+    torch.cuda.synchronize()
+    for k, x in enumerate(got):
+        assert torch.equal(x, ref[k % len(src)]), k
+    grid.close()
+    other.close()
